@@ -34,3 +34,21 @@ def test_voxel_driven_shapes(P, orc, Wt, nx, ny, dx, k):
     assert margin.min() > 1e-5  # no response decision within reach of FP32 rounding
     scale = np.abs(Ao).max(0, keepdims=True)
     assert_close(A, Ao, 1e-5, 1e-6 * scale + 1e-30, "voxel-driven A")
+
+
+@pytest.mark.parametrize("Wt,Wa,N", [(0, 0, 1), (1, 0, 9), (0, 3, 49), (3, 3, 1)])
+def test_truncation_whole_and_tiny_windows(P, orc, Wt, Wa, N):
+    """Windows down to one entry, all entries kept, a count of windows that
+    leaves warps without one; values whose FP32 total would overflow."""
+    E = (2 * Wt + 1) * (2 * Wa + 1)
+    rng = np.random.default_rng(7 + E)
+    w = rng.uniform(0, 1, size=(131, E, E)).astype(np.float32)
+    w[3] *= np.float32(1e38)
+    idx, wk = P.spread_topn(torch.from_numpy(w).cuda(), Wt, Wa, N)
+    out_o, idx_o = orc.spread_topn(w.astype(np.float64), Wt, Wa, N)
+    np.testing.assert_array_equal(idx.cpu().numpy(), idx_o)
+    keep = np.delete(np.arange(131), 3) if E > 1 else np.arange(131)  # row 3: beyond FP32
+    wo = np.take_along_axis(out_o.reshape(131, -1), idx_o.astype(np.int64), 1)
+    assert_close(wk.cpu().numpy()[keep], wo[keep], 2e-7, 1e-30, "kept weights")
+    # its scaled weights are the double ones rounded (infinite beyond the range)
+    np.testing.assert_allclose(wk.cpu().numpy()[3], np.minimum(wo[3], np.inf), rtol=2e-7)
