@@ -57,89 +57,263 @@ __device__ __forceinline__ void lor_ray(Ray &r, const Scan &sc, const Img &im, c
     make_ray(r, im, px, py, pz, qx, qy, qz);
 }
 
-__global__ void __launch_bounds__(ROWS_THREADS) g_count_kernel(
-    Scan sc, Img im, const int32_t *__restrict__ lors, int64_t n, int64_t *__restrict__ counts,
-    int *__restrict__ status) {
-    extern __shared__ double cs[];
-    stage_blocks(sc, cs);
-    __syncthreads();
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        Ray r;
-        lor_ray(r, sc, im, cs, lors[2 * k], lors[2 * k + 1]);
-        int64_t cnt = 0;
-        bool ok = trace_rows(r, [&](int, int, int x0, int x1, long long, long long) {
-            cnt += x1 - x0 + 1;
-        });
-        if (!ok) atomicExch(status, PSF_EDEBUG);
-        counts[k] = cnt;
+// K4 / K6 for listed LORs.  A warp takes G consecutive LORs; its lanes set up
+// one LOR's ray each (the FP64 part, shared by 32 rays), then the rays' (LOR, z
+// slab) pairs are flattened, 32 at a time, each lane finding its slab's y
+// rows; those are flattened again, a lane finding the voxel run of one (slab,
+// y row); and the runs' voxels once more, a lane storing one entry, so
+// consecutive lanes write consecutive slots however long a ray's runs are.
+// Every step is trace_rows' own for that slab, row and voxel, so the rows are
+// the same numbers.  Bound by the integer instructions of the run lookups (64-
+// bit parameters).  400,000 event LORs on the 3D ring (81e6 entries): with a
+// thread per LOR, a lane's whole ray serial and its neighbours' rows elsewhere,
+// the count took 2.74 ms and the fill 5.32 ms; now 0.96 and 1.61 ms.
+constexpr int GT_W = 4;  // warps per CTA
+
+enum { GT_COUNT = 0, GT_CSR = 1, GT_PAD = 2 };
+
+struct GtWarp {
+    Ray ray[32];
+    long long zl[32], zh[32];        // slab: clipped parameter interval
+    int4 slab[32];                   // slab: LOR, z index, first y row, -
+    long long yl[32], yh[32];        // run: clipped parameter interval
+    int4 run[32];                    // run: LOR, first x - start, column of x = 0, -
+    long long dst[32];               // run: output slot of its first voxel - start
+    int start[64];                   // run: flattened start; INT_MAX past the last
+    int cnt[32];                     // LOR: voxels so far
+};
+
+// The slab of axis a holding parameter al, with its bounds (voxel_at).
+__device__ __forceinline__ bool voxel_span(const Axis &a, long long al, int &k, long long &lo,
+                                           long long &hi) {
+    if (a.kind == 0) {
+        k = a.fixed;
+        lo = -FX_BIG;
+        hi = FX_BIG;
+        return true;
     }
+    const float af = u32_to_f((unsigned)(al >> 8)) * 2.3283064365386963e-10f;  // 2^-32
+    float g = fmaf(af, a.df, a.sf);
+    g = fminf(fmaxf(g, -2.0f), (float)a.n + 1.0f);
+    k = f2i_rd(g);
+    const int up = a.inc ? 1 : -1;
+    for (int it = 0; it < 64; ++it) {
+        slab(a, k, lo, hi);
+        if (al < lo) {
+            k -= up;
+        } else if (al >= hi) {
+            k += up;
+        } else {
+            return true;
+        }
+    }
+    slab(a, k, lo, hi);
+    return false;
 }
 
-// K6: each lane of a warp traces one LOR with a resumable cursor and stages
-// up to 32 of its voxels in shared memory; the warp then writes every lane's
-// chunk with full 128-byte stores (one row segment per store instruction).
-constexpr int FILL_WARPS = 8;
-constexpr int FILL_PAD = 33;  // staging row stride (conflict-free lane-major writes)
+// Index of the lane whose inclusive prefix `incl` first exceeds f (every lane
+// calls; 31 when none does).
+__device__ __forceinline__ int owner_of(int incl, int f) {
+    int q = 0;
+#pragma unroll
+    for (int step = 16; step >= 1; step >>= 1) {
+        const int v = __shfl_sync(0xffffffffu, incl, q + step - 1);
+        if (v <= f) q += step;
+    }
+    return q > 31 ? 31 : q;
+}
 
-__global__ void __launch_bounds__(FILL_WARPS * 32) g_fill_kernel(
-    Scan sc, Img im, const int32_t *__restrict__ lors, int64_t n,
-    const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col, float *__restrict__ val,
-    int *__restrict__ status) {
-    extern __shared__ double cs[];
+__device__ __forceinline__ int warp_incl_scan(int v, int lane) {
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// Left shift that gives 0 for shift counts of 32 and more (PTX shl.b32
+// clamps the count; a C++ shift by 32 is undefined).
+__device__ __forceinline__ unsigned shl_clamped(unsigned v, int n) {
+    unsigned r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+    return r;
+}
+
+// MODE GT_COUNT: counts[k] = entries of LOR k.  GT_CSR: rows at row_ptr.
+// GT_PAD: rows at k * stride (stride >= nx + ny + nz, more than a row can
+// hold), counts too.
+template <int MODE>
+__global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
+    Scan sc, Img im, const int32_t *__restrict__ lors, int64_t n, int G,
+    int64_t *__restrict__ counts, const int64_t *__restrict__ row_ptr, int64_t stride,
+    int32_t *__restrict__ col, float *__restrict__ val, int *__restrict__ status) {
+    extern __shared__ __align__(16) unsigned char gt_raw[];
+    GtWarp &W = reinterpret_cast<GtWarp *>(gt_raw)[threadIdx.x >> 5];
+    double *cs = reinterpret_cast<double *>(reinterpret_cast<GtWarp *>(gt_raw) + GT_W);
     stage_blocks(sc, cs);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int32_t *scol = reinterpret_cast<int32_t *>(cs + 2 * sc.R) + warp * 32 * FILL_PAD;
-    float *sval = reinterpret_cast<float *>(reinterpret_cast<int32_t *>(cs + 2 * sc.R) +
-                                            FILL_WARPS * 32 * FILL_PAD) +
-                  warp * 32 * FILL_PAD;
     __syncthreads();
+    const unsigned F = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned le = (2u << lane) - 1u;
     const int nx = im.nx, nxy = im.nx * im.ny;
-    for (int64_t base = ((int64_t)blockIdx.x * FILL_WARPS + warp) * 32; base < n;
-         base += (int64_t)gridDim.x * FILL_WARPS * 32) {
-        const int64_t k = base + lane;
-        Ray r;
-        VoxelCursor c;
-        int64_t pos = 0, end = 0;
-        float to_mm = 0.0f;
-        c.done = true;
-        c.ok = true;
-        if (k < n) {
+    bool ok = true;
+    for (int64_t k0 = ((int64_t)blockIdx.x * GT_W + warp) * G; k0 < n;
+         k0 += (int64_t)gridDim.x * GT_W * G) {
+        const int64_t k = k0 + lane;
+        const bool mine = lane < G && k < n;
+        int nsl = 0, z0 = 0;
+        if (mine) {
+            Ray r;
             lor_ray(r, sc, im, cs, lors[2 * k], lors[2 * k + 1]);
-            cursor_start(r, c);
-            pos = row_ptr[k];
-            end = row_ptr[k + 1];
-            to_mm = r.len_mm * (float)(1.0 / FX);
+            if (!r.empty) {
+                int za, zb;
+                ok &= voxel_at(r.ax[2], r.amin, za);
+                ok &= voxel_at(r.ax[2], r.amax - 1, zb);
+                z0 = za < zb ? za : zb;
+                int z1 = za < zb ? zb : za;
+                z0 = z0 < 0 ? 0 : z0;
+                z1 = z1 > im.nz - 1 ? im.nz - 1 : z1;
+                nsl = z1 >= z0 ? z1 - z0 + 1 : 0;
+                W.ray[lane] = r;
+            }
         }
-        bool bad = false;
-        while (__any_sync(0xffffffffu, !c.done)) {
-            int cnt = 0;
-            while (cnt < 32 && !c.done) {
-                int iz, iy, ix;
-                long long ch;
-                cursor_take(r, c, iz, iy, ix, ch);
-                scol[lane * FILL_PAD + cnt] = iz * nxy + iy * nx + ix;
-                sval[lane * FILL_PAD + cnt] = units_to_f(ch) * to_mm;
-                ++cnt;
-            }
-            if (pos + cnt > end) {  // never for a consistent count pass; stay in the row
-                bad = true;
-                cnt = (int)(end - pos > 0 ? end - pos : 0);
-            }
-            __syncwarp();
-            for (int j = 0; j < 32; ++j) {
-                const int cj = __shfl_sync(0xffffffffu, cnt, j);
-                const int64_t pj = __shfl_sync(0xffffffffu, pos, j);
-                if (lane < cj) {
-                    col[pj + lane] = scol[j * FILL_PAD + lane];
-                    val[pj + lane] = sval[j * FILL_PAD + lane];
+        W.cnt[lane] = 0;
+        const int incl = warp_incl_scan(nsl, lane);
+        const int zfirst = z0 - (incl - nsl);  // z index = zfirst + flattened slab
+        const int slabs = __shfl_sync(F, incl, 31);
+        __syncwarp();
+        for (int s0 = 0; s0 < slabs; s0 += 32) {
+            // 32 slabs -> their y rows
+            const int s = s0 + lane, q = owner_of(incl, s);
+            const int iz = __shfl_sync(F, zfirst, q) + s;
+            int rows = 0;
+            if (s < slabs) {
+                const Ray &r = W.ray[q];
+                long long zl, zh;
+                slab(r.ax[2], iz, zl, zh);
+                zl = zl > r.amin ? zl : r.amin;
+                zh = zh < r.amax ? zh : r.amax;
+                if (zh > zl) {
+                    int ya, yb;
+                    ok &= voxel_at(r.ax[1], zl, ya);
+                    ok &= voxel_at(r.ax[1], zh - 1, yb);
+                    int y0 = ya < yb ? ya : yb, y1 = ya < yb ? yb : ya;
+                    y0 = y0 < 0 ? 0 : y0;
+                    y1 = y1 > im.ny - 1 ? im.ny - 1 : y1;
+                    rows = y1 >= y0 ? y1 - y0 + 1 : 0;
+                    W.zl[lane] = zl;
+                    W.zh[lane] = zh;
+                    W.slab[lane] = make_int4(q, iz, y0, 0);
                 }
             }
-            pos += cnt;
+            const int rincl = warp_incl_scan(rows, lane);
+            const int nrows = __shfl_sync(F, rincl, 31);
             __syncwarp();
+            for (int f0 = 0; f0 < nrows; f0 += 32) {
+                // 32 (slab, y row) pairs -> their voxel runs
+                const int f = f0 + lane, o = owner_of(rincl, f);
+                const int before = __shfl_sync(F, rincl - rows, o);
+                int c = 0, rq = -1, x0 = 0, base = 0;
+                long long yl = 0, yh = 0;
+                if (f < nrows) {
+                    const int4 sl = W.slab[o];
+                    rq = sl.x;
+                    const Ray &r = W.ray[rq];
+                    const int iy = sl.z + (f - before);
+                    const long long zl = W.zl[o], zh = W.zh[o];
+                    slab(r.ax[1], iy, yl, yh);
+                    yl = yl > zl ? yl : zl;
+                    yh = yh < zh ? yh : zh;
+                    if (yh > yl) {
+                        int x1;
+                        long long la, ha, lb, hb;
+                        ok &= voxel_span(r.ax[0], yl, x0, la, ha);
+                        ok &= voxel_span(r.ax[0], yh - 1, x1, lb, hb);
+                        if (x0 > x1) {
+                            const int t = x0;
+                            x0 = x1;
+                            x1 = t;
+                            const long long tl = la, th = ha;
+                            la = lb;
+                            ha = hb;
+                            lb = tl;
+                            hb = th;
+                        }
+                        if (x0 < 0) {
+                            x0 = 0;
+                            slab(r.ax[0], x0, la, ha);
+                        }
+                        if (x1 > nx - 1) {
+                            x1 = nx - 1;
+                            slab(r.ax[0], x1, lb, hb);
+                        }
+                        la = la > yl ? la : yl;
+                        ha = ha < yh ? ha : yh;
+                        lb = lb > yl ? lb : yl;
+                        hb = hb < yh ? hb : yh;
+                        if (x1 >= x0 && ha - la < r.min_units) ++x0;
+                        if (x1 >= x0 && hb - lb < r.min_units) --x1;
+                        c = x1 >= x0 ? x1 - x0 + 1 : 0;
+                        base = sl.y * nxy + iy * nx;
+                    }
+                }
+                // entries before this run: in the chunk, and in its LOR
+                const int eincl = warp_incl_scan(c, lane), off = eincl - c;
+                const int pq = __shfl_up_sync(F, rq, 1), nq = __shfl_down_sync(F, rq, 1);
+                const unsigned heads = __ballot_sync(F, lane == 0 || pq != rq);
+                const int ofirst = __shfl_sync(F, off, 31 - __clz(heads & le));
+                const int had = rq >= 0 ? W.cnt[rq] : 0;
+                __syncwarp();
+                if (rq >= 0 && (lane == 31 || nq != rq)) W.cnt[rq] = had + eincl - ofirst;
+                if (MODE != GT_COUNT) {
+                    const int total = __shfl_sync(F, eincl, 31);
+                    const unsigned live = __ballot_sync(F, c > 0);
+                    const int nrun = __popc(live), at = __popc(live & (le >> 1));
+                    if (c > 0) {
+                        const int64_t kq = k0 + rq;
+                        const int64_t first = MODE == GT_CSR ? row_ptr[kq] : kq * stride;
+                        const int64_t room =
+                            (MODE == GT_CSR ? row_ptr[kq + 1] : first + stride) - first;
+                        const int inrow = had + off - ofirst;
+                        if (inrow + c > room) ok = false;  // never after a consistent count
+                        W.start[at] = off;
+                        W.dst[at] = inrow + c > room ? -1 : first + inrow - off;
+                        W.run[at] = make_int4(rq, x0 - off, base, 0);
+                        W.yl[at] = yl;
+                        W.yh[at] = yh;
+                    }
+                    W.start[nrun + lane] = 0x7fffffff;
+                    __syncwarp();
+                    int gbase = -1;  // run holding the entry before the step
+                    for (int e0 = 0; e0 < total; e0 += 32) {
+                        const unsigned B =
+                            __reduce_or_sync(F, shl_clamped(1u, W.start[gbase + 1 + lane] - e0));
+                        const int e = e0 + lane;
+                        if (e < total) {
+                            const int g = gbase + __popc(B & le);
+                            const int4 R = W.run[g];
+                            const long long d = W.dst[g];
+                            const Ray &r = W.ray[R.x];
+                            const int ix = R.y + e;
+                            const float ch =
+                                units_to_f(chord_in_row(r.ax[0], ix, W.yl[g], W.yh[g])) *
+                                (r.len_mm * (float)(1.0 / FX));
+                            if (d >= 0) {
+                                col[d + e] = R.z + ix;
+                                val[d + e] = ch;
+                            }
+                        }
+                        gbase += __popc(B);
+                    }
+                }
+                __syncwarp();
+            }
         }
-        if (k < n && (!c.ok || bad || pos != end)) atomicExch(status, PSF_EDEBUG);
+        if (MODE != GT_CSR && mine) counts[k] = W.cnt[lane];
+        if (MODE == GT_CSR && mine && row_ptr[k] + W.cnt[lane] != row_ptr[k + 1]) ok = false;
+        __syncwarp();
     }
+    if (!ok) atomicExch(status, PSF_EDEBUG);
 }
 
 // ------------------------------------------- rows traced on the fly
@@ -449,19 +623,40 @@ static int sm_count() {
     return sms;
 }
 
+// LORs of a warp in g_rows_kernel: 32 share the FP64 ray set-up best, fewer
+// when the list would otherwise leave the chip's warps idle.
+template <int MODE>
+static int g_rows(const Scan &sc, const Img &im, const int32_t *lors, int64_t n, int64_t *counts,
+                  const int64_t *row_ptr, int64_t stride, int32_t *col, float *val, int *status,
+                  cudaStream_t st) {
+    const size_t shm = sizeof(GtWarp) * GT_W + sizeof(double) * 2 * sc.R;
+    PSF_TRY(cudaFuncSetAttribute(g_rows_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)shm));
+    int per_sm = 0;
+    PSF_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, g_rows_kernel<MODE>, GT_W * 32,
+                                                          shm));
+    const int64_t cap = (int64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
+    int G = 32;
+    while (G > 1 && n < cap * GT_W * G) G /= 2;
+    const int64_t need = (n + GT_W * G - 1) / (GT_W * G);
+    {
+        PSF_TIMED(MODE == GT_COUNT ? "g_rows_kernel<count>" : "g_rows_kernel<fill>", st);
+        g_rows_kernel<MODE><<<(int)(need < 4 * cap ? need : 4 * cap), GT_W * 32, shm, st>>>(
+            sc, im, lors, n, G, counts, row_ptr, stride, col, val, status);
+    }
+    PSF_LAUNCHED();
+    return PSF_OK;
+}
+
 // Geometric rows into (row_ptr, col, val); col == NULL: counts + scan only.
 static int geom_rows(const Scan &sc, const Img &im, const int32_t *lors, int64_t n,
                      int64_t *row_ptr, int32_t *col, float *val, int64_t capacity,
                      int64_t *nnz_out, int64_t *tile_sums, int *status, cudaStream_t st) {
-    const size_t shm = sizeof(double) * 2 * sc.R;
-    const int grid = sm_count() * 16;
     PSF_TRY(cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), st));
-    {
-        PSF_TIMED("g_count_kernel", st);
-        g_count_kernel<<<grid, ROWS_THREADS, shm, st>>>(sc, im, lors, n, row_ptr + 1, status);
-    }
-    PSF_LAUNCHED();
-    int rc = inclusive_scan(row_ptr + 1, n, tile_sums, st);
+    int rc = g_rows<GT_COUNT>(sc, im, lors, n, row_ptr + 1, nullptr, 0, nullptr, nullptr, status,
+                              st);
+    if (rc) return rc;
+    rc = inclusive_scan(row_ptr + 1, n, tile_sums, st);
     if (rc) return rc;
     int64_t nnz = 0;
     int h_status = 0;
@@ -472,17 +667,8 @@ static int geom_rows(const Scan &sc, const Img &im, const int32_t *lors, int64_t
     if (h_status) return h_status;
     if (!col) return PSF_OK;
     if (nnz > capacity) return PSF_ECAPACITY;
-    const size_t fshm = shm + sizeof(int32_t) * 2 * FILL_WARPS * 32 * FILL_PAD;
-    PSF_TRY(cudaFuncSetAttribute(g_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fshm));
-    int64_t fgrid = (n + FILL_WARPS * 32 - 1) / (FILL_WARPS * 32);
-    if (fgrid > (int64_t)sm_count() * 3) fgrid = (int64_t)sm_count() * 3;
-    {
-        PSF_TIMED("g_fill_kernel", st);
-        g_fill_kernel<<<(int)fgrid, FILL_WARPS * 32, fshm, st>>>(sc, im, lors, n, row_ptr, col, val,
-                                                                status);
-    }
-    PSF_LAUNCHED();
+    rc = g_rows<GT_CSR>(sc, im, lors, n, nullptr, row_ptr, 0, col, val, status, st);
+    if (rc) return rc;
     PSF_TRY(cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st));
     PSF_TRY(cudaStreamSynchronize(st));
     return h_status;
@@ -1049,14 +1235,6 @@ __global__ void __launch_bounds__(SET_T, 4) set_count_kernel(Scan sc, Img im, Lo
             __syncwarp();
         }
     }
-}
-
-// Left shift that gives 0 for shift counts of 32 and more (PTX shl.b32
-// clamps the count; a C++ shift by 32 is undefined).
-__device__ __forceinline__ unsigned shl_clamped(unsigned v, int n) {
-    unsigned r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
-    return r;
 }
 
 // General emission of one round (any keep pattern): a keep decision per cell

@@ -19,6 +19,26 @@ def P():
     return psf
 
 
+@pytest.mark.parametrize("name", ["RING2D", "RING3D_SMALL"])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 700, 1999])
+def test_listed_rows_any_length(P, name, n):
+    """Rows of a shuffled list, some ids out of range, are the set's rows bit
+    for bit (out-of-range ids: empty rows), whatever the LORs per warp."""
+    w = I.workload(name)
+    s, im, ls = w["scanner"], w["image"], w["lors"]
+    ptr, col, val = P.sysmat_rows_set(s, im, ls)
+    L = P.lor_set_list(s, ls)
+    pick = torch.from_numpy(np.random.default_rng(n).permutation(L.shape[0])[:n]).cuda()
+    lors = L[pick].contiguous()
+    bad = torch.arange(n, device="cuda") % 5 == 3
+    lors[bad, 0] = I.n_crystals(s) + 7
+    rp, rc, rv, _ = P.sysmat_rows(s, im, lors)
+    cnt = torch.where(bad, 0, ptr[pick + 1] - ptr[pick])
+    assert torch.equal(rp[1:] - rp[:-1], cnt)
+    at = torch.repeat_interleave(ptr[pick] - rp[:-1], cnt) + torch.arange(int(cnt.sum()), device="cuda")
+    assert torch.equal(rc, col[at]) and torch.equal(rv, val[at])
+
+
 @pytest.mark.parametrize("Wt,nx,ny,dx,k", [(3, 21, 13, 1.0, 59), (4, 7, 9, 3.0, 120), (2, 18, 19, 7.0, 250),
                                            (0, 5, 5, 2.0, 61)])
 def test_voxel_driven_shapes(P, orc, Wt, nx, ny, dx, k):
