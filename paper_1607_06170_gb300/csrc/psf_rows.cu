@@ -67,48 +67,131 @@ __device__ __forceinline__ void lor_ray(Ray &r, const Scan &sc, const Img &im, c
 // the same numbers.  Bound by the integer instructions of the run lookups (64-
 // bit parameters).  400,000 event LORs on the 3D ring (81e6 entries): with a
 // thread per LOR, a lane's whole ray serial and its neighbours' rows elsewhere,
-// the count took 2.74 ms and the fill 5.32 ms; now 0.96 and 1.61 ms.
+// the count took 2.74 ms and the fill 5.32 ms; now 0.73 and 1.29 ms (0.96 and
+// 1.61 ms with make_ray's general axes and per-entry records in place of linear
+// slabs by their lower bound and 32-bit slots).
 constexpr int GT_W = 4;  // warps per CTA
 
 enum { GT_COUNT = 0, GT_CSR = 1, GT_PAD = 2 };
 
-struct GtWarp {
-    Ray ray[32];
-    long long zl[32], zh[32];        // slab: clipped parameter interval
-    int4 slab[32];                   // slab: LOR, z index, first y row, -
-    long long yl[32], yh[32];        // run: clipped parameter interval
-    int4 run[32];                    // run: LOR, first x - start, column of x = 0, -
-    long long dst[32];               // run: output slot of its first voxel - start
-    int start[64];                   // run: flattened start; INT_MAX past the last
-    int cnt[32];                     // LOR: voxels so far
+// A linear axis by the lower parameter bound of its slabs: slab k holds
+// [B + k D, B + k D + |D|).  An axis parallel to its planes is the slab
+// `fixed` of one 2^45 wide, all other slabs beyond every parameter.
+struct GtAxis {
+    long long B, D;
+    float sf, df;  // coordinate = sf + parameter * df
 };
 
-// The slab of axis a holding parameter al, with its bounds (voxel_at).
-__device__ __forceinline__ bool voxel_span(const Axis &a, long long al, int &k, long long &lo,
-                                           long long &hi) {
+struct GtRay {
+    GtAxis x, y, z;
+    long long amin, amax, minu;
+    float to_mm;
+    int slow;  // an axis is nearly parallel to its planes: make_ray's FP64 form
+};
+
+struct GtWarp {
+    GtRay ray[32];
+    longlong2 zspan[32];  // slab: clipped parameter interval
+    int4 slab[32];        // slab: LOR, z index, first y row, -
+    longlong2 yspan[32];  // run: clipped parameter interval
+    longlong2 xpos[32];   // run: lower bound of its first voxel - start, step per voxel
+    int4 run[32];         // run: column of its first voxel - start, output slot of
+                          // that voxel past the group's first - start, mm per unit, -
+    int start[64];        // run: flattened start; INT_MAX past the last
+    int cnt[32];          // LOR: voxels so far
+};
+
+__device__ __forceinline__ void gt_axis(const Axis &a, GtAxis &o, int &slow) {
+    o.sf = a.sf;
+    o.df = a.df;
+    o.D = a.DA;
+    o.B = a.DA > 0 ? a.A0 : a.A0 + a.DA;
     if (a.kind == 0) {
-        k = a.fixed;
-        lo = -FX_BIG;
-        hi = FX_BIG;
-        return true;
+        o.D = 1ll << 45;
+        o.B = -(1ll << 44) - (long long)a.fixed * o.D;
+        o.sf = (float)a.fixed + 0.5f;
+        o.df = 0.0f;
+        slow |= a.fixed >= (1 << 17);
     }
+    slow |= a.kind == 2;
+}
+
+// The slab of a linear axis (n voxels) holding parameter al and the slab's
+// lower bound: voxel_at's guess and steps.
+__device__ __forceinline__ bool gt_span(const GtAxis &a, int n, long long al, int &k,
+                                        long long &lo) {
     const float af = u32_to_f((unsigned)(al >> 8)) * 2.3283064365386963e-10f;  // 2^-32
     float g = fmaf(af, a.df, a.sf);
-    g = fminf(fmaxf(g, -2.0f), (float)a.n + 1.0f);
+    g = fminf(fmaxf(g, -2.0f), (float)n + 1.0f);
     k = f2i_rd(g);
-    const int up = a.inc ? 1 : -1;
+    lo = a.B + (long long)k * a.D;
+    const long long w = a.D < 0 ? -a.D : a.D;
+    const int up = a.D < 0 ? -1 : 1;
     for (int it = 0; it < 64; ++it) {
-        slab(a, k, lo, hi);
         if (al < lo) {
             k -= up;
-        } else if (al >= hi) {
+            lo -= w;
+        } else if (al - lo >= w) {
             k += up;
+            lo += w;
         } else {
             return true;
         }
     }
-    slab(a, k, lo, hi);
     return false;
+}
+
+// y rows [y0, y1] that LOR (id1, id2) meets in parameter interval [zl, zh) of
+// a z slab, zl and zh the slab's, clipped here: make_ray's own axes (rays with
+// a nearly parallel axis).
+__device__ __noinline__ bool gt_slow_slab(const Scan &sc, const Img &im, const double *cs, int id1,
+                                          int id2, int iz, longlong2 &zs, int &y0, int &y1) {
+    Ray r;
+    lor_ray(r, sc, im, cs, id1, id2);
+    slab(r.ax[2], iz, zs.x, zs.y);
+    zs.x = zs.x > r.amin ? zs.x : r.amin;
+    zs.y = zs.y < r.amax ? zs.y : r.amax;
+    y0 = 0;
+    y1 = -1;
+    if (zs.y <= zs.x) return true;
+    int ya, yb;
+    bool ok = voxel_at(r.ax[1], zs.x, ya);
+    ok &= voxel_at(r.ax[1], zs.y - 1, yb);
+    y0 = ya < yb ? ya : yb;
+    y1 = ya < yb ? yb : ya;
+    return ok;
+}
+
+// The voxel run [x0, x1] of such a LOR in y row iy of that slab, short ends
+// trimmed; with col, its entries stored at slot `at` (none past `room`).
+__device__ __noinline__ bool gt_slow_run(const Scan &sc, const Img &im, const double *cs, int id1,
+                                         int id2, int iz, int iy, longlong2 zs, int &x0, int &x1,
+                                         int64_t at, int64_t room, int32_t *col, float *val) {
+    Ray r;
+    lor_ray(r, sc, im, cs, id1, id2);
+    long long yl, yh;
+    slab(r.ax[1], iy, yl, yh);
+    yl = yl > zs.x ? yl : zs.x;
+    yh = yh < zs.y ? yh : zs.y;
+    x0 = 0;
+    x1 = -1;
+    if (yh <= yl) return true;
+    int xa, xb;
+    bool ok = voxel_at(r.ax[0], yl, xa);
+    ok &= voxel_at(r.ax[0], yh - 1, xb);
+    x0 = xa < xb ? xa : xb;
+    x1 = xa < xb ? xb : xa;
+    x0 = x0 < 0 ? 0 : x0;
+    x1 = x1 > im.nx - 1 ? im.nx - 1 : x1;
+    if (x1 >= x0 && chord_in_row(r.ax[0], x0, yl, yh) < r.min_units) ++x0;
+    if (x1 >= x0 && chord_in_row(r.ax[0], x1, yl, yh) < r.min_units) --x1;
+    if (col)
+        for (int ix = x0; ix <= x1 && ix - x0 < room; ++ix) {
+            col[at + ix - x0] = (iz * im.ny + iy) * im.nx + ix;
+            val[at + ix - x0] = units_to_f(chord_in_row(r.ax[0], ix, yl, yh)) *
+                                (r.len_mm * (float)(1.0 / FX));
+        }
+    return ok;
 }
 
 // Index of the lane whose inclusive prefix `incl` first exceeds f (every lane
@@ -155,7 +238,9 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
     const unsigned F = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned le = (2u << lane) - 1u;
-    const int nx = im.nx, nxy = im.nx * im.ny;
+    const int nx = im.nx;
+    // slabs and runs taken together (one where 32 could hold 2^31 rows or voxels)
+    const int spc = im.ny < (1 << 25) ? 32 : 1, rpc = nx < (1 << 25) ? 32 : 1;
     bool ok = true;
     for (int64_t k0 = ((int64_t)blockIdx.x * GT_W + warp) * G; k0 < n;
          k0 += (int64_t)gridDim.x * GT_W * G) {
@@ -174,88 +259,120 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                 z0 = z0 < 0 ? 0 : z0;
                 z1 = z1 > im.nz - 1 ? im.nz - 1 : z1;
                 nsl = z1 >= z0 ? z1 - z0 + 1 : 0;
-                W.ray[lane] = r;
+                GtRay &o = W.ray[lane];
+                int slow = 0;
+                gt_axis(r.ax[0], o.x, slow);
+                gt_axis(r.ax[1], o.y, slow);
+                gt_axis(r.ax[2], o.z, slow);
+                o.amin = r.amin;
+                o.amax = r.amax;
+                o.minu = r.min_units;
+                o.to_mm = r.len_mm * (float)(1.0 / FX);
+                o.slow = slow;
             }
         }
         W.cnt[lane] = 0;
+        // the group's first slot; a LOR's slots follow at most 32 rows on
+        const int64_t slot0 = MODE == GT_CSR ? row_ptr[k0] : k0 * stride;
+        int rowat = 0, room = 0;  // the lane's LOR: first slot past slot0, slots
+        if (MODE == GT_CSR && mine) {
+            rowat = (int)(row_ptr[k] - slot0);
+            room = (int)(row_ptr[k + 1] - row_ptr[k]);
+        } else if (MODE == GT_PAD) {
+            rowat = lane * (int)stride;
+            room = (int)stride;
+        }
         const int incl = warp_incl_scan(nsl, lane);
         const int zfirst = z0 - (incl - nsl);  // z index = zfirst + flattened slab
         const int slabs = __shfl_sync(F, incl, 31);
         __syncwarp();
-        for (int s0 = 0; s0 < slabs; s0 += 32) {
+        for (int s0 = 0; s0 < slabs; s0 += spc) {
             // 32 slabs -> their y rows
             const int s = s0 + lane, q = owner_of(incl, s);
             const int iz = __shfl_sync(F, zfirst, q) + s;
             int rows = 0;
-            if (s < slabs) {
-                const Ray &r = W.ray[q];
-                long long zl, zh;
-                slab(r.ax[2], iz, zl, zh);
-                zl = zl > r.amin ? zl : r.amin;
-                zh = zh < r.amax ? zh : r.amax;
-                if (zh > zl) {
-                    int ya, yb;
-                    ok &= voxel_at(r.ax[1], zl, ya);
-                    ok &= voxel_at(r.ax[1], zh - 1, yb);
-                    int y0 = ya < yb ? ya : yb, y1 = ya < yb ? yb : ya;
-                    y0 = y0 < 0 ? 0 : y0;
-                    y1 = y1 > im.ny - 1 ? im.ny - 1 : y1;
-                    rows = y1 >= y0 ? y1 - y0 + 1 : 0;
-                    W.zl[lane] = zl;
-                    W.zh[lane] = zh;
-                    W.slab[lane] = make_int4(q, iz, y0, 0);
+            if (s < slabs && lane < spc) {
+                const GtRay &r = W.ray[q];
+                longlong2 zs;
+                int y0 = 0, y1 = -1;
+                if (!r.slow) {
+                    const long long zl = r.z.B + (long long)iz * r.z.D;
+                    const long long zh = zl + (r.z.D < 0 ? -r.z.D : r.z.D);
+                    zs.x = zl > r.amin ? zl : r.amin;
+                    zs.y = zh < r.amax ? zh : r.amax;
+                    if (zs.y > zs.x) {
+                        long long lo;
+                        int ya, yb;
+                        ok &= gt_span(r.y, im.ny, zs.x, ya, lo);
+                        ok &= gt_span(r.y, im.ny, zs.y - 1, yb, lo);
+                        y0 = ya < yb ? ya : yb;
+                        y1 = ya < yb ? yb : ya;
+                    }
+                } else {
+                    ok &= gt_slow_slab(sc, im, cs, lors[2 * (k0 + q)], lors[2 * (k0 + q) + 1], iz,
+                                       zs, y0, y1);
                 }
+                y0 = y0 < 0 ? 0 : y0;
+                y1 = y1 > im.ny - 1 ? im.ny - 1 : y1;
+                rows = y1 >= y0 ? y1 - y0 + 1 : 0;
+                W.zspan[lane] = zs;
+                W.slab[lane] = make_int4(q, iz, y0, 0);
             }
             const int rincl = warp_incl_scan(rows, lane);
             const int nrows = __shfl_sync(F, rincl, 31);
             __syncwarp();
-            for (int f0 = 0; f0 < nrows; f0 += 32) {
+            for (int f0 = 0; f0 < nrows; f0 += rpc) {
                 // 32 (slab, y row) pairs -> their voxel runs
                 const int f = f0 + lane, o = owner_of(rincl, f);
                 const int before = __shfl_sync(F, rincl - rows, o);
-                int c = 0, rq = -1, x0 = 0, base = 0;
-                long long yl = 0, yh = 0;
-                if (f < nrows) {
-                    const int4 sl = W.slab[o];
+                int c = 0, rq = -1, x0 = 0, x1 = -1, iy = 0, slow = 0;
+                int4 sl = make_int4(0, 0, 0, 0);
+                longlong2 ys = make_longlong2(0, 0), zs = ys;
+                long long la = 0, step = 0;
+                if (f < nrows && lane < rpc) {
+                    sl = W.slab[o];
+                    zs = W.zspan[o];
                     rq = sl.x;
-                    const Ray &r = W.ray[rq];
-                    const int iy = sl.z + (f - before);
-                    const long long zl = W.zl[o], zh = W.zh[o];
-                    slab(r.ax[1], iy, yl, yh);
-                    yl = yl > zl ? yl : zl;
-                    yh = yh < zh ? yh : zh;
-                    if (yh > yl) {
-                        int x1;
-                        long long la, ha, lb, hb;
-                        ok &= voxel_span(r.ax[0], yl, x0, la, ha);
-                        ok &= voxel_span(r.ax[0], yh - 1, x1, lb, hb);
-                        if (x0 > x1) {
-                            const int t = x0;
-                            x0 = x1;
-                            x1 = t;
-                            const long long tl = la, th = ha;
-                            la = lb;
-                            ha = hb;
-                            lb = tl;
-                            hb = th;
+                    iy = sl.z + (f - before);
+                    const GtRay &r = W.ray[rq];
+                    slow = r.slow;
+                    if (!slow) {
+                        const long long yl = r.y.B + (long long)iy * r.y.D;
+                        const long long yh = yl + (r.y.D < 0 ? -r.y.D : r.y.D);
+                        ys.x = yl > zs.x ? yl : zs.x;
+                        ys.y = yh < zs.y ? yh : zs.y;
+                        if (ys.y > ys.x) {
+                            const GtAxis X = r.x;
+                            const long long w = X.D < 0 ? -X.D : X.D, minu = r.minu;
+                            long long lb;
+                            step = X.D;
+                            // voxels at the run's two parameter ends; x falls
+                            // along the ray when D < 0
+                            ok &= gt_span(X, nx, X.D < 0 ? ys.y - 1 : ys.x, x0, la);
+                            ok &= gt_span(X, nx, X.D < 0 ? ys.x : ys.y - 1, x1, lb);
+                            if (x0 < 0) {
+                                x0 = 0;
+                                la = X.B;
+                            }
+                            if (x1 > nx - 1) {
+                                x1 = nx - 1;
+                                lb = X.B + (long long)x1 * X.D;
+                            }
+                            const long long ha = la + w < ys.y ? la + w : ys.y;
+                            const long long hb = lb + w < ys.y ? lb + w : ys.y;
+                            const bool cut_a = ha - (la > ys.x ? la : ys.x) < minu;
+                            const bool cut_b = hb - (lb > ys.x ? lb : ys.x) < minu;
+                            if (x1 >= x0 && cut_a) {
+                                ++x0;
+                                la += X.D;
+                            }
+                            if (x1 >= x0 && cut_b) --x1;
                         }
-                        if (x0 < 0) {
-                            x0 = 0;
-                            slab(r.ax[0], x0, la, ha);
-                        }
-                        if (x1 > nx - 1) {
-                            x1 = nx - 1;
-                            slab(r.ax[0], x1, lb, hb);
-                        }
-                        la = la > yl ? la : yl;
-                        ha = ha < yh ? ha : yh;
-                        lb = lb > yl ? lb : yl;
-                        hb = hb < yh ? hb : yh;
-                        if (x1 >= x0 && ha - la < r.min_units) ++x0;
-                        if (x1 >= x0 && hb - lb < r.min_units) --x1;
-                        c = x1 >= x0 ? x1 - x0 + 1 : 0;
-                        base = sl.y * nxy + iy * nx;
+                    } else {
+                        ok &= gt_slow_run(sc, im, cs, lors[2 * (k0 + rq)], lors[2 * (k0 + rq) + 1],
+                                          sl.y, iy, zs, x0, x1, 0, 0, nullptr, nullptr);
                     }
+                    c = x1 >= x0 ? x1 - x0 + 1 : 0;
                 }
                 // entries before this run: in the chunk, and in its LOR
                 const int eincl = warp_incl_scan(c, lane), off = eincl - c;
@@ -269,21 +386,27 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                     const int total = __shfl_sync(F, eincl, 31);
                     const unsigned live = __ballot_sync(F, c > 0);
                     const int nrun = __popc(live), at = __popc(live & (le >> 1));
+                    const int ra = __shfl_sync(F, rowat, rq >= 0 ? rq : 0);
+                    const int rm = __shfl_sync(F, room, rq >= 0 ? rq : 0);
                     if (c > 0) {
-                        const int64_t kq = k0 + rq;
-                        const int64_t first = MODE == GT_CSR ? row_ptr[kq] : kq * stride;
-                        const int64_t room =
-                            (MODE == GT_CSR ? row_ptr[kq + 1] : first + stride) - first;
                         const int inrow = had + off - ofirst;
-                        if (inrow + c > room) ok = false;  // never after a consistent count
+                        const bool fits = inrow + c <= rm;
+                        ok &= fits;  // always, after a consistent count
                         W.start[at] = off;
-                        W.dst[at] = inrow + c > room ? -1 : first + inrow - off;
-                        W.run[at] = make_int4(rq, x0 - off, base, 0);
-                        W.yl[at] = yl;
-                        W.yh[at] = yh;
+                        W.yspan[at] = ys;
+                        W.xpos[at] = make_longlong2(la - (long long)off * step, step);
+                        W.run[at] = make_int4((sl.y * im.ny + iy) * nx + x0 - off,
+                                              fits && !slow ? ra + inrow - off : INT32_MIN,
+                                              __float_as_int(W.ray[rq].to_mm), 0);
+                        if (slow)
+                            gt_slow_run(sc, im, cs, lors[2 * (k0 + rq)], lors[2 * (k0 + rq) + 1],
+                                        sl.y, iy, zs, x0, x1, slot0 + ra + inrow, rm - inrow, col,
+                                        val);
                     }
                     W.start[nrun + lane] = 0x7fffffff;
                     __syncwarp();
+                    int32_t *cdst = col + slot0;
+                    float *vdst = val + slot0;
                     int gbase = -1;  // run holding the entry before the step
                     for (int e0 = 0; e0 < total; e0 += 32) {
                         const unsigned B =
@@ -292,15 +415,15 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                         if (e < total) {
                             const int g = gbase + __popc(B & le);
                             const int4 R = W.run[g];
-                            const long long d = W.dst[g];
-                            const Ray &r = W.ray[R.x];
-                            const int ix = R.y + e;
+                            const longlong2 xp = W.xpos[g], yb = W.yspan[g];
+                            const long long lo = xp.x + (long long)e * xp.y;
+                            const long long hi = lo + (xp.y < 0 ? -xp.y : xp.y);
                             const float ch =
-                                units_to_f(chord_in_row(r.ax[0], ix, W.yl[g], W.yh[g])) *
-                                (r.len_mm * (float)(1.0 / FX));
-                            if (d >= 0) {
-                                col[d + e] = R.z + ix;
-                                val[d + e] = ch;
+                                units_to_f((hi < yb.y ? hi : yb.y) - (lo > yb.x ? lo : yb.x)) *
+                                __int_as_float(R.z);
+                            if (R.y != INT32_MIN) {
+                                cdst[R.y + e] = R.x + e;
+                                vdst[R.y + e] = ch;
                             }
                         }
                         gbase += __popc(B);
@@ -310,7 +433,7 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
             }
         }
         if (MODE != GT_CSR && mine) counts[k] = W.cnt[lane];
-        if (MODE == GT_CSR && mine && row_ptr[k] + W.cnt[lane] != row_ptr[k + 1]) ok = false;
+        if (MODE == GT_CSR && mine) ok &= W.cnt[lane] == room;
         __syncwarp();
     }
     if (!ok) atomicExch(status, PSF_EDEBUG);
@@ -637,7 +760,9 @@ static int g_rows(const Scan &sc, const Img &im, const int32_t *lors, int64_t n,
                                                           shm));
     const int64_t cap = (int64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
     int G = 32;
-    while (G > 1 && n < cap * GT_W * G) G /= 2;
+    while (G > 1 && (n < cap * GT_W * G ||
+                     G * ((int64_t)im.nx + im.ny + im.nz) > (1 << 30)))  // 32-bit slots in a group
+        G /= 2;
     const int64_t need = (n + GT_W * G - 1) / (GT_W * G);
     {
         PSF_TIMED(MODE == GT_COUNT ? "g_rows_kernel<count>" : "g_rows_kernel<fill>", st);
