@@ -272,6 +272,33 @@ int psf_sysmat_rows(const psf_scanner *scanner, const psf_image *image, const in
                     int64_t capacity, int64_t *nnz_out, void *stream);
 
 /*
+ * The PSF rows A = S G of psf_sysmat_rows in two calls that share a workspace
+ * of the caller's, so that a caller that sizes its arrays from the entry count
+ * has the rows merged once (psf_sysmat_rows merges them for the size query and
+ * again for the fill).  No counterpart in the paper.
+ *  psf_psf_rows_workspace: *bytes (host) = device bytes of the workspace, 0 when
+ *    n_lors is 0 or the list is too large for it (above 256 MiB: use
+ *    psf_sysmat_rows).  Host only; PSF_EINVAL where psf_sysmat_rows refuses the
+ *    image, window or scanner.
+ *  psf_psf_rows_merge: merges the rows into the workspace (device, 16-byte
+ *    aligned), writes row_ptr and *nnz_out (host); synchronises `stream` once.
+ *    PSF_ECAPACITY when the merged rows do not fit the workspace.
+ *  psf_psf_rows_emit: writes col, val and row_scale (dtype as in
+ *    psf_sysmat_rows; room for *nnz_out entries) from that workspace and
+ *    row_ptr, after a psf_psf_rows_merge of the same scanner, image and n_lors
+ *    on the same stream.  Does not synchronise.
+ */
+int psf_psf_rows_workspace(const psf_scanner *scanner, const psf_image *image, int64_t n_lors,
+                           int32_t half_t, int32_t half_a, int64_t *bytes);
+int psf_psf_rows_merge(const psf_scanner *scanner, const psf_image *image, const int32_t *lors,
+                       int64_t n_lors, const float *spread, int32_t half_t, int32_t half_a,
+                       int64_t *row_ptr, void *workspace, int64_t bytes, int64_t *nnz_out,
+                       void *stream);
+int psf_psf_rows_emit(const psf_scanner *scanner, const psf_image *image, int64_t n_lors,
+                      int32_t dtype, const int64_t *row_ptr, const void *workspace, int32_t *col,
+                      void *val, float *row_scale, void *stream);
+
+/*
  * Geometric rows G of a structured LOR set (rows in set order), the same
  * matrix psf_sysmat_rows returns for the list psf_lor_set_list writes, with
  * the same conventions, size query, capacity rule and synchronisation.  All

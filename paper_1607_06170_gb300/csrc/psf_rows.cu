@@ -585,11 +585,39 @@ __global__ void __launch_bounds__(SCAN_T) scan_apply_kernel(int64_t *__restrict_
     }
 }
 
+// The whole scan by one CTA, for arrays that three launches would only wait for.
+constexpr int SCAN1_T = 1024;
+constexpr int64_t SCAN1_N = 8192;
+
+__global__ void __launch_bounds__(SCAN1_T) scan_one_kernel(int64_t *__restrict__ x, int64_t n) {
+    __shared__ int64_t sh[32];
+    __shared__ int64_t last;
+    int64_t carry = 0;
+    for (int64_t b = 0; b < n; b += SCAN1_T * 2) {
+        const int64_t i = b + 2 * threadIdx.x;
+        const int64_t v0 = i < n ? x[i] : 0, v1 = i + 1 < n ? x[i + 1] : 0;
+        const int64_t inc = carry + block_incl_scan(v0 + v1, sh);
+        if (i < n) x[i] = inc - v1;
+        if (i + 1 < n) x[i + 1] = inc;
+        if (threadIdx.x == SCAN1_T - 1) last = inc;
+        __syncthreads();
+        carry = last;
+        __syncthreads();
+    }
+}
+
 int64_t scan_tile_count(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
 
 // In-place inclusive scan of x[0..n) (int64); tile_sums has ceil(n/TILE) slots.
 int inclusive_scan(int64_t *x, int64_t n, int64_t *tile_sums, cudaStream_t st) {
     if (n <= 0) return PSF_OK;
+    // a CTA scans 2048 values in about 2 us; three launches take about 12 us
+    if (n <= SCAN1_N) {
+        PSF_TIMED("scan_one_kernel", st);
+        scan_one_kernel<<<1, SCAN1_T, 0, st>>>(x, n);
+        PSF_LAUNCHED();
+        return PSF_OK;
+    }
     int64_t nt = (n + SCAN_TILE - 1) / SCAN_TILE;
     {
         PSF_TIMED("scan_tiles_kernel", st);
@@ -630,32 +658,71 @@ __device__ __forceinline__ __nv_bfloat16 to_val<__nv_bfloat16>(float v) {
 template <>
 __device__ __forceinline__ __half to_val<__half>(float v) { return __float2half_rn(v); }
 
-constexpr int MERGE_T = 256;
+// Geometric rows as the merge reads them: CSR (ptr), or row k at k * stride
+// with cnt[k] entries.
+struct MergeSrc {
+    const int64_t *ptr, *cnt;
+    int64_t stride;
+    const int32_t *col;
+    const float *val;
+};
 
-// pass 0: counts[m] = nnz of row m;  pass 1: write row m.
-template <typename VT>
-__global__ void __launch_bounds__(MERGE_T) merge_kernel(
-    int pass, Scan sc, int64_t nvox, const int32_t *__restrict__ lors, int64_t n,
-    const int32_t *__restrict__ map, const int64_t *__restrict__ gptr,
-    const int32_t *__restrict__ gcol, const float *__restrict__ gval,
-    const float *__restrict__ w, int Wt, int Wa, int64_t *__restrict__ counts_or_ptr,
-    int32_t *__restrict__ col, VT *__restrict__ val, float *__restrict__ row_scale) {
+// Where merged rows go.  MG_TEMP: row m's entries anywhere in (tcol, tval), at
+// off[m], and its count, length and largest value; MG_COUNT: the counts only;
+// MG_FILL: the CSR arrays at row_ptr.
+enum { MG_TEMP = 0, MG_COUNT = 1, MG_FILL = 2 };
+struct MergeOut {
+    int64_t *counts;
+    int64_t *off;
+    float *rmax;
+    unsigned long long *cursor;
+    int64_t cap;
+    int32_t *tcol;
+    float *tval;
+    const int64_t *row_ptr;
+    int32_t *col;
+    void *val;
+    float *row_scale;
+};
+
+// A CTA per merged row.  The sources (geometric LORs whose window lands on the
+// row) are listed in window order, then added one after the other into the
+// row's dense image in shared memory -- a source's voxels are distinct, so its
+// entries add in parallel and the sums have a fixed order -- the next source's
+// entries loaded while the current ones add; then each warp compacts its part
+// of the image.  A chain of about 50 sources, so it is bound by latency: 128
+// threads (one entry each of most sources) and as many CTAs as the images fit.
+// RING2D, 2,016 rows: 22 us (57 us a pass, twice, when 256 threads added
+// sources of 40 entries with each fetched after the one before was added).  The
+// merged rows go to a workspace once and are written out from there, so a sized
+// call traces and merges once: 1.48 -> 0.125 ms with the outputs' allocation.
+template <int MODE, typename VT>
+__global__ void __launch_bounds__(256) merge_kernel(Scan sc, int nvox, const int32_t *__restrict__ lors, int64_t n,
+                             const int32_t *__restrict__ map, MergeSrc g,
+                             const float *__restrict__ w, int Wt, int Wa, MergeOut o) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int E = (2 * Wt + 1) * (2 * Wa + 1), W2a = 2 * Wa + 1;
     const int NC = 2 * E * E;
-    float *acc = (float *)smraw;                         // [nvox]
-    int32_t *src = (int32_t *)(acc + nvox);              // [NC] source row or -1
-    float *sw = (float *)(src + NC);                     // [NC] weight
-    int *red = (int *)(sw + NC);                         // [MERGE_T/32 + 2]
-    float *redf = (float *)(red + MERGE_T / 32 + 2);     // [MERGE_T/32]
+    float *acc = (float *)smraw;             // [nvox]
+    int32_t *src = (int32_t *)(acc + nvox);  // [NC] source row or -1, then the listed ones
+    float *sw = (float *)(src + NC);         // [NC] weight
+    __shared__ int red[9];  // per warp; the last the listed sources
+    __shared__ float redf[8];
+    __shared__ long long s_off;
     const int64_t nc = (int64_t)sc.Nt * sc.NR;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nw = T >> 5;
+    const unsigned F = 0xffffffffu, lt = (1u << lane) - 1u;
+    const int seg = (nvox + T - 1) / T * 32;  // voxels of a warp
+    const int v0 = warp * seg < nvox ? warp * seg : nvox;
+    const int v1 = v0 + seg < nvox ? v0 + seg : nvox;
+    for (int v = t; v < nvox; v += T) acc[v] = 0.0f;
+    auto first = [&](int row) { return g.ptr ? g.ptr[row] : row * g.stride; };
+    auto length = [&](int row) { return (int)(g.ptr ? g.ptr[row + 1] - g.ptr[row] : g.cnt[row]); };
     for (int64_t m = blockIdx.x; m < n; m += gridDim.x) {
-        for (int64_t v = t; v < nvox; v += MERGE_T) acc[v] = 0.0f;
         const int X = lors[2 * m], Y = lors[2 * m + 1];
         const int rX = X / sc.Nt, tX = X - rX * sc.Nt;
         const int rY = Y / sc.Nt, tY = Y - rY * sc.Nt;
-        for (int c = t; c < NC; c += MERGE_T) {
+        for (int c = t; c < NC; c += T) {
             int cs = c / (E * E), e = c - cs * E * E;
             int e1 = e / E, e2 = e - e1 * E;
             int dt1 = e1 / W2a - Wt, da1 = e1 % W2a - Wa;
@@ -673,7 +740,7 @@ __global__ void __launch_bounds__(MERGE_T) merge_kernel(
                     row = map[g1 * nc + g2];
                     if (row >= 0) {
                         wv = w[(int64_t)row * E * E + e];
-                        if (!(wv > 0.0f) || gptr[row + 1] == gptr[row]) row = -1;
+                        if (!(wv > 0.0f) || length(row) == 0) row = -1;
                     }
                 }
             }
@@ -681,61 +748,140 @@ __global__ void __launch_bounds__(MERGE_T) merge_kernel(
             sw[c] = wv;
         }
         __syncthreads();
-        // accumulate the sources in candidate order (deterministic)
-        for (int c = 0; c < NC; ++c) {
-            int32_t row = src[c];
-            if (row < 0) continue;
-            float wv = sw[c];
-            for (int64_t j = gptr[row] + t; j < gptr[row + 1]; j += MERGE_T)
-                acc[gcol[j]] += wv * gval[j];
+        if (warp == 0) {  // the listed sources move to the front, in order
+            int ns = 0;
+            for (int b = 0; b < NC; b += 32) {
+                const int c = b + lane;
+                const int row = c < NC ? src[c] : -1;
+                const float wv = c < NC ? sw[c] : 0.0f;
+                const unsigned on = __ballot_sync(F, row >= 0);
+                __syncwarp();
+                if (row >= 0) {
+                    src[ns + __popc(on & lt)] = row;
+                    sw[ns + __popc(on & lt)] = wv;
+                }
+                ns += __popc(on);
+                __syncwarp();
+            }
+            if (lane == 0) red[8] = ns;
+        }
+        __syncthreads();
+        const int ns = red[8];
+        // add the sources in that order
+        int64_t a0 = 0;
+        int an = 0, cc = 0;
+        float cv = 0.0f;
+        auto fetch = [&](int k, int64_t &at, int &len, int &col, float &val) {
+            len = 0;
+            if (k >= ns) return;
+            at = first(src[k]);
+            len = length(src[k]);
+            if (t < len) {
+                col = g.col[at + t];
+                val = g.val[at + t];
+            }
+        };
+        fetch(0, a0, an, cc, cv);
+        for (int k = 0; k < ns; ++k) {
+            const float wv = sw[k];
+            int64_t b0 = 0;
+            int bn, bc = 0;
+            float bv = 0.0f;
+            fetch(k + 1, b0, bn, bc, bv);
+            if (t < an) acc[cc] += wv * cv;
+            for (int j = t + T; j < an; j += T) acc[g.col[a0 + j]] += wv * g.val[a0 + j];
+            a0 = b0;
+            an = bn;
+            cc = bc;
+            cv = bv;
             __syncthreads();
         }
-        // compact non-zeros in ascending voxel order
-        int64_t per = (nvox + MERGE_T - 1) / MERGE_T;
-        int64_t v0 = t * per, v1 = v0 + per < nvox ? v0 + per : nvox;
+        // non-zeros of the warp's part, then their places in ascending order
         int cnt = 0;
         float mx = 0.0f;
-        for (int64_t v = v0; v < v1; ++v) {
-            float a = acc[v];
+        for (int v = v0 + lane; v < v1; v += 32) {
+            const float a = acc[v];
             cnt += a > 0.0f;
             mx = fmaxf(mx, a);
         }
-        int inc = cnt;
-        for (int o = 1; o < 32; o <<= 1) {
-            int tt = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += tt;
+        cnt = __reduce_add_sync(F, cnt);
+        for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(F, mx, d));
+        if (lane == 0) {
+            red[warp] = cnt;
+            redf[warp] = mx;
         }
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 31) red[warp] = inc;
-        if (lane == 0) redf[warp] = mx;
         __syncthreads();
         int before = 0, total = 0;
         float rmax = 0.0f;
-        for (int w2 = 0; w2 < MERGE_T / 32; ++w2) {
-            if (w2 < warp) before += red[w2];
-            total += red[w2];
-            rmax = fmaxf(rmax, redf[w2]);
+        for (int k = 0; k < nw; ++k) {
+            if (k < warp) before += red[k];
+            total += red[k];
+            rmax = fmaxf(rmax, redf[k]);
         }
-        if (pass == 0) {
-            if (t == 0) counts_or_ptr[m] = total;
-        } else {
-            int64_t pos = counts_or_ptr[m] + before + inc - cnt;
-            float scale = 1.0f, inv = 1.0f;
-            if (row_scale) {
-                scale = rmax > 0.0f ? rmax : 1.0f;
-                inv = 1.0f / scale;
-                if (t == 0) row_scale[m] = scale;
+        if (MODE == MG_TEMP) {
+            if (t == 0) {
+                const unsigned long long at = atomicAdd(o.cursor, (unsigned long long)total);
+                s_off = (int64_t)at + total <= o.cap ? (long long)at : -1;
+                o.counts[m] = total;
+                o.off[m] = s_off;
+                o.rmax[m] = rmax;
             }
-            for (int64_t v = v0; v < v1; ++v) {
-                float a = acc[v];
-                if (a > 0.0f) {
-                    col[pos] = (int32_t)v;
-                    val[pos] = to_val<VT>(row_scale ? a * inv : a);
-                    ++pos;
+            __syncthreads();
+        }
+        if (MODE == MG_COUNT && t == 0) o.counts[m] = total;
+        const bool put = MODE == MG_FILL || (MODE == MG_TEMP && s_off >= 0);
+        int64_t pos = (MODE == MG_FILL ? o.row_ptr[m] : MODE == MG_TEMP ? s_off : 0) + before;
+        float inv = 1.0f;
+        if (MODE == MG_FILL && o.row_scale) {
+            const float scale = rmax > 0.0f ? rmax : 1.0f;
+            inv = 1.0f / scale;
+            if (t == 0) o.row_scale[m] = scale;
+        }
+        for (int b = v0; b < v1; b += 32) {  // and the image back to zero
+            const int v = b + lane;
+            const float a = v < v1 ? acc[v] : 0.0f;
+            if (v < v1) acc[v] = 0.0f;
+            const unsigned on = __ballot_sync(F, a > 0.0f);
+            if (put && a > 0.0f) {
+                const int64_t at = pos + __popc(on & lt);
+                if (MODE == MG_FILL) {
+                    o.col[at] = v;
+                    ((VT *)o.val)[at] = to_val<VT>(o.row_scale ? a * inv : a);
+                } else {
+                    o.tcol[at] = v;
+                    o.tval[at] = a;
                 }
             }
+            pos += __popc(on);
         }
         __syncthreads();
+    }
+}
+
+// Merged rows from where the merge put them to the CSR arrays, in the value
+// format: a warp per row.
+template <typename VT>
+__global__ void __launch_bounds__(256) merge_emit_kernel(
+    int64_t n, const int64_t *__restrict__ row_ptr, const int64_t *__restrict__ off,
+    const float *__restrict__ rmax, const int32_t *__restrict__ tcol,
+    const float *__restrict__ tval, int32_t *__restrict__ col, VT *__restrict__ val,
+    float *__restrict__ row_scale) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t m = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); m < n;
+         m += (int64_t)gridDim.x * 8) {
+        const int64_t a = row_ptr[m], from = off[m];
+        const int len = (int)(row_ptr[m + 1] - a);
+        float inv = 1.0f;
+        if (row_scale) {
+            const float scale = rmax[m] > 0.0f ? rmax[m] : 1.0f;
+            inv = 1.0f / scale;
+            if (lane == 0) row_scale[m] = scale;
+        }
+        for (int j = lane; j < len; j += 32) {
+            const float v = tval[from + j];
+            col[a + j] = tcol[from + j];
+            val[a + j] = to_val<VT>(row_scale ? v * inv : v);
+        }
     }
 }
 
@@ -1815,6 +1961,223 @@ extern "C" int psf_sysmat_rows_set_typed(const psf_scanner *scanner, const psf_i
     return rc;
 }
 
+namespace psf {
+
+// Images and windows the dense merge takes.
+static bool merge_ok(const Scan &sc, const Img &im, int half_t, int half_a) {
+    const int64_t E = (2 * (int64_t)half_t + 1) * (2 * (int64_t)half_a + 1);
+    return (int64_t)im.nx * im.ny * im.nz <= 49152 && E * E <= 2401 &&
+           (int64_t)sc.Nt * sc.NR <= 4096;
+}
+
+// Workspace of a merge in one pass: the geometric rows in slots of the most
+// voxels a ray can meet, and room for merged rows four times as long (each in
+// the space its length takes; a planar row and its +-3 window merge to about
+// 2.4 times).  Lists that would need more than MERGE_SPACE_MAX take two passes
+// over exactly sized rows instead.
+constexpr size_t MERGE_SPACE_MAX = (size_t)256 << 20;
+
+struct MergeSpace {
+    size_t head, tiles, map, gcnt, off, rmax, gcol, gval, tcol, tval, total;
+    int64_t stride, cap;
+};
+
+static MergeSpace merge_space(const Scan &sc, const Img &im, int64_t n) {
+    MergeSpace s;
+    const int64_t nc = (int64_t)sc.Nt * sc.NR, nvox = (int64_t)im.nx * im.ny * im.nz;
+    s.stride = (int64_t)im.nx + im.ny + im.nz;
+    s.cap = n * (4 * s.stride < nvox ? 4 * s.stride : nvox);
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t here = at;
+        at += (bytes + 15) & ~(size_t)15;
+        return here;
+    };
+    s.head = take(64);  // status word, entry cursor
+    s.tiles = take(sizeof(int64_t) * scan_tile_count(n));
+    s.map = take(sizeof(int32_t) * nc * nc);
+    s.gcnt = take(sizeof(int64_t) * n);
+    s.off = take(sizeof(int64_t) * n);
+    s.rmax = take(sizeof(float) * n);
+    s.gcol = take(sizeof(int32_t) * n * s.stride);
+    s.gval = take(sizeof(float) * n * s.stride);
+    s.tcol = take(sizeof(int32_t) * s.cap);
+    s.tval = take(sizeof(float) * s.cap);
+    s.total = at;
+    return s;
+}
+
+template <int MODE, typename VT>
+static int merge_launch(const Scan &sc, const Img &im, const int32_t *lors, int64_t n,
+                        const int32_t *map, const MergeSrc &g, const float *spread, int half_t,
+                        int half_a, const MergeOut &o, cudaStream_t st) {
+    const int nvox = im.nx * im.ny * im.nz;
+    const int E = (2 * half_t + 1) * (2 * half_a + 1);
+    const size_t shm = sizeof(float) * nvox + (sizeof(int32_t) + sizeof(float)) * 2 * E * E;
+    // 128 threads take most sources in one step; an image that leaves an SM
+    // room for only one or two CTAs gets 256
+    const int threads = shm <= 64 * 1024 ? 128 : 256;
+    PSF_TRY(cudaFuncSetAttribute(merge_kernel<MODE, VT>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    int per_sm = 0;
+    PSF_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, merge_kernel<MODE, VT>, threads,
+                                                          shm));
+    const int64_t cap = (int64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
+    {
+        PSF_TIMED("merge_kernel", st);
+        merge_kernel<MODE, VT><<<(int)(n < cap ? n : cap), threads, shm, st>>>(
+            sc, nvox, lors, n, map, g, spread, half_t, half_a, o);
+    }
+    PSF_LAUNCHED();
+    return PSF_OK;
+}
+
+static int merge_map(const Scan &sc, const int32_t *lors, int64_t n, int32_t *map,
+                     cudaStream_t st) {
+    const int64_t nc = (int64_t)sc.Nt * sc.NR;
+    PSF_TRY(cudaMemsetAsync(map, 0xff, sizeof(int32_t) * nc * nc, st));
+    {
+        PSF_TIMED("pair_map_kernel", st);
+        pair_map_kernel<<<grid_for(n, 256), 256, 0, st>>>(lors, n, nc, map);
+    }
+    PSF_LAUNCHED();
+    return PSF_OK;
+}
+
+// The merged rows into the workspace and their row_ptr; PSF_ECAPACITY (with
+// *nnz_out) when they do not fit.  Synchronises once.
+static int merge_rows(const Scan &sc, const Img &im, const int32_t *lors, int64_t n,
+                      const float *spread, int half_t, int half_a, int64_t *row_ptr,
+                      const MergeSpace &sp, unsigned char *ws, int64_t *nnz_out, cudaStream_t st) {
+    int *status = reinterpret_cast<int *>(ws + sp.head);
+    unsigned long long *cursor = reinterpret_cast<unsigned long long *>(ws + sp.head + 16);
+    int32_t *map = reinterpret_cast<int32_t *>(ws + sp.map);
+    int64_t *gcnt = reinterpret_cast<int64_t *>(ws + sp.gcnt);
+    int32_t *gcol = reinterpret_cast<int32_t *>(ws + sp.gcol);
+    float *gval = reinterpret_cast<float *>(ws + sp.gval);
+    PSF_TRY(cudaMemsetAsync(ws + sp.head, 0, 64, st));
+    PSF_TRY(cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), st));
+    int rc = merge_map(sc, lors, n, map, st);
+    if (rc) return rc;
+    rc = g_rows<GT_PAD>(sc, im, lors, n, gcnt, nullptr, sp.stride, gcol, gval, status, st);
+    if (rc) return rc;
+    MergeOut o{};
+    o.counts = row_ptr + 1;
+    o.off = reinterpret_cast<int64_t *>(ws + sp.off);
+    o.rmax = reinterpret_cast<float *>(ws + sp.rmax);
+    o.cursor = cursor;
+    o.cap = sp.cap;
+    o.tcol = reinterpret_cast<int32_t *>(ws + sp.tcol);
+    o.tval = reinterpret_cast<float *>(ws + sp.tval);
+    rc = merge_launch<MG_TEMP, float>(sc, im, lors, n, map,
+                                      MergeSrc{nullptr, gcnt, sp.stride, gcol, gval}, spread,
+                                      half_t, half_a, o, st);
+    if (rc) return rc;
+    rc = inclusive_scan(row_ptr + 1, n, reinterpret_cast<int64_t *>(ws + sp.tiles), st);
+    if (rc) return rc;
+    unsigned long long head[3] = {0, 0, 0};  // status, -, entries (the cursor's end)
+    PSF_TRY(cudaMemcpyAsync(head, ws + sp.head, sizeof head, cudaMemcpyDeviceToHost, st));
+    PSF_TRY(cudaStreamSynchronize(st));
+    *nnz_out = (int64_t)head[2];
+    const int h_status = (int)(unsigned)head[0];
+    if (h_status) return h_status;
+    return (int64_t)head[2] > sp.cap ? PSF_ECAPACITY : PSF_OK;
+}
+
+static int merge_emit(const MergeSpace &sp, const unsigned char *ws, int64_t n, int dtype,
+                      const int64_t *row_ptr, int32_t *col, void *val, float *row_scale,
+                      cudaStream_t st) {
+    const int64_t need = (n + 7) / 8, cap = (int64_t)sm_count() * 8;
+    auto launch = [&](auto *v) -> int {
+        using VT = std::remove_pointer_t<decltype(v)>;
+        {
+            PSF_TIMED("merge_emit_kernel", st);
+            merge_emit_kernel<VT><<<(int)(need < cap ? need : cap), 256, 0, st>>>(
+                n, row_ptr, reinterpret_cast<const int64_t *>(ws + sp.off),
+                reinterpret_cast<const float *>(ws + sp.rmax),
+                reinterpret_cast<const int32_t *>(ws + sp.tcol),
+                reinterpret_cast<const float *>(ws + sp.tval), col, v, row_scale);
+        }
+        PSF_LAUNCHED();
+        return PSF_OK;
+    };
+    if (dtype == PSF_F32) return launch((float *)val);
+    if (dtype == PSF_BF16) return launch((__nv_bfloat16 *)val);
+    return launch((__half *)val);
+}
+
+// The same rows through exactly sized geometric rows, merged once to count and
+// once to fill (lists whose workspace would be too large).
+static int merge_rows_exact(const Scan &sc, const Img &im, const int32_t *lors, int64_t n,
+                            const float *spread, int half_t, int half_a, int dtype,
+                            int64_t *row_ptr, int32_t *col, void *val, float *row_scale,
+                            int64_t capacity, int64_t *nnz_out, cudaStream_t st) {
+    const int64_t nc = (int64_t)sc.Nt * sc.NR, ntiles = scan_tile_count(n);
+    // scratch: G (ptr, col, val), pair map, scan tiles, status
+    int64_t gnnz = 0;
+    int64_t *gptr = nullptr;
+    unsigned char *misc = nullptr;
+    int32_t *gcol = nullptr;
+    float *gval = nullptr;
+    int rc = PSF_OK;
+    if (cudaMallocAsync(&gptr, sizeof(int64_t) * (n + 1), st) != cudaSuccess ||
+        cudaMallocAsync(&misc, sizeof(int64_t) * ntiles + sizeof(int32_t) * nc * nc + 256, st) !=
+            cudaSuccess)
+        rc = PSF_ECUDA;
+    int64_t *tiles = reinterpret_cast<int64_t *>(misc);
+    int32_t *map = reinterpret_cast<int32_t *>(tiles + ntiles);
+    int *status = reinterpret_cast<int *>(map + nc * nc);
+    if (!rc && cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) rc = PSF_ECUDA;
+    if (!rc) rc = geom_rows(sc, im, lors, n, gptr, nullptr, nullptr, 0, &gnnz, tiles, status, st);
+    if (!rc && (cudaMallocAsync(&gcol, sizeof(int32_t) * (gnnz + 1), st) != cudaSuccess ||
+                cudaMallocAsync(&gval, sizeof(float) * (gnnz + 1), st) != cudaSuccess))
+        rc = PSF_ECUDA;
+    if (!rc) rc = g_rows<GT_CSR>(sc, im, lors, n, nullptr, gptr, 0, gcol, gval, status, st);
+    if (!rc) rc = merge_map(sc, lors, n, map, st);
+    const MergeSrc g{gptr, nullptr, 0, gcol, gval};
+    MergeOut o{};
+    o.counts = row_ptr + 1;
+    o.row_ptr = row_ptr;
+    o.col = col;
+    o.val = val;
+    o.row_scale = row_scale;
+    if (!rc && cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), st) != cudaSuccess) rc = PSF_ECUDA;
+    if (!rc)
+        rc = merge_launch<MG_COUNT, float>(sc, im, lors, n, map, g, spread, half_t, half_a, o, st);
+    if (!rc) rc = inclusive_scan(row_ptr + 1, n, tiles, st);
+    int64_t nnz = 0;
+    int h_status = 0;
+    if (!rc) {
+        if (cudaMemcpyAsync(&nnz, row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st) !=
+                cudaSuccess ||
+            cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            rc = PSF_ECUDA;
+        *nnz_out = nnz;
+        if (!rc) rc = h_status;
+    }
+    if (!rc && col) {
+        if (nnz > capacity) rc = PSF_ECAPACITY;
+        else if (dtype == PSF_F32)
+            rc = merge_launch<MG_FILL, float>(sc, im, lors, n, map, g, spread, half_t, half_a, o,
+                                              st);
+        else if (dtype == PSF_BF16)
+            rc = merge_launch<MG_FILL, __nv_bfloat16>(sc, im, lors, n, map, g, spread, half_t,
+                                                      half_a, o, st);
+        else
+            rc = merge_launch<MG_FILL, __half>(sc, im, lors, n, map, g, spread, half_t, half_a, o,
+                                               st);
+    }
+    if (gcol) cudaFreeAsync(gcol, st);
+    if (gval) cudaFreeAsync(gval, st);
+    if (gptr) cudaFreeAsync(gptr, st);
+    if (misc) cudaFreeAsync(misc, st);
+    return rc;
+}
+
+}  // namespace psf
+
 extern "C" int psf_sysmat_rows(const psf_scanner *scanner, const psf_image *image,
                                const int32_t *lors, int64_t n_lors, const float *spread,
                                int32_t half_t, int32_t half_a, int32_t dtype, int64_t *row_ptr,
@@ -1833,7 +2196,6 @@ extern "C" int psf_sysmat_rows(const psf_scanner *scanner, const psf_image *imag
     if (col && !val) return PSF_EINVAL;
     if (n_lors > 0 && !lors) return PSF_EINVAL;
     cudaStream_t st = as_stream(stream);
-    const int64_t nvox = (int64_t)im.nx * im.ny * im.nz;
     const int64_t ntiles = (n_lors + SCAN_TILE - 1) / SCAN_TILE + 1;
     *nnz_out = 0;
     if (!spread) {
@@ -1853,86 +2215,83 @@ extern "C" int psf_sysmat_rows(const psf_scanner *scanner, const psf_image *imag
         return rc;
     }
     // PSF rows A = S G, merged densely per output row
-    if (half_t < 0 || half_a < 0) return PSF_EINVAL;
-    const int E = (2 * half_t + 1) * (2 * half_a + 1);
-    const int64_t nc = (int64_t)sc.Nt * sc.NR;
-    if (nvox > 49152 || E * E > 2401 || nc > 4096) return PSF_EINVAL;
+    if (!merge_ok(sc, im, half_t, half_a)) return PSF_EINVAL;
     if (n_lors == 0) {
         PSF_TRY(cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), st));
         return PSF_OK;
     }
-    // scratch: G (ptr, col, val), pair map, scan tiles, status
-    int64_t gnnz = 0;
-    int64_t *gptr = nullptr;
-    void *misc = nullptr;
-    size_t misc_bytes = sizeof(int64_t) * ntiles + sizeof(int32_t) * nc * nc + 256;
-    PSF_TRY(cudaMallocAsync(&gptr, sizeof(int64_t) * (n_lors + 1), st));
-    PSF_TRY(cudaMallocAsync(&misc, misc_bytes, st));
-    int64_t *tiles = (int64_t *)misc;
-    int32_t *map = (int32_t *)(tiles + ntiles);
-    int *status = (int *)(map + nc * nc);
-    cudaMemsetAsync(status, 0, sizeof(int), st);
-    int32_t *gcol = nullptr;
-    float *gval = nullptr;
-    rc = geom_rows(sc, im, lors, n_lors, gptr, nullptr, nullptr, 0, &gnnz, tiles, status, st);
-    if (!rc) {
-        if (cudaMallocAsync(&gcol, sizeof(int32_t) * (gnnz + 1), st) != cudaSuccess ||
-            cudaMallocAsync(&gval, sizeof(float) * (gnnz + 1), st) != cudaSuccess)
-            rc = PSF_ECUDA;
+    const MergeSpace sp = merge_space(sc, im, n_lors);
+    if (sp.total <= MERGE_SPACE_MAX) {
+        unsigned char *ws = nullptr;
+        PSF_TRY(cudaMallocAsync(&ws, sp.total, st));
+        rc = merge_rows(sc, im, lors, n_lors, spread, half_t, half_a, row_ptr, sp, ws, nnz_out, st);
+        const bool crowded = rc == PSF_ECAPACITY;  // more entries than the workspace has room for
+        if (!rc && col) rc = *nnz_out > capacity ? PSF_ECAPACITY
+                                                 : merge_emit(sp, ws, n_lors, dtype, row_ptr, col,
+                                                              val, row_scale, st);
+        cudaFreeAsync(ws, st);
+        if (!crowded) return rc;
     }
-    if (!rc)
-        rc = geom_rows(sc, im, lors, n_lors, gptr, gcol, gval, gnnz, &gnnz, tiles, status, st);
-    if (!rc) {
-        cudaMemsetAsync(map, 0xff, sizeof(int32_t) * nc * nc, st);
-        {
-            PSF_TIMED("pair_map_kernel", st);
-            pair_map_kernel<<<grid_for(n_lors, 256), 256, 0, st>>>(lors, n_lors, nc, map);
-        }
-        size_t shm = sizeof(float) * nvox + (sizeof(int32_t) + sizeof(float)) * 2 * E * E +
-                     sizeof(int) * (MERGE_T / 32 + 2) + sizeof(float) * (MERGE_T / 32) + 16;
-        int grid = sm_count() * 4;
-        auto launch = [&](int pass, auto *vptr) -> int {
-            using VT = std::remove_pointer_t<decltype(vptr)>;
-            PSF_TRY(cudaFuncSetAttribute(merge_kernel<VT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-            {
-                PSF_TIMED("merge_kernel", st);
-                merge_kernel<VT><<<grid, MERGE_T, shm, st>>>(
-                    pass, sc, nvox, lors, n_lors, map, gptr, gcol, gval, spread, half_t, half_a,
-                    pass == 0 ? row_ptr + 1 : row_ptr, col, vptr, row_scale);
-            }
-            PSF_LAUNCHED();
-            return PSF_OK;
-        };
-        cudaMemsetAsync(row_ptr, 0, sizeof(int64_t), st);
-        rc = launch(0, (float *)nullptr);
-        if (!rc) rc = inclusive_scan(row_ptr + 1, n_lors, tiles, st);
-        int64_t nnz = 0;
-        if (!rc) {
-            if (cudaMemcpyAsync(&nnz, row_ptr + n_lors, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                                st) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess)
-                rc = PSF_ECUDA;
-            *nnz_out = nnz;
-        }
-        if (!rc && col) {
-            if (nnz > capacity) {
-                rc = PSF_ECAPACITY;
-            } else if (dtype == PSF_F32) {
-                rc = launch(1, (float *)val);
-            } else if (dtype == PSF_BF16) {
-                rc = launch(1, (__nv_bfloat16 *)val);
-            } else {
-                rc = launch(1, (__half *)val);
-            }
-        }
-    }
-    if (gcol) cudaFreeAsync(gcol, st);
-    if (gval) cudaFreeAsync(gval, st);
-    cudaFreeAsync(gptr, st);
-    cudaFreeAsync(misc, st);
-    if (!rc && cudaStreamSynchronize(st) != cudaSuccess) rc = PSF_ECUDA;
-    return rc;
+    return merge_rows_exact(sc, im, lors, n_lors, spread, half_t, half_a, dtype, row_ptr, col, val,
+                            row_scale, capacity, nnz_out, st);
+}
+
+extern "C" int psf_psf_rows_workspace(const psf_scanner *scanner, const psf_image *image,
+                                      int64_t n_lors, int32_t half_t, int32_t half_a,
+                                      int64_t *bytes) {
+    Scan sc;
+    Img im;
+    int rc = make_scan(scanner, &sc);
+    if (rc) return rc;
+    rc = make_img(image, &im);
+    if (rc) return rc;
+    if (!bytes || n_lors < 0 || half_t < 0 || half_a < 0) return PSF_EINVAL;
+    if (!merge_ok(sc, im, half_t, half_a)) return PSF_EINVAL;
+    const MergeSpace sp = merge_space(sc, im, n_lors);
+    *bytes = n_lors > 0 && sp.total <= MERGE_SPACE_MAX ? (int64_t)sp.total : 0;
+    return PSF_OK;
+}
+
+extern "C" int psf_psf_rows_merge(const psf_scanner *scanner, const psf_image *image,
+                                  const int32_t *lors, int64_t n_lors, const float *spread,
+                                  int32_t half_t, int32_t half_a, int64_t *row_ptr,
+                                  void *workspace, int64_t bytes, int64_t *nnz_out, void *stream) {
+    PSF_RANGE("psf_psf_rows_merge");
+    Scan sc;
+    Img im;
+    int rc = make_scan(scanner, &sc);
+    if (rc) return rc;
+    rc = make_img(image, &im);
+    if (rc) return rc;
+    if (!nnz_out || !row_ptr || !lors || !spread || !workspace || n_lors < 1 || half_t < 0 ||
+        half_a < 0)
+        return PSF_EINVAL;
+    if (!merge_ok(sc, im, half_t, half_a)) return PSF_EINVAL;
+    const MergeSpace sp = merge_space(sc, im, n_lors);
+    if (sp.total > MERGE_SPACE_MAX || bytes < (int64_t)sp.total ||
+        (reinterpret_cast<uintptr_t>(workspace) & 15))
+        return PSF_EINVAL;
+    return merge_rows(sc, im, lors, n_lors, spread, half_t, half_a, row_ptr, sp,
+                      static_cast<unsigned char *>(workspace), nnz_out, as_stream(stream));
+}
+
+extern "C" int psf_psf_rows_emit(const psf_scanner *scanner, const psf_image *image,
+                                 int64_t n_lors, int32_t dtype, const int64_t *row_ptr,
+                                 const void *workspace, int32_t *col, void *val, float *row_scale,
+                                 void *stream) {
+    PSF_RANGE("psf_psf_rows_emit");
+    Scan sc;
+    Img im;
+    int rc = make_scan(scanner, &sc);
+    if (rc) return rc;
+    rc = make_img(image, &im);
+    if (rc) return rc;
+    if (n_lors < 1 || !row_ptr || !workspace || !col || !val) return PSF_EINVAL;
+    if (dtype < PSF_F32 || dtype > PSF_F16) return PSF_EINVAL;
+    if ((dtype == PSF_F32) != (row_scale == nullptr)) return PSF_EINVAL;
+    return merge_emit(merge_space(sc, im, n_lors),
+                      static_cast<const unsigned char *>(workspace), n_lors, dtype, row_ptr, col,
+                      val, row_scale, as_stream(stream));
 }
 
 // ------------------------------------------------ no-allocation entry point

@@ -17,6 +17,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "_build", "libpsf.so")
 
 PSF_F32, PSF_BF16, PSF_F16 = 0, 1, 2
+PSF_ECAPACITY = -2
 NORM_NONE, NORM_EFF, NORM_UNIT = 0, 1, 2
 _DT = {"f32": PSF_F32, "bf16": PSF_BF16, "f16": PSF_F16}
 _TORCH_DT = {PSF_F32: torch.float32, PSF_BF16: torch.bfloat16, PSF_F16: torch.float16}
@@ -32,7 +33,8 @@ FUNCTIONS = [
     "psf_forward_masked", "psf_sino_bins", "psf_voxel_homog", "psf_matrix_set_stencil_form",
     "psf_matrix_check", "psf_matrix_build_sparse_adjoint", "psf_bin_spread_classes",
     "psf_set_wait_limit", "psf_matrix_create_otf", "psf_matrix_set_image",
-    "psf_spread_topn_bf16", "psf_matrix_set_spread_topn_bf16",
+    "psf_spread_topn_bf16", "psf_matrix_set_spread_topn_bf16", "psf_psf_rows_workspace",
+    "psf_psf_rows_merge", "psf_psf_rows_emit",
 ]
 
 
@@ -110,6 +112,9 @@ _SIGS = {
     "psf_set_wait_limit": (C.c_int, [_I64]),
     "psf_matrix_build_sparse_adjoint": (C.c_int, [_P, _P]),
     "psf_matrix_create_otf": (C.c_int, [_P, _P, _P, _P, _P]),
+    "psf_psf_rows_workspace": (C.c_int, [_P, _P, _I64, _I32, _I32, _P]),
+    "psf_psf_rows_merge": (C.c_int, [_P, _P, _P, _I64, _P, _I32, _I32, _P, _P, _I64, _P, _P]),
+    "psf_psf_rows_emit": (C.c_int, [_P, _P, _I64, _I32, _P, _P, _P, _P, _P, _P]),
 }
 
 _lock = threading.Lock()
@@ -344,7 +349,7 @@ def sysmat_rows(sc: dict, im: dict, lors, spread=None, half_t: int = 0, half_a: 
     """CSR rows (row_ptr int64, col int32, val, row_scale or None).
 
     Without `buffers`: a size query, then the fill into buffers of exactly the
-    required size.  With buffers=(row_ptr, col, val, row_scale) of sufficient
+    required size (PSF rows are merged once, into a workspace, for both).  With buffers=(row_ptr, col, val, row_scale) of sufficient
     capacity: one call that fills them (PSFError with PSF_ECAPACITY if short).
     """
     s, i = scanner(sc), image(im)
@@ -361,6 +366,23 @@ def sysmat_rows(sc: dict, im: dict, lors, spread=None, half_t: int = 0, half_a: 
         return row_ptr, col[: nnz.value], val[: nnz.value], row_scale
     row_ptr = torch.empty(n + 1, dtype=torch.int64, device=dev)
     row_scale = None if dt == PSF_F32 else torch.empty(n, dtype=torch.float32, device=dev)
+    room = C.c_int64()
+    if spread is not None:
+        _ok(L.psf_psf_rows_workspace(C.byref(s), C.byref(i), n, half_t, half_a, C.byref(room)),
+            "psf_sysmat_rows(size)")
+    if room.value:  # merged once into a workspace, sized, then written out
+        ws = torch.empty(room.value, dtype=torch.uint8, device=dev)
+        rc = L.psf_psf_rows_merge(C.byref(s), C.byref(i), _ptr(lors), n, _ptr(spread), half_t,
+                                  half_a, _ptr(row_ptr), _ptr(ws), room.value, C.byref(nnz),
+                                  _stream())
+        if rc != PSF_ECAPACITY:
+            _ok(rc, "psf_sysmat_rows(size)")
+            col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
+            val = torch.empty(max(nnz.value, 1), dtype=_TORCH_DT[dt], device=dev)
+            _ok(L.psf_psf_rows_emit(C.byref(s), C.byref(i), n, dt, _ptr(row_ptr), _ptr(ws),
+                                    _ptr(col), _ptr(val), _ptr(row_scale), _stream()),
+                "psf_sysmat_rows")
+            return row_ptr, col[: nnz.value], val[: nnz.value], row_scale
     _ok(L.psf_sysmat_rows(C.byref(s), C.byref(i), _ptr(lors), n, _ptr(spread), half_t, half_a,
                           dt, _ptr(row_ptr), None, None, _ptr(row_scale), 0, C.byref(nnz),
                           _stream()), "psf_sysmat_rows(size)")

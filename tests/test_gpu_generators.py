@@ -74,3 +74,54 @@ def test_truncation_whole_and_tiny_windows(P, orc, Wt, Wa, N):
     with np.errstate(over="ignore"):
         want = wo[3].astype(np.float32)
     np.testing.assert_allclose(wk.cpu().numpy()[3], want, rtol=2e-7)
+
+
+@pytest.mark.parametrize("case", ["wide window", "large list", "one row"])
+def test_merged_rows_paths(P, case):
+    """PSF rows whose merged entries outgrow the workspace (a wide window), whose
+    workspace would be too large (a list over an image of many voxels) and of a
+    single LOR: against S (G x) in 64 bits, and the 16-bit formats against FP32."""
+    w = I.workload("RING2D")
+    s, t, im, Wt = dict(w["scanner"]), w["table"], w["image"], 3
+    if case == "wide window":
+        Wt = 12
+    elif case == "large list":
+        s.update(n_blocks=32, radius=130.0)
+        im = I.image(220, 200, 1, 0.8, 0.9, 1.0)
+    nt = I.n_transaxial(s)
+    lors = P.lor_set_list(s, dict(fan_half=nt // 2 - 1, max_ring_diff=0))
+    lors = lors[32:33].contiguous() if case == "one row" else lors[:16000].contiguous()
+    n, nv = lors.shape[0], im["nx"] * im["ny"]
+    T, eta = P.response_build(s, t)
+    W = P.bin_spread(s, t, T, eta, lors, Wt, 0)
+    ptr, col, val, _ = P.sysmat_rows(s, im, lors, W, Wt, 0)
+    d = col[1:].long() - col[:-1].long()
+    inner = torch.ones(len(col) - 1, dtype=torch.bool, device="cuda") if len(col) else d.bool()
+    ends = ptr[1:-1]
+    inner[ends[(ends > 0) & (ends < len(col))] - 1] = False
+    assert bool((d[inner] > 0).all()) and bool((val > 0).all())
+    x = torch.rand(nv, device="cuda", dtype=torch.float64)
+
+    def times(p, c, v):
+        y = torch.zeros(n, device="cuda", dtype=torch.float64)
+        row = torch.repeat_interleave(torch.arange(n, device="cuda"), p[1:] - p[:-1])
+        return y.index_add_(0, row, v.double() * x[c.long()])
+
+    gx = times(*P.sysmat_rows(s, im, lors)[:3])
+    index = torch.full((nt, nt), -1, dtype=torch.int64, device="cuda")
+    index[lors[:, 0].long(), lors[:, 1].long()] = torch.arange(n, device="cuda")
+    want = torch.zeros(n, device="cuda", dtype=torch.float64)
+    for d1 in range(-Wt, Wt + 1):
+        for d2 in range(-Wt, Wt + 1):
+            a, b = (lors[:, 0].long() + d1) % nt, (lors[:, 1].long() + d2) % nt
+            to = torch.where(a != b, torch.maximum(index[a, b], index[b, a]), -1)
+            on = (to >= 0) & (W[:, d1 + Wt, d2 + Wt] > 0)
+            want.index_add_(0, to[on], W[on, d1 + Wt, d2 + Wt].double() * gx[on])
+    # sums of positive FP32 products of at most 2 E^2 terms per voxel
+    assert_close(times(ptr, col, val).cpu(), want.cpu(), 2 * (2 * Wt + 1) ** 2 * 6e-8,
+                 1e-30, "merged rows")
+    for dt, tol in (("bf16", 2.0 ** -8), ("f16", 2.0 ** -10)):
+        p2, c2, v2, sc = P.sysmat_rows(s, im, lors, W, Wt, 0, dtype=dt)
+        assert torch.equal(p2, ptr) and torch.equal(c2, col)
+        per = torch.repeat_interleave(sc, ptr[1:] - ptr[:-1])
+        assert float((v2.float() * per - val).abs().max()) <= tol * float(sc.max())
