@@ -551,6 +551,135 @@ __global__ void __launch_bounds__(SP_THREADS, 3) spread_q_kernel(
     }
 }
 
+// Spreads of a planar ring's LORs (one window row), whose crystals have only a
+// few sub-positions: a CTA per LOR would keep 8 warps for 16 sub-LORs.  G lanes
+// take a LOR (a half-warp for 16 sub-LORs), a lane a sub-LOR; the two responses
+// go to shared memory over the whole window width, zero on the side the photon
+// does not travel to, so the window is one small product sum_s r1_s (x) r2_s
+// whatever the travel patterns, each lane owning a few of its entries (fixed
+// order over s).  Responses and node decisions are spread_q_kernel's.  Bound by
+// latency: RING2D, 2,016 LORs of 16 sub-LORs: 70 -> 18 us
+// between events (about 5 us of which are the events').
+constexpr int SPL_T = 128;
+constexpr int SPL_NSUB = 64;  // most sub-LORs: above, a warp's serial chunks lose to a CTA
+
+template <int WT, int G>
+__global__ void __launch_bounds__(SPL_T) spread_planar_kernel(
+    Scan sc, Tab tb, const float *__restrict__ T, const double *__restrict__ eta,
+    const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
+    const int32_t *__restrict__ sym) {
+    constexpr int E = 2 * WT + 1, OWN = (E * E + G - 1) / G, NG = SPL_T / G;
+    constexpr int RS = (2 * E) | 1;  // odd: the lanes' rows start in different banks
+    extern __shared__ float spl_tabs[];          // node tangents
+    __shared__ float R[NG][G][RS];                // a chunk's responses at both ends
+    const GapConst gk = make_gapconst(sc, tb, spl_tabs);
+    __syncthreads();
+    const int t = threadIdx.x, grp = t / G, l = t % G;
+    const unsigned mask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << ((t & 31) / G * G);
+    const int NP = tb.Pt * tb.Pa, nsub = NP * NP, nc = sc.Nt * sc.NR;
+    for (int64_t lor = (int64_t)blockIdx.x * NG + grp; lor < n_lors;
+         lor += (int64_t)gridDim.x * NG) {
+        if (sym && sym[lor] >= 0) continue;  // an image of another class under the mirrors
+        const int id1 = lors[2 * lor], id2 = lors[2 * lor + 1];
+        const int ring1 = id1 / sc.Nt, c1 = id1 - ring1 * sc.Nt;
+        const int ring2 = id2 / sc.Nt, c2 = id2 - ring2 * sc.Nt;
+        const int b1 = c1 / sc.Nb, i1 = c1 - b1 * sc.Nb;
+        const int b2 = c2 / sc.Nb, i2 = c2 - b2 * sc.Nb;
+        float *o = out + lor * (int64_t)(E * E);
+        if (b1 == b2 || id1 < 0 || id2 < 0 || id1 >= nc || id2 >= nc) {
+            for (int e = l; e < E * E; e += G) o[e] = 0.0f;
+            continue;
+        }
+        float sb1, cb1, sb2, cb2;
+        sincospif(2.0f * b1 / sc.R, &sb1, &cb1);
+        sincospif(2.0f * b2 / sc.R, &sb2, &cb2);
+        float acc[OWN];
+#pragma unroll
+        for (int u = 0; u < OWN; ++u) acc[u] = 0.0f;
+        double sfull = 0.0;
+        for (int s0 = 0; s0 < nsub; s0 += G) {
+            const int s = s0 + l, s1 = s / NP, s2 = s - s1 * NP;
+            float *r1 = R[grp][l], *r2 = r1 + E;
+#pragma unroll
+            for (int e = 0; e < 2 * E; ++e) r1[e] = 0.0f;
+            if (s < nsub) {
+                const int p1 = s1 / tb.Pa, q1 = s1 - p1 * tb.Pa;
+                const int p2 = s2 / tb.Pa, q2 = s2 - p2 * tb.Pa;
+                const float se1 =
+                    (i1 - 0.5f * (sc.Nb - 1)) * sc.pt + ((p1 + 0.5f) / tb.Pt - 0.5f) * sc.wt;
+                const float ze1 = sc.z0 + ring1 * sc.pa + ((q1 + 0.5f) / tb.Pa - 0.5f) * sc.wa;
+                const float se2 =
+                    (i2 - 0.5f * (sc.Nb - 1)) * sc.pt + ((p2 + 0.5f) / tb.Pt - 0.5f) * sc.wt;
+                const float ze2 = sc.z0 + ring2 * sc.pa + ((q2 + 0.5f) / tb.Pa - 0.5f) * sc.wa;
+                const float x1 = sc.radius * cb1 - se1 * sb1, y1 = sc.radius * sb1 + se1 * cb1;
+                const float x2 = sc.radius * cb2 - se2 * sb2, y2 = sc.radius * sb2 + se2 * cb2;
+                const float dx = x1 - x2, dy = y1 - y2, dz = ze1 - ze2;
+                float vn1, vt1, vn2, vt2;
+                end_dir(dx, dy, cb1, sb1, vn1, vt1);
+                end_dir(-dx, -dy, cb2, sb2, vn2, vt2);
+                if (vn1 > 0.0f && vn2 > 0.0f) {
+                    QResp<WT, 0> r;
+                    end_resp_q<WT, 0>(sc, tb, gk, T, eta, i1, ring1, p1, q1, se1, ze1, vn1, vt1,
+                                      dz, r);
+                    const double e1 = r.eta;
+                    const int g1 = vt1 >= 0.0f ? 1 : -1, g2 = vt2 >= 0.0f ? 1 : -1;
+#pragma unroll
+                    for (int x = 0; x <= WT; ++x) r1[WT + g1 * x] = r.q[x];
+                    end_resp_q<WT, 0>(sc, tb, gk, T, eta, i2, ring2, p2, q2, se2, ze2, vn2, vt2,
+                                      -dz, r);
+#pragma unroll
+                    for (int x = 0; x <= WT; ++x) r2[WT + g2 * x] = r.q[x];
+                    sfull += e1 * r.eta;
+                }
+            }
+            __syncwarp(mask);
+            const int ns = nsub - s0 < G ? nsub - s0 : G;
+#pragma unroll
+            for (int u = 0; u < OWN; ++u) {
+                const int e = l + u * G, e1 = e / E, e2 = e - e1 * E;
+                if (e < E * E)
+                    for (int k = 0; k < ns; ++k)
+                        acc[u] = fmaf(R[grp][k][e1], R[grp][k][E + e2], acc[u]);
+            }
+            __syncwarp(mask);
+        }
+        // FP64 totals: sfull over sub-LORs, sw over the accumulated window
+        double sw = 0.0;
+#pragma unroll
+        for (int u = 0; u < OWN; ++u) sw += (double)acc[u];
+#pragma unroll
+        for (int d = G / 2; d > 0; d >>= 1) {
+            sfull += __shfl_xor_sync(mask, sfull, d);
+            sw += __shfl_xor_sync(mask, sw, d);
+        }
+        double scale = 1.0 / nsub;                                          // NONE: mean
+        if (norm == PSF_NORM_EFF && sw > 0.0) scale = sfull / (sw * nsub);  // total = mean eta1 eta2
+        if (norm == PSF_NORM_UNIT && sw > 0.0) scale = 1.0 / sw;            // total = 1
+        const float fs = (float)scale;
+#pragma unroll
+        for (int u = 0; u < OWN; ++u)
+            if (l + u * G < E * E) o[l + u * G] = acc[u] * fs;
+    }
+}
+
+template <int WT, int G>
+static int launch_spread_planar(const Scan &sc, const Tab &tb, const float *T, const double *eta,
+                                const int32_t *lors, int64_t n_lors, int norm, float *out,
+                                const int32_t *sym, cudaStream_t st) {
+    const size_t shm = sizeof(float) * (2 * tb.Kt + tb.Ka);
+    int dev = 0, sms = 148;
+    PSF_TRY(cudaGetDevice(&dev));
+    PSF_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t need = (n_lors + SPL_T / G - 1) / (SPL_T / G), cap = (int64_t)sms * 8;
+    {
+        PSF_TIMED("spread_planar_kernel", st);
+        spread_planar_kernel<WT, G><<<(int)(need < cap ? need : cap), SPL_T, shm, st>>>(
+            sc, tb, T, eta, lors, n_lors, norm, out, sym);
+    }
+    PSF_LAUNCHED();
+    return PSF_OK;
+}
+
 template <int WT, int WA>
 static int launch_spread_q(const Scan &sc, const Tab &tb, const float *T, const double *eta,
                            const int32_t *lors, int64_t n_lors, int norm, float *out,
@@ -698,6 +827,13 @@ static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, co
         return launch_spread_q<3, 3>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
     if (half_t == 3 && half_a == 2)
         return launch_spread_q<3, 2>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
+    const int nsub = tb.Pt * tb.Pa * tb.Pt * tb.Pa;
+    if (half_t == 3 && half_a == 0 && nsub <= SPL_NSUB && 2 * tb.Kt + tb.Ka <= 4096)
+        return nsub <= 16
+                   ? launch_spread_planar<3, 16>(sc, tb, table, eta, lors, n_lors, norm, spread,
+                                                 sym, st)
+                   : launch_spread_planar<3, 32>(sc, tb, table, eta, lors, n_lors, norm, spread,
+                                                 sym, st);
     if (half_t == 3 && half_a == 0)
         return launch_spread_q<3, 0>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
     size_t shm = spread_smem(tb, half_t, half_a);

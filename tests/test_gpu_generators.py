@@ -125,3 +125,21 @@ def test_merged_rows_paths(P, case):
         assert torch.equal(p2, ptr) and torch.equal(c2, col)
         per = torch.repeat_interleave(sc, ptr[1:] - ptr[:-1])
         assert float((v2.float() * per - val).abs().max()) <= tol * float(sc.max())
+
+
+@pytest.mark.parametrize("n_sub", [2, 4, 8])
+@pytest.mark.parametrize("norm", [0, 1, 2])
+def test_planar_spreads(P, orc, n_sub, norm):
+    """Planar spreads with 4, 16 and 64 sub-LORs (lanes idle, a half-warp, two
+    chunks), a LOR count that leaves groups without one, every normalisation."""
+    w = I.workload("RING2D")
+    s, t = w["scanner"], dict(w["table"], n_sub_t=n_sub)
+    T, eta = P.response_build(s, t)
+    To, _ = orc.table_build(s, t)
+    L = I.workload_lors(w)[:1999]
+    got = P.bin_spread(s, t, T, eta, torch.from_numpy(L).cuda(), 3, 0, norm=norm).cpu().numpy()
+    want = orc.spread(s, t, To, L, 3, 0, norm=norm)
+    sure = orc.tie_margin(s, t, To, L) > 1e-5
+    assert sure.mean() > 0.5
+    scale = np.abs(want).reshape(len(L), -1).max(1)[:, None, None]
+    assert_close(got[sure], want[sure], 1e-5, (1e-6 * scale + 1e-30)[sure], "planar spreads")
