@@ -565,6 +565,17 @@ int psf_em_ratio(const float *y, const float *yhat, float *ratio, int64_t n, voi
 int psf_em_update(float *x, const float *bp, const float *sens, float floor, int64_t n,
                   void *stream);
 
+/* MLEM (Sec. 3), every iteration enqueued by one call: `iters` times
+ *   ratio = y / (A x),  x <- x A^T ratio / sens where sens >= 1e-12 max(sens),
+ * else 0.  given: bit 0, sens (device float [n_cols]) is an input, else A^T 1 is
+ * written to it; bit 1, x (device float [n_cols]) holds the start image, else it
+ * starts from 1 on the voxels the scanner sees (the sensitivity then comes with
+ * the first back-projection).  yhat, ratio (device float [n_rows]) and bp
+ * (device float [n_cols]) are scratch.  The floor stays on the device: the call
+ * does not synchronise. */
+int psf_mlem(const psf_matrix *m, const float *y, float *x, float *sens, int32_t given,
+             int32_t iters, float *yhat, float *ratio, float *bp, void *stream);
+
 /*
  * Kernel timing -- instrumentation of the library, no counterpart in the
  * paper.  While enabled, every kernel the library launches is bracketed by a

@@ -164,6 +164,33 @@ __host__ __device__ __forceinline__ int angle_node(float ang, float inv_step, in
     return k < K - 1 ? k : K - 1;
 }
 
+// Programmatic dependent launch.  A kernel launched with launch_after may begin
+// while the kernel before it on the stream still runs: it prepares what that
+// kernel does not write, calls grid_wait (the kernel before it has then
+// finished and its writes are visible), and only then grid_trigger, which lets
+// the next such kernel begin.  The first kernel of a chain is launched plainly,
+// so everything enqueued before the chain is visible to all of it.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_after(void (*kernel)(KArgs...), int grid, int block, size_t shm,
+                                cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = shm;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ double warp_sum_d(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;

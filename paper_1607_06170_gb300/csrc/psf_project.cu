@@ -1067,6 +1067,164 @@ __global__ void split_pair_kernel(const float2 *__restrict__ x2, float *__restri
     }
 }
 
+// MLEM on stored rows in three launches an iteration (psf_mlem): the forward
+// projection ends in the ratio y / (A x), and the image update also clears the
+// back-projection for the next iteration.  Small matrices (a planar ring's PSF
+// rows stay in L2) are bound by launches and the latency of each kernel's
+// dependent loads, so the launches are programmatic: a kernel begins while the
+// one before it runs and has its first 128 entries a row (the matrix does not
+// change) in registers when it may go on.  RING2D, 10 iterations:
+// 460 us with 4 calls and 5 launches an iteration, 166 us with one call and
+// three plain launches, 91 us now.
+template <typename VT>
+struct RowHead {  // the first 128 entries of a warp's row
+    int64_t j0, j1;
+    int c[4];
+    float v[4];
+    __device__ __forceinline__ void load(const int64_t *__restrict__ ptr,
+                                         const int32_t *__restrict__ col,
+                                         const VT *__restrict__ val, int64_t r, int lane) {
+        j0 = ptr[r];
+        j1 = ptr[r + 1];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t j = j0 + lane + 32 * u;
+            c[u] = j < j1 ? col[j] : -1;
+            v[u] = j < j1 ? ld_val(val, j) : 0.0f;
+        }
+    }
+};
+
+// ratio = y / (A x) (0 where A x <= 0); x == NULL: an image of ones, and the
+// pair image img2 [nv] and the key of the largest sensitivity are cleared.
+template <typename VT>
+__global__ void __launch_bounds__(PJ_T) mlem_ratio_kernel(
+    int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+    const VT *__restrict__ val, const float *__restrict__ scale, const float *x,
+    const float *__restrict__ y, float *__restrict__ ratio, float2 *__restrict__ img2, int64_t nv,
+    unsigned *__restrict__ key) {
+    const int lane = threadIdx.x & 31;
+    const int64_t wpb = PJ_T / 32, r0 = blockIdx.x * wpb + (threadIdx.x >> 5);
+    RowHead<VT> h;
+    float sc = 1.0f, yr = 0.0f;
+    auto head = [&](int64_t r) {
+        h.load(ptr, col, val, r, lane);
+        sc = scale ? scale[r] : 1.0f;
+        yr = y[r];
+    };
+    if (r0 < n) head(r0);
+    grid_wait();
+    grid_trigger();
+    if (!x) {
+        for (int64_t i = blockIdx.x * (int64_t)PJ_T + threadIdx.x; i < nv;
+             i += (int64_t)gridDim.x * PJ_T)
+            img2[i] = make_float2(0.0f, 0.0f);
+        if (blockIdx.x == 0 && threadIdx.x == 0) *key = 0u;
+    }
+    for (int64_t r = r0; r < n; r += gridDim.x * wpb) {
+        if (r != r0) head(r);
+        float acc = 0.0f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (h.c[u] >= 0) acc = fmaf(h.v[u], x ? x[h.c[u]] : 1.0f, acc);
+        for (int64_t j = h.j0 + 128 + lane; j < h.j1; j += 32)
+            acc = fmaf(ld_val(val, j), x ? x[col[j]] : 1.0f, acc);
+        acc = warp_sum_f(acc);
+        if (lane == 0) {
+            const float d = scale ? acc * sc : acc;
+            ratio[r] = d > 0.0f ? yr / d : 0.0f;
+        }
+    }
+}
+
+// bp += A^T ratio; PAIR: img2 += A^T (1, ratio).
+template <typename VT, bool PAIR>
+__global__ void __launch_bounds__(PJ_T) mlem_back_kernel(
+    int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+    const VT *__restrict__ val, const float *__restrict__ scale, const float *ratio,
+    float *__restrict__ bp, float2 *__restrict__ img2) {
+    const int lane = threadIdx.x & 31;
+    const int64_t wpb = PJ_T / 32, r0 = blockIdx.x * wpb + (threadIdx.x >> 5);
+    RowHead<VT> h;
+    float sc = 1.0f;
+    auto head = [&](int64_t r) {
+        h.load(ptr, col, val, r, lane);
+        sc = scale ? scale[r] : 1.0f;
+    };
+    if (r0 < n) head(r0);
+    grid_wait();
+    grid_trigger();
+    for (int64_t r = r0; r < n; r += gridDim.x * wpb) {
+        if (r != r0) head(r);
+        const float q = ratio[r] * sc;
+        if (!PAIR && q == 0.0f) continue;
+        auto add = [&](int c, float v) {
+            if (PAIR)
+                atomicAdd(img2 + c, make_float2(v * sc, v * q));
+            else
+                atomicAdd(bp + c, v * q);
+        };
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (h.c[u] >= 0) add(h.c[u], h.v[u]);
+        for (int64_t j = h.j0 + 128 + lane; j < h.j1; j += 32) add(col[j], ld_val(val, j));
+    }
+}
+
+// A float as a key that orders as the values do (not a number above all).
+__device__ __forceinline__ unsigned order_key(float v) {
+    const unsigned b = __float_as_uint(v);
+    return (b & 0x7fffffffu) > 0x7f800000u ? 0xffffffffu : (b >> 31 ? ~b : b | 0x80000000u);
+}
+
+// The largest sensitivity's key into *key (0 before); img2: sens and bp are
+// first taken from the pair image.
+__global__ void mlem_sens_kernel(const float2 *img2, float *sens, float *__restrict__ bp,
+                                 int64_t n, unsigned *__restrict__ key) {
+    grid_wait();
+    grid_trigger();
+    unsigned k = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        float s;
+        if (img2) {
+            const float2 v = img2[i];
+            s = v.x;
+            sens[i] = s;
+            bp[i] = v.y;
+        } else {
+            s = sens[i];
+        }
+        const unsigned q = order_key(s);
+        k = q > k ? q : k;
+    }
+    k = __reduce_max_sync(0xffffffffu, k);
+    if ((threadIdx.x & 31) == 0) atomicMax(key, k);
+}
+
+// x <- x bp / sens where sens >= 1e-12 max(sens), else 0 (em_update_kernel with
+// the floor from the key of the largest sensitivity); ONES: x was 1; clear: bp
+// becomes 0.
+template <bool ONES>
+__global__ void __launch_bounds__(PJ_T) mlem_update_kernel(float *x, const float *factor,
+                                                          float *bp, const float *sens,
+                                                          const unsigned *key, int64_t n,
+                                                          bool clear) {
+    grid_wait();
+    grid_trigger();
+    const unsigned k = *key;
+    const float mx = k == 0xffffffffu ? CUDART_NAN_F
+                                      : __uint_as_float(k >> 31 ? k & 0x7fffffffu : ~k);
+    const float floor_ = (float)(1e-12 * (double)mx);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const float s = sens[i];
+        const bool seen = s >= floor_ && s > 0.0f;
+        x[i] = seen ? (ONES ? 1.0f : x[i]) * factor[i] / s : 0.0f;
+        if (clear) bp[i] = 0.0f;
+    }
+}
+
 __global__ void fill_kernel(float *__restrict__ a, float v, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -3043,9 +3201,9 @@ extern "C" int psf_matrix_create(psf_matrix **out, int64_t n_rows, int64_t n_col
     m->tr_w = nullptr;
     m->tr_list = nullptr;
     m->tr_nz = nullptr;
-    // row counters [2], the status word and the stencil's pair counter, one
-    // allocation
-    if (cudaMalloc(&m->queue, 4 * sizeof(unsigned long long)) != cudaSuccess) {
+    // row counters [2], the status word, the stencil's pair counter and the
+    // key of the largest sensitivity, one allocation
+    if (cudaMalloc(&m->queue, 5 * sizeof(unsigned long long)) != cudaSuccess) {
         delete m;
         return PSF_ECUDA;
     }
@@ -3868,4 +4026,96 @@ extern "C" int psf_matrix_check(const psf_matrix *m, void *stream) {
     PSF_TRY(cudaStreamSynchronize(st));
     if (h) PSF_TRY(cudaMemsetAsync(m->status, 0, sizeof(int), st));
     return h;
+}
+
+// MLEM (Sec. 3), all iterations enqueued by one call.
+extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *sens,
+                        int32_t given, int32_t iters, float *yhat, float *ratio, float *bp,
+                        void *stream) {
+    PSF_RANGE("psf_mlem");
+    if (!m || !x || !sens || !bp || iters < 0 || given < 0 || given > 3) return PSF_EINVAL;
+    if (m->n_rows > 0 && (!y || !yhat || !ratio)) return PSF_EINVAL;
+    cudaStream_t st = as_stream(stream);
+    const bool have_sens = given & 1, have_x = given & 2;
+    const int64_t nv = m->n_cols, n = m->n_rows;
+    unsigned *key = reinterpret_cast<unsigned *>(m->queue + 4);
+    const int vgrid = grid_for(nv, PJ_T), rgrid = grid_for(n * 32, PJ_T);
+    // three launches an iteration for stored rows at the grid-stride launches
+    // (a tuned plan keeps its own kernels)
+    const bool fused = !m->factored && !m->otf && n > 0 && m->fwd_chunk == 0 && m->wq_chunk == 0;
+    // (a chain's first kernel is launched plainly: see launch_after)
+    auto launch = [&](const char *name, bool first, auto kernel, int grid, auto... args) -> int {
+        PSF_TIMED(name, st);
+        if (first)
+            kernel<<<grid, PJ_T, 0, st>>>(args...);
+        else
+            PSF_TRY(launch_after(kernel, grid, PJ_T, 0, st, args...));
+        PSF_LAUNCHED();
+        return PSF_OK;
+    };
+    auto to_ratio = [&](bool ones) -> int {
+        if (!fused) {
+            const int rc = psf_forward(m, x, yhat, stream);
+            return rc ? rc : psf_em_ratio(y, yhat, ratio, n, stream);
+        }
+        return dispatch_dtype(m->dtype, [&](auto tag) -> int {
+            using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
+            return launch("mlem_ratio_kernel", ones, mlem_ratio_kernel<VT>, rgrid, n, m->row_ptr,
+                          m->col, (const VT *)m->val, m->row_scale,
+                          ones ? (const float *)nullptr : x, y, ratio, m->img2, nv, key);
+        });
+    };
+    auto back = [&](bool pair) -> int {
+        return dispatch_dtype(m->dtype, [&](auto tag) -> int {
+            using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
+            return launch("mlem_back_kernel", false,
+                          pair ? mlem_back_kernel<VT, true> : mlem_back_kernel<VT, false>, rgrid, n,
+                          m->row_ptr, m->col, (const VT *)m->val, m->row_scale, ratio, bp,
+                          m->img2);
+        });
+    };
+    auto sens_key = [&](bool pair) -> int {  // the floor of the updates
+        if (!pair) PSF_TRY(cudaMemsetAsync(key, 0, sizeof(unsigned), st));
+        return launch("mlem_sens_kernel", !pair, mlem_sens_kernel, vgrid,
+                      pair ? m->img2 : (const float2 *)nullptr, sens, bp, nv, key);
+    };
+    auto update = [&](bool ones, const float *factor, bool clear) -> int {
+        return launch("mlem_update_kernel", false,
+                      ones ? mlem_update_kernel<true> : mlem_update_kernel<false>, vgrid, x, factor,
+                      bp, sens, key, nv, clear);
+    };
+    int rc = PSF_OK;
+    if (!have_x && !have_sens && iters > 0) {
+        // first iteration from an image of ones: its forward projection equals
+        // that of ones on the voxels the scanner sees (the others' columns are
+        // zero), so A^T 1 comes with the first back-projection
+        if (fused) {
+            rc = to_ratio(true);
+            if (!rc) rc = back(true);
+            if (!rc) rc = sens_key(true);
+        } else {
+            {
+                PSF_TIMED("fill_kernel", st);
+                fill_kernel<<<vgrid, PJ_T, 0, st>>>(x, 1.0f, nv);
+            }
+            PSF_LAUNCHED();
+            rc = to_ratio(false);
+            if (!rc) rc = psf_back_sens(m, ratio, bp, sens, stream);
+            if (!rc) rc = sens_key(false);
+        }
+        --iters;
+        if (!rc) rc = update(true, bp, fused && iters > 0);
+    } else {
+        if (!have_sens) rc = psf_sensitivity(m, sens, stream);
+        if (!rc) rc = sens_key(false);
+        // 1 on the voxels the scanner sees; a given image stays as it is
+        if (!rc && !have_x) rc = update(true, sens, false);
+        if (!rc && fused && iters > 0) PSF_TRY(cudaMemsetAsync(bp, 0, sizeof(float) * nv, st));
+    }
+    for (int it = 0; it < iters && !rc; ++it) {
+        rc = to_ratio(false);
+        if (!rc) rc = fused ? back(false) : psf_back(m, ratio, bp, stream);
+        if (!rc) rc = update(false, bp, fused && it + 1 < iters);
+    }
+    return rc;
 }

@@ -34,7 +34,7 @@ FUNCTIONS = [
     "psf_matrix_check", "psf_matrix_build_sparse_adjoint", "psf_bin_spread_classes",
     "psf_set_wait_limit", "psf_matrix_create_otf", "psf_matrix_set_image",
     "psf_spread_topn_bf16", "psf_matrix_set_spread_topn_bf16", "psf_psf_rows_workspace",
-    "psf_psf_rows_merge", "psf_psf_rows_emit",
+    "psf_psf_rows_merge", "psf_psf_rows_emit", "psf_mlem",
 ]
 
 
@@ -114,6 +114,7 @@ _SIGS = {
     "psf_matrix_create_otf": (C.c_int, [_P, _P, _P, _P, _P]),
     "psf_psf_rows_workspace": (C.c_int, [_P, _P, _I64, _I32, _I32, _P]),
     "psf_psf_rows_merge": (C.c_int, [_P, _P, _P, _I64, _P, _I32, _I32, _P, _P, _I64, _P, _P]),
+    "psf_mlem": (C.c_int, [_P, _P, _P, _P, _I32, _I32, _P, _P, _P, _P]),
     "psf_psf_rows_emit": (C.c_int, [_P, _P, _I64, _I32, _P, _P, _P, _P, _P, _P]),
 }
 
@@ -584,6 +585,20 @@ class Matrix:
             out = torch.empty(self.n_cols, dtype=torch.float32, device=y.device)
         _ok(lib().psf_back(self._h, _ptr(y), _ptr(out), _stream()), "psf_back")
         return out
+
+    def mlem(self, y, iters: int, x=None, sens=None):
+        """`iters` MLEM iterations in one call (psf_mlem): x, the start image,
+        is updated in place and returned (None: from the voxels the scanner
+        sees); sens None: A^T 1 is formed on the way."""
+        given = (1 if sens is not None else 0) | (2 if x is not None else 0)
+        new = lambda n: torch.empty(n, dtype=torch.float32, device=y.device)
+        x = new(self.n_cols) if x is None else x
+        sens = new(self.n_cols) if sens is None else sens
+        # kept until the call returns: scratch of the enqueued iterations
+        yhat, ratio, bp = new(self.n_rows), new(self.n_rows), new(self.n_cols)
+        _ok(lib().psf_mlem(self._h, _ptr(y), _ptr(x), _ptr(sens), given, int(iters), _ptr(yhat),
+                           _ptr(ratio), _ptr(bp), _stream()), "psf_mlem")
+        return x
 
     def __del__(self):
         try:

@@ -36,11 +36,14 @@ def mlem(matrix, y, iters: int = 10, x0=None, sens=None, graph: bool = False):
     """MLEM (Sec. 3): sens = A^T 1; x <- x * A^T(y / A x) / sens.
 
     Voxels with sens < 1e-12 * max(sens) are held at zero, and 0/0 in the
-    ratio is zero.  All steps are library kernels (psf_forward, psf_em_ratio,
-    psf_back, psf_em_update).  With graph=True the `iters` iterations are
-    captured once in a CUDA graph (after one uncaptured iteration on a copy,
-    which sets up the kernels' launch attributes) and replayed as one launch.
+    ratio is zero.  All steps are library kernels, enqueued by one call
+    (psf_mlem).  With graph=True the `iters` iterations (psf_forward,
+    psf_em_ratio, psf_back, psf_em_update) are captured once in a CUDA graph
+    (after one uncaptured iteration on a copy, which sets up the kernels' launch
+    attributes) and replayed as one launch.
     """
+    if not graph:
+        return matrix.mlem(y, iters, None if x0 is None else x0.clone(), sens)
     yhat = torch.empty_like(y)
     ratio = torch.empty_like(y)
     if sens is None and x0 is None and iters > 0:
@@ -72,10 +75,6 @@ def mlem(matrix, y, iters: int = 10, x0=None, sens=None, graph: bool = False):
         matrix.back(ratio, out=bp)
         psf.em_update(xi, bp, sens, floor)
 
-    if not graph:
-        for _ in range(iters):
-            iteration(x)
-        return x
     if iters == 0:
         return x
     iteration(x.clone())  # uncaptured warm-up on a scratch copy

@@ -143,3 +143,34 @@ def test_planar_spreads(P, orc, n_sub, norm):
     assert sure.mean() > 0.5
     scale = np.abs(want).reshape(len(L), -1).max(1)[:, None, None]
     assert_close(got[sure], want[sure], 1e-5, (1e-6 * scale + 1e-30)[sure], "planar spreads")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("start", ["nothing", "sens", "x0", "both"])
+@pytest.mark.parametrize("iters", [0, 1, 3])
+def test_mlem_forms(P, dtype, start, iters):
+    """psf_mlem from every start against the single steps, on a plan at its
+    default launches (fused) and at the work queue's."""
+    from paper_1607_06170_gb300.torch_api import mlem
+
+    w = I.workload("RING2D_NARROW")
+    s, t, im, ls = w["scanner"], w["table"], w["image"], w["lors"]
+    T, eta = P.response_build(s, t)
+    lors = P.lor_set_list(s, ls)
+    rows = P.sysmat_rows(s, im, lors, P.bin_spread(s, t, T, eta, lors, 3, 0), 3, 0, dtype=dtype)
+    nv = im["nx"] * im["ny"]
+    for chunk in (0, 2):
+        M = P.Matrix(*rows[:3], nv, row_scale=rows[3]).set_launch(chunk, 128)
+        y = M.forward(torch.from_numpy(I.phantom_discs(im, 3).reshape(-1)).cuda())
+        sens = M.sensitivity()
+        x0 = torch.rand(nv, device="cuda")
+        got = mlem(M, y, iters, x0 if start in ("x0", "both") else None,
+                   sens if start in ("sens", "both") else None)
+        floor = 1e-12 * float(sens.max())
+        x = torch.ones_like(sens)
+        P.em_update(x, sens, sens, floor)
+        x = x0.clone() if start in ("x0", "both") else x
+        for _ in range(iters):
+            P.em_update(x, M.back(P.em_ratio(y, M.forward(x))), sens, floor)
+        # three iterations of FP32 sums of up to 2,000 terms in another order
+        assert_close(got.cpu(), x.cpu(), 2e-5, 1e-6 * float(x.max()), "MLEM image")
