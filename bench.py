@@ -271,7 +271,8 @@ def kernel_model(name, s, t, ls, Wt, Wa, n_lors, n_cls, nnz, nv, vb=4):
     ent = (4.0 + vb) * nnz + (4.0 * n_lors if vb < 4 else 0.0)
     if name == "set_fill_kernel":  # writes column + chord, reads row_ptr
         return "hbm", ent + 8.0 * n_lors, "GB/s"
-    if name.startswith("csr_fwd"):  # column + value, row_ptr, LOR value, image
+    if name.startswith(("csr_fwd", "csr_back_single")):
+        # column + value, row_ptr, LOR value, image
         return "hbm", ent + 12.0 * n_lors + 4.0 * nv, "GB/s"
     if name.startswith(("csr_back_pair", "csr_back_patch")):
         # column + value, row_ptr, two LOR values, image pair
@@ -307,7 +308,7 @@ def kern_hbm_first(name, kern):
     """Sort key of the mixed step's roofline kernel: the HBM-bound kernel with
     the most device time (the 16-bit rows change only the HBM-bound kernels)."""
     hbm = name == "set_fill_kernel" or name.startswith(("csr_fwd", "csr_back_pair",
-                                                          "csr_back_patch"))
+                                                          "csr_back_single", "csr_back_patch"))
     return (hbm, kern[name]["ms_per_step"])
 
 

@@ -448,8 +448,10 @@ int psf_matrix_destroy(psf_matrix *m);
  * kernels (FP32 rows with 16-byte aligned column and value arrays: chunks of
  * 4096 entries brought into shared memory by cp.async.bulk copies completing
  * on an mbarrier, one chunk ahead; each chunk owns the rows that start in it),
+ * and, where psf_matrix_set_image allows it, the pair-streamed form,
  * on all-ones vectors, and keeps the fastest for psf_forward / psf_back of
- * this plan; the pair back-projection of psf_back_sens takes the faster of
+ * this plan (chunk_out / threads_out name the fastest of the others); the pair
+ * back-projection of psf_back_sens takes the faster of
  * the back launch and the bulk-staged kernel (psf_back keeps launches that
  * skip rows with y = 0, which a bulk-staged pass cannot); for a
  * factored plan with full-window spreads it also times the staged forms of the
@@ -503,18 +505,20 @@ int psf_matrix_check(const psf_matrix *m, void *stream);
 int psf_matrix_set_stencil_form(psf_matrix *m, int32_t form);
 
 /* Declare the voxel grid of the plan's columns (n_cols = nx * ny * nz, else
- * PSF_EINVAL; nx <= 65535).  No counterpart in the paper: it lets the pair
- * back-projection of psf_back_sens on a factored plan over a structured set
- * (rows in set order) accumulate each transaxial pair's rows in shared memory
- * and add each touched voxel to the image once (about 12 entries per voxel
- * on the 3D ring), instead of one global FP32-pair atomic per entry.  The
- * pair's cells are read from its direct-plane row of the middle ring; an
- * entry whose voxel is not among them, or past the shared-memory capacity,
- * takes the global atomic, so any rows give the same result up to FP32
- * summation order.  Used by default once declared (psf_matrix_autotune times
- * it against the other pair forms).  Host only; checks the division
- * constants it derives over the grid's range (grids up to 2^26 voxels;
- * PSF_EDEBUG if one fails). */
+ * PSF_EINVAL; nx <= 65535).  No counterpart in the paper: it lets the
+ * projections of a factored plan over a structured set (rows in set order,
+ * full-window spreads) work on a transaxial pair at a time, the pair's voxels
+ * held in shared memory: psf_forward reads the image there, and psf_back and
+ * psf_back_sens add each touched voxel to the image once (about 12 entries per
+ * voxel on the 3D ring), instead of one global access per entry.  The pair's
+ * cells are read from its direct-plane row of the middle ring; an entry whose
+ * voxel is not among them, or past the shared-memory capacity, takes the global
+ * access, so any rows give the same result up to FP32 summation order.  Used
+ * by default once declared where a pair's cells mostly fit
+ * (psf_matrix_autotune times it against the other forms; psf_matrix_set_launch
+ * switches psf_forward and psf_back to the launch it sets).  Host only; checks
+ * the division constants it derives over the grid's range (PSF_EDEBUG if one
+ * fails). */
 int psf_matrix_set_image(psf_matrix *m, const psf_image *image);
 
 /*

@@ -80,12 +80,13 @@ struct psf_matrix {
     psf::Scan otf_sc;
     psf::Img otf_im;
     psf::LorSet otf_ls;
-    // the voxel grid of the columns (psf_matrix_set_image): nx, ny, nz and the
-    // multiply-shift forms of the divisions by nx * ny and nx; enables the
-    // per-pair shared-memory accumulation of psf_back_sens (pair form -3)
+    // the voxel grid of the columns (psf_matrix_set_image); enables the
+    // pair-streamed projections (psf_back_sens: pair form -3)
     int img_nx, img_ny, img_nz;
-    unsigned dv_xy_m, dv_x_m;
-    int dv_xy_k, dv_x_k;
+    unsigned img_zm;  // column / (nx * ny) = umulhi(column, img_zm) >> img_zk
+    int img_zk;
+    // is a direction (forward, back) pair-streamed: 0 where it fits, 1 no, 2 yes
+    int stream_form[2];
 };
 
 namespace psf {
@@ -514,235 +515,6 @@ __global__ void csr_back_pair_kernel(int64_t n, const int64_t *__restrict__ ptr,
             }
         }
         r0 = queue ? wq_take(queue, chunk, lane) : r0 + wpg;
-    }
-}
-
-// Division by a fixed divisor with a multiply and a shift (Granlund and
-// Montgomery, 1994): for d >= 1 and every n < 2^N, n / d = (n m) >> k with
-// k = N + ceil(log2 d) and m = ceil(2^k / d).
-struct DivMagic {
-    unsigned m;  // < 2^32 for N <= 30
-    int k;
-    __host__ __device__ unsigned div(unsigned n) const {
-        return (unsigned)(((unsigned long long)n * m) >> k);
-    }
-};
-
-static DivMagic div_magic(unsigned d, unsigned long long n_end) {
-    int N = 1, l = 0;
-    while (N < 32 && (1ull << N) < n_end) ++N;
-    while ((1ull << l) < d) ++l;
-    DivMagic q;
-    q.k = N + l;
-    q.m = (unsigned)(((1ull << q.k) + d - 1) / d);
-    return q;
-}
-
-// Pair back-projection with each transaxial pair's voxels accumulated in
-// shared memory (pair form -3, factored plans whose image is set).  All ring
-// pairs of a transaxial pair cut the same 2D cells, each voxel of the pair is
-// hit by about 12 of its 1,372 rows (RING3D), and the global 8-byte reductions
-// of the row-by-row form are bound by the L2's reduction rate; here one CTA
-// per SM takes pairs from a counter, adds every entry's two products into a
-// [z slice][cell] array of float pairs in shared memory, and flushes each
-// touched voxel with one global reduction.  The cells and their voxel-order
-// positions are read from the pair's direct-plane row of the middle ring
-// (one z slice holding every cell of a pair whose plane crosses the image):
-// a per-y-row table gives a voxel's position from its x index for the y rows
-// whose cells form one run of consecutive x, so an entry outside the list
-// (or past the array's capacity) is reduced into the image directly; a
-// voxel's z slice and x/y index come from multiply-shift divisions.  The
-// entries are read 128 per warp step, independently of row boundaries.
-// Each lane keeps the start of its entries' next row in a register, so
-// following the rows costs a shared-memory read only when a row ends.
-// RING3D: 12.6 ms against 13.7 ms for the row-by-row form (timing copies
-// with parts skipped, before the register: entry stream and set-up 7.0 ms,
-// row tracking 2.2 ms, shared atomics 1.5 ms, voxel decode 1.2 ms).
-constexpr int PP_T = 1024;
-
-struct PatchGrid {
-    int nx, ny, nz, nxy;
-    DivMagic dxy, dx;  // column -> z slice, x/y index -> y row
-    int cap;           // cells of a pair held in shared memory
-    int jm;            // ring-pair index of the cell-list row
-};
-
-static size_t patch_smem_bytes(const PatchGrid &g, int nrp) {
-    return sizeof(float) * 2 * (size_t)g.nz * g.cap + sizeof(int) * (size_t)g.cap +
-           sizeof(int2) * (size_t)g.ny + sizeof(int) * 4 * (size_t)g.ny +
-           sizeof(int) * ((size_t)nrp + 1) + sizeof(float2) * (size_t)nrp;
-}
-
-static bool patch_grid(const psf_matrix *m, PatchGrid *g, int *sms_out, size_t *shm_out);
-
-template <typename VT>
-__global__ void __launch_bounds__(PP_T, 1) csr_back_patch_kernel(
-    int64_t ntp, int nrp, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-    const VT *__restrict__ val, const float *__restrict__ scale, const float *__restrict__ ya,
-    const float *__restrict__ yb, float2 *__restrict__ x2, unsigned long long *pair_ctr,
-    PatchGrid g) {
-    extern __shared__ __align__(16) unsigned char pp_raw[];
-    float *px = reinterpret_cast<float *>(pp_raw);  // [nz][cap] sums of the first LOR vector
-    float *ps = px + (size_t)g.nz * g.cap;          // [nz][cap] and of the second
-    float2 *rq = reinterpret_cast<float2 *>(ps + (size_t)g.nz * g.cap);  // [nrp] row values
-    int2 *run = reinterpret_cast<int2 *>(rq + nrp);  // [ny] y row -> x of its first cell,
-                                                     //   first cell << 16 | cells (0: none)
-    int *xyl = reinterpret_cast<int *>(run + g.ny);  // [cap] cell -> x/y index
-    int *rs = xyl + g.cap;                           // [nrp + 1] row starts in the pair
-    int *r_first = rs + nrp + 1, *r_x = r_first + g.ny, *r_end = r_x + g.ny,
-        *r_gap = r_end + g.ny;  // [ny] each: run assembly
-    __shared__ long long s_T;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    constexpr int NW = PP_T / 32;
-    for (int i = t; i < 2 * g.nz * g.cap; i += PP_T) px[i] = 0.0f;
-    for (;;) {
-        __syncthreads();  // the previous pair's flush is complete
-        if (t == 0) s_T = (long long)atomicAdd(pair_ctr, 1ull);
-        __syncthreads();
-        const long long T = s_T;
-        if (T >= ntp) return;
-        const int64_t row0 = T * nrp;
-        const int64_t E0 = ptr[row0];
-        for (int i = t; i <= nrp; i += PP_T) rs[i] = (int)(ptr[row0 + i] - E0);
-        for (int i = t; i < nrp; i += PP_T) {
-            const float sc = scale ? scale[row0 + i] : 1.0f;
-            rq[i] = make_float2(ya[row0 + i] * sc, yb[row0 + i] * sc);
-        }
-        for (int i = t; i < g.ny; i += PP_T) {
-            r_first[i] = -1;
-            r_gap[i] = 0;  // runs started in this y row, or 2 when one has a gap
-        }
-        __syncthreads();
-        const int m0 = rs[g.jm];
-        const int nc_all = rs[g.jm + 1] - m0, nc = nc_all < g.cap ? nc_all : g.cap;
-        for (int i = t; i < nc; i += PP_T) {  // the cell list and its y runs
-            const int c = col[E0 + m0 + i];
-            const int xy = c - (int)g.dxy.div((unsigned)c) * g.nxy;
-            const int iy = (int)g.dx.div((unsigned)xy), ix = xy - iy * g.nx;
-            xyl[i] = xy;
-            int iyp = -1, ixp = 0, iyn = -1;
-            if (i > 0) {
-                const int cp = col[E0 + m0 + i - 1];
-                const int xyp = cp - (int)g.dxy.div((unsigned)cp) * g.nxy;
-                iyp = (int)g.dx.div((unsigned)xyp);
-                ixp = xyp - iyp * g.nx;
-            }
-            if (i + 1 < nc) {
-                const int cn = col[E0 + m0 + i + 1];
-                const int xyn = cn - (int)g.dxy.div((unsigned)cn) * g.nxy;
-                iyn = (int)g.dx.div((unsigned)xyn);
-            }
-            if (iyp != iy) {
-                r_first[iy] = i;
-                r_x[iy] = ix;
-                atomicAdd(r_gap + iy, 1);
-            } else if (ix != ixp + 1) {
-                atomicAdd(r_gap + iy, 2);  // not consecutive in x
-            }
-            if (iyn != iy) r_end[iy] = i + 1;
-        }
-        __syncthreads();
-        for (int i = t; i < g.ny; i += PP_T) {
-            // a y row's cells are used only as one run of consecutive x (a
-            // cell list out of voxel order could split a y row in two)
-            const int f = r_first[i];
-            run[i] = f >= 0 && r_gap[i] == 1 ? make_int2(r_x[i], (f << 16) | (r_end[i] - f))
-                                             : make_int2(0, 0);
-        }
-        __syncthreads();
-        // entries in blocks of 128, entry base + lane + 32 u of each block to
-        // lane u-th (consecutive entries of a row are neighbouring cells of
-        // one z slice: consecutive words of the arrays, so the lanes' shared
-        // atomics fall on different banks); each warp takes a contiguous run
-        // of blocks, every lane finds the row of its entries by stepping
-        // forward, and the next block's entries are loaded while the current
-        // one is added
-        const int E = rs[nrp];
-        const int nblk = (E + 127) >> 7;
-        const int per = (nblk + NW - 1) / NW;
-        const int b0 = warp * per, b1 = b0 + per < nblk ? b0 + per : nblk;
-        if (b0 < b1) {
-            int r[4];    // per u: largest r with rs[r] <= the lane's entry
-            int nxt[4];  // and rs[r + 1], the start of the next row
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int key = (b0 << 7) + lane + 32 * u;
-                int lo = 0, hi = nrp - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (rs[mid] <= key) lo = mid; else hi = mid - 1;
-                }
-                r[u] = lo;
-                nxt[u] = rs[lo + 1];
-            }
-            int c4[4];
-            float v4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int rel = (b0 << 7) + lane + 32 * u;
-                c4[u] = rel < E ? __ldcs(col + E0 + rel) : 0;
-                v4[u] = rel < E ? ld_val_cs(val, E0 + rel) : 0.0f;
-            }
-            const int32_t *cb = col + E0 + lane;
-            const VT *vb = val + E0 + lane;
-            for (int bk = b0; bk < b1; ++bk) {
-                int cn[4];
-                float vn[4];
-                const int nx0 = ((bk + 1) << 7) + lane;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool ld = bk + 1 < b1 && nx0 + 32 * u < E;
-                    cn[u] = ld ? __ldcs(cb + ((bk + 1) << 7) + 32 * u) : 0;
-                    vn[u] = ld ? ld_val_cs(vb, ((bk + 1) << 7) + 32 * u) : 0.0f;
-                }
-                const int rel0 = (bk << 7) + lane;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int rel = rel0 + 32 * u;
-                    if (rel < E) {
-                        while (nxt[u] <= rel) {
-                            ++r[u];
-                            nxt[u] = rs[r[u] + 1];
-                        }
-                        const float2 q = rq[r[u]];
-                        const float pa = v4[u] * q.x, pb = v4[u] * q.y;
-                        const int c = c4[u];
-                        const int iz = (int)g.dxy.div((unsigned)c), xy = c - iz * g.nxy;
-                        const int iy = (int)g.dx.div((unsigned)xy);
-                        const int2 ru = run[iy];
-                        const int k = xy - iy * g.nx - ru.x;
-                        const int pc = (ru.y >> 16) + k;
-                        if (((unsigned)k < (unsigned)(ru.y & 0xffff)) & (iz < g.nz)) {
-                            const int slot = iz * g.cap + pc;
-                            atomicAdd(px + slot, pa);
-                            atomicAdd(ps + slot, pb);
-                        } else {
-                            atomicAdd(x2 + c, make_float2(pa, pb));
-                        }
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    c4[u] = cn[u];
-                    v4[u] = vn[u];
-                }
-            }
-        }
-        __syncthreads();
-        // flush each touched voxel with one reduction, and clear the array
-        const float inv = 1.0f / (float)(nc > 0 ? nc : 1);
-        for (int i = t; i < g.nz * nc; i += PP_T) {
-            int iz = (int)((float)i * inv);
-            iz -= iz * nc > i ? 1 : 0;
-            iz += (iz + 1) * nc <= i ? 1 : 0;
-            const int pc = i - iz * nc, slot = iz * g.cap + pc;
-            const float2 v = make_float2(px[slot], ps[slot]);
-            if (v.x != 0.0f || v.y != 0.0f) {
-                atomicAdd(x2 + (int64_t)iz * g.nxy + xyl[pc], v);
-                px[slot] = 0.0f;
-                ps[slot] = 0.0f;
-            }
-        }
     }
 }
 
@@ -2833,6 +2605,80 @@ static int bk_table(psf_matrix *m, cudaStream_t st) {
     return PSF_OK;
 }
 
+}  // namespace psf
+
+#include "psf_pair_stream.cuh"
+
+namespace psf {
+
+// The pair-streamed form of a plan (a factored plan over the full set with its
+// image declared): its grid, and whether a pair's cells mostly fit -- the longest
+// side of the image -- so that it is the default.
+static bool pair_grid(const psf_matrix *m, int vectors, PairGrid *g, int *sms, bool *fits) {
+    if (!m->factored || m->topn > 0 || m->otf || m->img_nz <= 0 || m->n_rows == 0) return false;
+    if (m->n_rows != m->ls.ntp * m->ls.nrp) return false;
+    int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess)
+        return false;
+    const int64_t nxy = (int64_t)m->img_nx * m->img_ny;
+    if (nxy < 4 || nxy > optin || m->n_cols >= (1ll << 30)) return false;
+    g->nx = m->img_nx;
+    g->ny = m->img_ny;
+    g->nz = m->img_nz;
+    g->nxy = (int)nxy;
+    g->nrp = (int)m->ls.nrp;
+    g->zm = m->img_zm;
+    g->zk = m->img_zk;
+    const int rm = m->ls.NR / 2;  // the direct-plane row of the middle ring lists the cells
+    int64_t jm = 0;
+    for (int r = 0; r < rm; ++r) jm += m->ls.rp_count(r);
+    g->jm = (int)(jm + (rm - m->ls.rp_lo(rm)));
+    if (!pair_layout(*g, vectors, (size_t)optin - 256)) return false;  // + static shared memory
+    *fits = g->cap >= g->nx && g->cap >= g->ny;
+    return true;
+}
+
+// One pair-streamed projection (the outputs of the back-projections are added
+// to: the caller clears them).
+template <int MODE>
+static int rows_pair_stream(const psf_matrix *m, const float *in, const float *in2, float *out,
+                            float2 *out2, cudaStream_t st) {
+    PairGrid g{};
+    int sms = 0;
+    bool fits = false;
+    if (!pair_grid(m, MODE == PS_PAIR ? 2 : 1, &g, &sms, &fits)) return PSF_EINVAL;
+    PSF_TRY(cudaMemsetAsync(m->queue + 3, 0, sizeof(unsigned long long), st));  // pair counter
+    return dispatch_dtype(m->dtype, [&](auto tag) -> int {
+        using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
+        PSF_TRY(cudaFuncSetAttribute(pair_stream_kernel<VT, MODE>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.bytes));
+        const int grid = (int)(m->ls.ntp < sms ? m->ls.ntp : sms);
+        {
+            PSF_TIMED(MODE == PS_FWD    ? "csr_fwd_patch_kernel"
+                      : MODE == PS_BACK ? "csr_back_single_kernel"
+                                        : "csr_back_patch_kernel",
+                      st);
+            pair_stream_kernel<VT, MODE><<<grid, PsShape<MODE>::T, g.bytes, st>>>(
+                m->ls.ntp, m->row_ptr, m->col, (const VT *)m->val, m->row_scale, in, in2, out,
+                out2, m->queue + 3, m->status, (long long)wait_limit(), g);
+        }
+        PSF_LAUNCHED();
+        return PSF_OK;
+    });
+}
+
+// Is a direction (0 forward, 1 back) pair-streamed: as timed, else where it fits.
+static bool use_pair_stream(const psf_matrix *m, int dir) {
+    if (m->stream_form[dir]) return m->stream_form[dir] == 2;
+    PairGrid g{};
+    int sms = 0;
+    bool fits = false;
+    return pair_grid(m, 1, &g, &sms, &fits) && fits;
+}
+
 static int rows_fwd_with(const psf_matrix *m, const float *x, float *y, int chunk, int threads,
                          cudaStream_t st) {
     if (chunk == -2) {  // bulk-staged chunks
@@ -2938,6 +2784,7 @@ static int rows_fwd(const psf_matrix *m, const float *x, float *y, cudaStream_t 
     if (m->otf)
         return otf_rows_fwd(m->otf_sc, m->otf_im, m->otf_ls, nullptr, nullptr, x, y, m->status,
                             st);
+    if (use_pair_stream(m, 0)) return rows_pair_stream<PS_FWD>(m, x, nullptr, y, nullptr, st);
     return rows_fwd_with(m, x, y, m->fwd_chunk, m->fwd_threads, st);
 }
 
@@ -2946,6 +2793,10 @@ static int rows_back(const psf_matrix *m, const float *y, float *x, cudaStream_t
         PSF_TRY(cudaMemsetAsync(x, 0, sizeof(float) * m->n_cols, st));
         return otf_rows_back(m->otf_sc, m->otf_im, m->otf_ls, nullptr, nullptr, y, x, m->status,
                              st);
+    }
+    if (use_pair_stream(m, 1)) {
+        PSF_TRY(cudaMemsetAsync(x, 0, sizeof(float) * m->n_cols, st));
+        return rows_pair_stream<PS_BACK>(m, y, nullptr, x, nullptr, st);
     }
     return rows_back_with(m, y, x, m->wq_chunk, m->wq_threads, st);
 }
@@ -3668,15 +3519,38 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
                 m->wq_chunk = bc;
                 m->wq_threads = bt;
             }
+            // against the pair-streamed form, where the plan allows it
+            PairGrid sg{};
+            int ssms = 0;
+            bool sfits = false;
+            m->stream_form[dir] = 1;
+            if (pair_grid(m, 1, &sg, &ssms, &sfits)) {
+                for (int rep = 0; rep < 3 && !rc; ++rep) {
+                    float ms = 0.0f;
+                    if (cudaEventRecord(e0, st) != cudaSuccess) rc = PSF_ECUDA;
+                    m->stream_form[dir] = 2;
+                    if (!rc) rc = dir == 0 ? rows_fwd(m, x, y, st) : rows_back(m, y, x, st);
+                    m->stream_form[dir] = 1;
+                    if (!rc && (cudaEventRecord(e1, st) != cudaSuccess ||
+                                cudaEventSynchronize(e1) != cudaSuccess ||
+                                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+                        rc = PSF_ECUDA;
+                    if (!rc && rep > 0 && ms < best) {
+                        best = ms;
+                        bc = -4;
+                    }
+                }
+                if (!rc && bc == -4) m->stream_form[dir] = 2;
+            }
         }
         // the pair back-projection of psf_back_sens: the back launch or the
         // bulk-staged kernel (the single back keeps the row-skipping launches:
         // a bulk-staged pass streams every chunk whatever y holds)
         m->pair_form = 0;
-        PatchGrid pg;
+        PairGrid pg{};
         int psms = 0;
-        size_t pshm = 0;
-        const bool patch = patch_grid(m, &pg, &psms, &pshm);
+        bool pfits = false;
+        const bool patch = pair_grid(m, 2, &pg, &psms, &pfits);
         if ((bulk || patch) && !rc) {
             const int forms[3] = {0, -2, -3};
             float best[3] = {1e30f, 1e30f, 1e30f};
@@ -3752,23 +3626,25 @@ extern "C" int psf_matrix_set_image(psf_matrix *m, const psf_image *image) {
     Img im;
     int rc = make_img(image, &im);
     if (rc) return rc;
-    const int64_t nxy = (int64_t)im.nx * im.ny, nv = nxy * im.nz;
+    const int64_t nv = (int64_t)im.nx * im.ny * im.nz;
     if (nv != m->n_cols || im.nx > 65535 || nv >= (1ll << 30)) return PSF_EINVAL;
-    const DivMagic a = div_magic((unsigned)nxy, (unsigned long long)nv),
-                   b = div_magic((unsigned)im.nx, (unsigned long long)nxy);
-    if (nv <= (1ll << 26)) {  // the theorem, checked over the grid's range
-        for (int64_t n = 0; n < nv; ++n)
-            if (a.div((unsigned)n) != (unsigned)(n / nxy)) return PSF_EDEBUG;
-        for (int64_t n = 0; n < nxy; ++n)
-            if (b.div((unsigned)n) != (unsigned)(n / im.nx)) return PSF_EDEBUG;
-    }
+    // Division by nx * ny with a multiply and a shift (Granlund and Montgomery,
+    // 1994): for d >= 1 and every n < 2^30, n / d = (n m) >> k with k = 30 +
+    // ceil(log2 d) and m = ceil(2^k / d) < 2^32; k >= 32 for d >= 4, so the shift
+    // is a multiply-high and a shift by k - 32
+    const int64_t nxy = (int64_t)im.nx * im.ny;
+    int l = 0;
+    while ((1ll << l) < nxy) ++l;
+    const unsigned long long zm = ((1ull << (30 + l)) + nxy - 1) / nxy;
+    // (checked where the quotient steps: it is monotone)
+    for (int64_t z = 0; z < im.nz && l >= 2; ++z)
+        for (int64_t n = z * nxy; n < nv && n <= (z + 1) * nxy - 1; n += nxy > 1 ? nxy - 1 : 1)
+            if ((int64_t)(((unsigned long long)n * zm) >> (30 + l)) != z) return PSF_EDEBUG;
+    m->img_zm = (unsigned)zm;
+    m->img_zk = l - 2;
     m->img_nx = im.nx;
     m->img_ny = im.ny;
     m->img_nz = im.nz;
-    m->dv_xy_m = a.m;
-    m->dv_xy_k = a.k;
-    m->dv_x_m = b.m;
-    m->dv_x_k = b.k;
     return PSF_OK;
 }
 
@@ -3795,6 +3671,7 @@ extern "C" int psf_matrix_set_launch(psf_matrix *m, int32_t chunk, int32_t threa
     m->wq_chunk = chunk > 0 || chunk == -2 ? chunk : 0;
     m->wq_threads = chunk > 0 ? threads : 0;
     m->pair_form = chunk == -2 ? -2 : 0;
+    m->stream_form[0] = m->stream_form[1] = 1;  // the launch asked for
     return PSF_OK;
 }
 
@@ -3891,10 +3768,10 @@ extern "C" int psf_back_sens(const psf_matrix *m, const float *y, float *x, floa
     // autotuner)
     int form = m->pair_form;
     if (form == 0) {
-        PatchGrid g;
+        PairGrid g{};
         int sms = 0;
-        size_t shm = 0;
-        form = patch_grid(m, &g, &sms, &shm) ? -3 : 0;
+        bool fits = false;
+        form = pair_grid(m, 2, &g, &sms, &fits) && fits ? -3 : 0;
     } else if (form == 1) {
         form = 0;
     }
@@ -3910,74 +3787,14 @@ extern "C" int psf_back_sens(const psf_matrix *m, const float *y, float *x, floa
 
 namespace psf {
 
-// The launch of the per-pair shared-memory form: its grid (one CTA per SM),
-// the cells a pair may hold, and whether the plan allows it (a factored plan
-// over the full set with its image declared).
-static bool patch_grid(const psf_matrix *m, PatchGrid *g, int *sms_out, size_t *shm_out) {
-    if (!m->factored || m->topn > 0 || m->otf || m->img_nz <= 0 || m->n_rows == 0) return false;
-    if (m->n_rows != m->ls.ntp * m->ls.nrp) return false;
-    int dev = 0, sms = 0, optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-            cudaSuccess)
-        return false;
-    g->nx = m->img_nx;
-    g->ny = m->img_ny;
-    g->nz = m->img_nz;
-    g->nxy = m->img_nx * m->img_ny;
-    g->dxy.m = m->dv_xy_m;
-    g->dxy.k = m->dv_xy_k;
-    g->dx.m = m->dv_x_m;
-    g->dx.k = m->dv_x_k;
-    const int rm = m->ls.NR / 2;  // the direct-plane row of the middle ring lists the cells
-    int64_t jm = 0;
-    for (int r = 0; r < rm; ++r) jm += m->ls.rp_count(r);
-    g->jm = (int)(jm + (rm - m->ls.rp_lo(rm)));
-    // + the kernel's static shared memory
-    const size_t fixed = sizeof(int2) * (size_t)g->ny + sizeof(int) * 4 * (size_t)g->ny +
-                         sizeof(int) * ((size_t)m->ls.nrp + 1) + sizeof(float2) * m->ls.nrp + 512;
-    if ((size_t)optin <= fixed) return false;
-    int cap = (int)(((size_t)optin - fixed) / (sizeof(float2) * g->nz + sizeof(int)));
-    cap = cap / 4 * 4;
-    cap = cap < 32767 ? cap : 32764;  // a cell index and a run length in 16 bits
-    if (cap < 32) return false;
-    g->cap = cap;
-    *sms_out = sms;
-    *shm_out = patch_smem_bytes(*g, (int)m->ls.nrp);
-    return true;
-}
-
-static int rows_back_patch(const psf_matrix *m, const float *qa, const float *qb,
-                           cudaStream_t st) {
-    PatchGrid g;
-    int sms = 0;
-    size_t shm = 0;
-    if (!patch_grid(m, &g, &sms, &shm)) return PSF_EINVAL;
-    PSF_TRY(cudaMemsetAsync(m->queue + 3, 0, sizeof(unsigned long long), st));  // pair counter
-    return dispatch_dtype(m->dtype, [&](auto tag) -> int {
-        using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
-        PSF_TRY(cudaFuncSetAttribute(csr_back_patch_kernel<VT>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-        {
-            PSF_TIMED("csr_back_patch_kernel", st);
-            csr_back_patch_kernel<VT><<<sms, PP_T, shm, st>>>(
-                m->ls.ntp, (int)m->ls.nrp, m->row_ptr, m->col, (const VT *)m->val,
-                m->row_scale, qa, qb, m->img2, m->queue + 3, g);
-        }
-        PSF_LAUNCHED();
-        return PSF_OK;
-    });
-}
-
-// img2 = A^T (qa, qb) as an interleaved pair: form -3 the per-pair
-// shared-memory kernel, -2 the bulk-staged kernel, else the pair kernel at
+// img2 = A^T (qa, qb) as an interleaved pair: form -3 the pair-streamed
+// kernel, -2 the bulk-staged kernel, else the pair kernel at
 // the back projection's launch.
 static int rows_back_pair(const psf_matrix *m, const float *qa, const float *qb, int form,
                           cudaStream_t st) {
     PSF_TRY(cudaMemsetAsync(m->img2, 0, sizeof(float2) * m->n_cols, st));
     if (m->otf) return PSF_EINVAL;  // psf_back_sens traces twice instead
-    if (form == -3) return rows_back_patch(m, qa, qb, st);
+    if (form == -3) return rows_pair_stream<PS_PAIR>(m, qa, qb, nullptr, m->img2, st);
     if (form == -2) {
         if (!m->bk_first) return PSF_EINVAL;
         int grid = 0;
