@@ -86,13 +86,16 @@ struct GtRay {
     GtAxis x, y, z;
     long long amin, amax, minu;
     float to_mm;
-    int slow;  // an axis is nearly parallel to its planes: make_ray's FP64 form
+    float eps;  // x coordinates this far from a plane are surely on their side of
+                // it, and leave a chord to store; > 1: never
+    int slow;   // an axis is nearly parallel to its planes: make_ray's FP64 form
 };
 
 struct GtWarp {
     GtRay ray[32];
     longlong2 zspan[32];  // slab: clipped parameter interval
-    int4 slab[32];        // slab: LOR, z index, first y row, -
+    int4 slab[32];        // slab: LOR, z index, first y row - flattened start, -
+    int sstart[64];       // slab: flattened start of its rows; INT_MAX past the last
     longlong2 yspan[32];  // run: clipped parameter interval
     longlong2 xpos[32];   // run: lower bound of its first voxel - start, step per voxel
     int4 run[32];         // run: column of its first voxel - start, output slot of
@@ -269,6 +272,15 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                 o.minu = r.min_units;
                 o.to_mm = r.len_mm * (float)(1.0 / FX);
                 o.slow = slow;
+                // The FP32 coordinate sf + a df errs by less than 1.8e-7 (|sf| +
+                // |df| + 1): the roundings of a, sf and df and of the sum.  At
+                // more than twice that (eps) from every plane its voxel is the
+                // exact one, and the piece of chord it cuts, over half of eps
+                // voxels, is stored when that is as long as the shortest stored
+                // chord.
+                const float e = 4e-7f * (fabsf(o.x.sf) + fabsf(o.x.df) + 1.0f);
+                const float w = fabsf((float)o.x.D);
+                o.eps = im.nx < (1 << 20) && 0.45f * e * w >= (float)r.min_units ? e : 2.0f;
             }
         }
         W.cnt[lane] = 0;
@@ -290,7 +302,8 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
             // 32 slabs -> their y rows
             const int s = s0 + lane, q = owner_of(incl, s);
             const int iz = __shfl_sync(F, zfirst, q) + s;
-            int rows = 0;
+            int rows = 0, slab_y0 = 0;
+            longlong2 zspan = make_longlong2(0, 0);
             if (s < slabs && lane < spc) {
                 const GtRay &r = W.ray[q];
                 longlong2 zs;
@@ -315,16 +328,29 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                 y0 = y0 < 0 ? 0 : y0;
                 y1 = y1 > im.ny - 1 ? im.ny - 1 : y1;
                 rows = y1 >= y0 ? y1 - y0 + 1 : 0;
-                W.zspan[lane] = zs;
-                W.slab[lane] = make_int4(q, iz, y0, 0);
+                zspan = zs;
+                slab_y0 = y0;
             }
             const int rincl = warp_incl_scan(rows, lane);
             const int nrows = __shfl_sync(F, rincl, 31);
+            {  // the slabs with rows, in order
+                const unsigned on = __ballot_sync(F, rows > 0);
+                const int at = __popc(on & (le >> 1)), first = rincl - rows;
+                if (rows > 0) {
+                    W.sstart[at] = first;
+                    W.zspan[at] = zspan;
+                    W.slab[at] = make_int4(q, iz, slab_y0 - first, 0);
+                }
+                W.sstart[__popc(on) + lane] = 0x7fffffff;
+            }
             __syncwarp();
+            int sbase = -1;  // slab holding the row before the step
             for (int f0 = 0; f0 < nrows; f0 += rpc) {
                 // 32 (slab, y row) pairs -> their voxel runs
-                const int f = f0 + lane, o = owner_of(rincl, f);
-                const int before = __shfl_sync(F, rincl - rows, o);
+                const unsigned SB =
+                    __reduce_or_sync(F, shl_clamped(1u, W.sstart[sbase + 1 + lane] - f0));
+                const int f = f0 + lane, o = sbase + __popc(SB & le);
+                sbase += rpc == 32 ? __popc(SB) : (int)(SB & 1u);
                 int c = 0, rq = -1, x0 = 0, x1 = -1, iy = 0, slow = 0;
                 int4 sl = make_int4(0, 0, 0, 0);
                 longlong2 ys = make_longlong2(0, 0), zs = ys;
@@ -333,7 +359,7 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                     sl = W.slab[o];
                     zs = W.zspan[o];
                     rq = sl.x;
-                    iy = sl.z + (f - before);
+                    iy = sl.z + f;
                     const GtRay &r = W.ray[rq];
                     slow = r.slow;
                     if (!slow) {
@@ -343,30 +369,46 @@ __global__ void __launch_bounds__(GT_W * 32, 5) g_rows_kernel(
                         ys.y = yh < zs.y ? yh : zs.y;
                         if (ys.y > ys.x) {
                             const GtAxis X = r.x;
-                            const long long w = X.D < 0 ? -X.D : X.D, minu = r.minu;
-                            long long lb;
                             step = X.D;
-                            // voxels at the run's two parameter ends; x falls
-                            // along the ray when D < 0
-                            ok &= gt_span(X, nx, X.D < 0 ? ys.y - 1 : ys.x, x0, la);
-                            ok &= gt_span(X, nx, X.D < 0 ? ys.x : ys.y - 1, x1, lb);
-                            if (x0 < 0) {
-                                x0 = 0;
-                                la = X.B;
+                            // x at the run's two parameter ends, in FP32
+                            const float ga =
+                                fmaf(u32_to_f((unsigned)(ys.x >> 8)) * 2.3283064365386963e-10f,
+                                     X.df, X.sf);
+                            const float gb = fmaf(
+                                u32_to_f((unsigned)((ys.y - 1) >> 8)) * 2.3283064365386963e-10f,
+                                X.df, X.sf);
+                            const float ka = floorf(ga), kb = floorf(gb), e = r.eps;
+                            const float lo = fminf(ga - ka, gb - kb), hi = fmaxf(ga - ka, gb - kb);
+                            x0 = (int)fminf(ka, kb);
+                            x1 = (int)fmaxf(ka, kb);
+                            if (lo > e && hi < 1.0f - e && x0 >= 0 && x1 < nx &&
+                                ys.y - ys.x >= r.minu) {
+                                if (MODE != GT_COUNT) la = X.B + (long long)x0 * X.D;
+                            } else {  // near a plane, or a short run: exactly
+                                const long long w = X.D < 0 ? -X.D : X.D, minu = r.minu;
+                                long long lb;
+                                // voxels at the run's two parameter ends; x falls
+                                // along the ray when D < 0
+                                ok &= gt_span(X, nx, X.D < 0 ? ys.y - 1 : ys.x, x0, la);
+                                ok &= gt_span(X, nx, X.D < 0 ? ys.x : ys.y - 1, x1, lb);
+                                if (x0 < 0) {
+                                    x0 = 0;
+                                    la = X.B;
+                                }
+                                if (x1 > nx - 1) {
+                                    x1 = nx - 1;
+                                    lb = X.B + (long long)x1 * X.D;
+                                }
+                                const long long ha = la + w < ys.y ? la + w : ys.y;
+                                const long long hb = lb + w < ys.y ? lb + w : ys.y;
+                                const bool cut_a = ha - (la > ys.x ? la : ys.x) < minu;
+                                const bool cut_b = hb - (lb > ys.x ? lb : ys.x) < minu;
+                                if (x1 >= x0 && cut_a) {
+                                    ++x0;
+                                    la += X.D;
+                                }
+                                if (x1 >= x0 && cut_b) --x1;
                             }
-                            if (x1 > nx - 1) {
-                                x1 = nx - 1;
-                                lb = X.B + (long long)x1 * X.D;
-                            }
-                            const long long ha = la + w < ys.y ? la + w : ys.y;
-                            const long long hb = lb + w < ys.y ? lb + w : ys.y;
-                            const bool cut_a = ha - (la > ys.x ? la : ys.x) < minu;
-                            const bool cut_b = hb - (lb > ys.x ? lb : ys.x) < minu;
-                            if (x1 >= x0 && cut_a) {
-                                ++x0;
-                                la += X.D;
-                            }
-                            if (x1 >= x0 && cut_b) --x1;
                         }
                     } else {
                         ok &= gt_slow_run(sc, im, cs, lors[2 * (k0 + rq)], lors[2 * (k0 + rq) + 1],
