@@ -67,7 +67,7 @@ __device__ __forceinline__ void lor_ray(Ray &r, const Scan &sc, const Img &im, c
 // the same numbers.  Bound by the integer instructions of the run lookups (64-
 // bit parameters).  400,000 event LORs on the 3D ring (81e6 entries): with a
 // thread per LOR, a lane's whole ray serial and its neighbours' rows elsewhere,
-// the count took 2.74 ms and the fill 5.32 ms; now 0.73 and 1.29 ms (0.96 and
+// the count took 2.74 ms and the fill 5.32 ms; now 0.53 and 1.20 ms (0.96 and
 // 1.61 ms with make_ray's general axes and per-entry records in place of linear
 // slabs by their lower bound and 32-bit slots).
 constexpr int GT_W = 4;  // warps per CTA

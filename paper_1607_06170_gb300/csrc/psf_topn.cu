@@ -18,24 +18,57 @@ __device__ __forceinline__ bool tn_before(float wa, unsigned ta, float wb, unsig
     return wa > wb || (wa == wb && ta < tb);
 }
 
-// s + c += x, the rounding error of s + x kept in c (Knuth's two-sum): the sum
-// of a window's weights to about 2^-46 of their sum of magnitudes in FP32.
+// s + c += x, the rounding error of s + x kept in c (Knuth's two-sum): sums
+// weights to about 2^-46 of their sum of magnitudes in FP32.
 __device__ __forceinline__ void tn_add(float &s, float &c, float x) {
     const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
     c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
     s = t;
 }
 
+// The same on two pairs at once (packed FP32 additions; a - b as b * -1 + a).
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+    return r;
+}
+__device__ __forceinline__ void tn_add2(uint64_t &s, uint64_t &c, float x, float y) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    const uint64_t t = f2_add(s, v), z = f2_sub(t, s);
+    c = f2_add(c, f2_add(f2_sub(s, f2_sub(t, z)), f2_sub(v, z)));
+    s = t;
+}
+
+// The sum over the warp of s + c (every lane's pair ends up with it).
+__device__ __forceinline__ void tn_warp(float &s, float &c) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const float so = __shfl_xor_sync(0xffffffffu, s, o);
+        const float co = __shfl_xor_sync(0xffffffffu, c, o);
+        tn_add(s, c, so);
+        c += co;
+    }
+}
+
 // One warp per LOR.  The window is copied to shared memory (asynchronous
-// copies, all in flight at once) and read three times there: its total, each
-// lane's best entry of its own contiguous piece (an odd number of words, so
-// the lanes' reads fall on different banks), and, N times, the piece of the
-// lane whose best was taken, by the whole warp, for that piece's next best --
-// so a rank costs one 32-bit warp maximum and about 3 reads a lane instead of
-// another pass over the window.  The read of the windows (9.6 KB each) bounds
-// it once the rest is cheap: RING3D, N = 5, 84,227 windows, 809 MB, 0.40 ms
-// (1.52 ms when every rank was another pass over the window in 64-bit keys
-// with a CTA barrier, and the total 2,401 FP64 additions).
+// copies, all in flight at once), and one pass over each lane's contiguous piece
+// (an odd number of words, so the lanes' reads fall on different banks) gives
+// its total and the piece's largest weight.  The N-th largest of the 32 pieces'
+// largest weights bounds the N-th weight of the window from below, so only the
+// pieces that reach it are read again, by the whole warp, for the entries that
+// do; those (a handful) rank themselves against each other.  Windows with more
+// than 32 such entries (ties, or no N positive pieces) and N above 32 take the
+// entries one after the other, each from the piece that holds the next.  Totals
+// and scale are pairs of FP32 numbers (FP64 beyond their range: the FP64 pipe
+// would cost more than all the rest).  RING3D, N = 5, 84,227 windows, 809 MB:
+// 0.27 ms (1.52 ms when every rank was another pass over the window in 64-bit
+// keys with a CTA barrier, 0.40 ms when each was taken from its piece in turn,
+// with FP64 totals).
 __global__ void __launch_bounds__(TN_W * 32) topn_kernel(const float *__restrict__ spread,
                                                          int64_t n, int Wt, int Wa, int N,
                                                          int piece, int32_t *__restrict__ idx,
@@ -44,7 +77,7 @@ __global__ void __launch_bounds__(TN_W * 32) topn_kernel(const float *__restrict
     const int W2a = 2 * Wa + 1, E = (2 * Wt + 1) * W2a, EE = E * E, words = 32 * piece;
     unsigned *tie = reinterpret_cast<unsigned *>(tn_raw);  // [words] tie rank of an entry
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const unsigned F = 0xffffffffu;
+    const unsigned F = 0xffffffffu, lt = (1u << lane) - 1u;
     float *win = reinterpret_cast<float *>(tie + words) + warp * (words + TN_MAX);  // [words]
     float *sel = win + words;                                                         // [N]
     for (int e = t; e < words; e += TN_W * 32) {
@@ -53,79 +86,159 @@ __global__ void __launch_bounds__(TN_W * 32) topn_kernel(const float *__restrict
                          abs(e2 % W2a - Wa);
         tie[e] = e < EE ? (unsigned)(dist * EE + e) : 0xffffffffu;
     }
-    for (int e = EE + lane; e < words; e += 32) win[e] = -1.0f;  // padding: after every entry
+    for (int e = EE + lane; e < words; e += 32) win[e] = 0.0f;  // padding: adds nothing
     __syncthreads();
-    // entry at `e`, ranked as the rule says (a negative weight, or none, as 0)
+    const uint32_t win32 = (uint32_t)__cvta_generic_to_shared(win);
+    // entry e's weight as the rule ranks it (a negative one, or none, as 0;
+    // padding after every entry)
     auto ranked = [&](int e) {
         const float w = win[e];
         return e < EE ? (w > 0.0f ? w : 0.0f) : -1.0f;
     };
     for (int64_t g = (int64_t)blockIdx.x * TN_W + warp; g < n; g += (int64_t)gridDim.x * TN_W) {
         const float *wg = spread + g * EE;
-        for (int e = lane; e < EE; e += 32)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
-                         ::"r"((unsigned)__cvta_generic_to_shared(win + e)), "l"(wg + e) : "memory");
+        {
+            const float *src = wg + lane;
+            uint32_t dst = win32 + 4 * lane;
+#pragma unroll 8
+            for (int e = lane; e < EE; e += 32, src += 32, dst += 128)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src)
+                             : "memory");
+        }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
-        // the lane's piece: its sum and its first entry in rank order
-        float s = 0.0f, c = 0.0f, bw = -2.0f;
-        unsigned bt = 0xffffffffu;
-        for (int j = 0; j < piece; ++j) {
-            const int e = lane * piece + j;
-            if (e >= EE) break;
-            const float w = win[e], r = w > 0.0f ? w : 0.0f;
-            const unsigned te = tie[e];
-            tn_add(s, c, w);
-            if (tn_before(r, te, bw, bt)) {
-                bw = r;
-                bt = te;
-            }
+        // the lane's piece: its sum and its largest weight (0 for none positive)
+        const float *mine = win + lane * piece;
+        uint64_t s2 = 0, c2 = 0;
+        float bw = 0.0f;
+#pragma unroll 4
+        for (int j = 0; j + 1 < piece; j += 2) {
+            const float w = mine[j], v = mine[j + 1];
+            tn_add2(s2, c2, w, v);
+            bw = fmaxf(bw, fmaxf(w, v));
         }
-        double all = warp_sum_d((double)s + (double)c);
-        if (!isfinite(all)) {  // beyond FP32's range on the way, or not a number
-            double part = 0.0;
-            for (int e = lane; e < EE; e += 32) part += (double)win[e];
-            all = warp_sum_d(part);
+        bw = fmaxf(bw, mine[piece - 1]);
+        bw = bw > 0.0f ? bw : 0.0f;
+        float s, c, sb, cb;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(s), "=f"(sb) : "l"(s2));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(c), "=f"(cb) : "l"(c2));
+        tn_add(s, c, sb);
+        tn_add(s, c, mine[piece - 1]);
+        c += cb;
+        tn_warp(s, c);
+        // T: the N-th largest piece
+        unsigned T = 0, left = N <= 32 ? F : 0u;
+        for (int k = 0; k < N && left; ++k) {
+            const bool in = (left >> lane) & 1u;
+            T = __reduce_max_sync(F, in ? __float_as_uint(bw) : 0u);
+            const unsigned who = __ballot_sync(F, in && __float_as_uint(bw) == T);
+            left &= ~(who & (0u - who));
         }
-        double kept = 0.0;
-        for (int k = 0; k < N; ++k) {
-            // the best of the lanes' bests: the weight's bits order as the
-            // weight (ranked weights are not negative; a lane without entries
-            // left takes no part)
-            const unsigned top = __reduce_max_sync(F, bw >= 0.0f ? __float_as_uint(bw) + 1u : 0u);
-            const bool mine = bw >= 0.0f && __float_as_uint(bw) + 1u == top;
-            const unsigned pt = __reduce_min_sync(F, mine ? bt : 0xffffffffu);
-            const float pw = __uint_as_float(top - 1u);
-            const int e = (int)(pt % (unsigned)EE), from = e / piece;
-            const float w = win[e];
-            kept += (double)w;
-            if (lane == 0) {
-                sel[k] = w;
-                idx[g * N + k] = e;
-            }
-            // that lane's next entry after (pw, pt), by the whole warp
-            float nw = -2.0f;
-            unsigned nt = 0xffffffffu;
-            for (int j = lane; j < piece; j += 32) {
-                const int f = from * piece + j;
-                const float r = ranked(f);
-                const unsigned tf = tie[f];
-                if (tn_before(pw, pt, r, tf) && tn_before(r, tf, nw, nt)) {
-                    nw = r;
-                    nt = tf;
+        int cnt = 33;  // candidates (33: not this way)
+        float cw = -1.0f;
+        unsigned ct = 0xffffffffu;
+        if (T > 0u && N <= 32) {
+            const float tw = __uint_as_float(T);
+            unsigned pieces = __ballot_sync(F, bw >= tw);
+            cnt = 0;
+            while (pieces && cnt <= 32) {
+                const int l = __ffs(pieces) - 1;
+                pieces &= pieces - 1;
+                for (int j0 = 0; j0 < piece; j0 += 32) {
+                    const int f = l * piece + j0 + lane;
+                    const bool on = j0 + lane < piece && ranked(f) >= tw;
+                    const unsigned m = __ballot_sync(F, on);
+                    if (on && cnt + __popc(m & lt) < 32)
+                        sel[32 + cnt + __popc(m & lt)] = __int_as_float(f);
+                    cnt += __popc(m);
                 }
             }
-            const unsigned nb = __reduce_max_sync(F, nw >= 0.0f ? __float_as_uint(nw) + 1u : 0u);
-            nt = __reduce_min_sync(
-                F, nw >= 0.0f && __float_as_uint(nw) + 1u == nb ? nt : 0xffffffffu);
-            if (lane == from) {
-                bw = nb ? __uint_as_float(nb - 1u) : -2.0f;
-                bt = nt;
+            __syncwarp();
+            if (cnt <= 32 && lane < cnt) {
+                const int f = __float_as_int(sel[32 + lane]);
+                cw = win[f];
+                ct = tie[f];
             }
         }
-        const double scale = kept != 0.0 ? all / kept : 1.0;
+        float ks = 0.0f, kc = 0.0f;
+        if (cnt <= 32) {  // (uniform) the candidates rank each other
+            int rank = 0;
+            for (int j = 0; j < cnt; ++j) {
+                const float ow = __shfl_sync(F, cw, j);
+                const unsigned ot = __shfl_sync(F, ct, j);
+                rank += tn_before(ow, ot, cw, ct);
+            }
+            const bool keep = lane < cnt && rank < N;
+            if (keep) idx[g * N + rank] = (int)(ct % (unsigned)EE);
+            __syncwarp();
+            if (keep) sel[rank] = cw;
+            ks = keep ? cw : 0.0f;
+            tn_warp(ks, kc);
+        } else {
+            // one after the other: (pw, pt) the last one taken; bw, bt: the first
+            // entry after it in the lane's piece
+            unsigned bt = 0xffffffffu;
+            bw = -2.0f;
+            for (int j = 0; j < piece; ++j) {
+                const float r = ranked(lane * piece + j);
+                const unsigned te = tie[lane * piece + j];
+                if (tn_before(r, te, bw, bt)) {
+                    bw = r;
+                    bt = te;
+                }
+            }
+            for (int k = 0; k < N; ++k) {
+                // (the weight's bits order as the weight; a lane without entries
+                // left takes no part)
+                const unsigned top =
+                    __reduce_max_sync(F, bw >= 0.0f ? __float_as_uint(bw) + 1u : 0u);
+                const bool tops = bw >= 0.0f && __float_as_uint(bw) + 1u == top;
+                const unsigned pt = __reduce_min_sync(F, tops ? bt : 0xffffffffu);
+                const float pw = __uint_as_float(top - 1u);
+                const int e = (int)(pt % (unsigned)EE), from = e / piece;
+                const float w = win[e];
+                tn_add(ks, kc, w);
+                if (lane == 0) {
+                    sel[k] = w;
+                    idx[g * N + k] = e;
+                }
+                float nw = -2.0f;
+                unsigned nt = 0xffffffffu;
+                for (int j = lane; j < piece; j += 32) {
+                    const int f = from * piece + j;
+                    const float r = ranked(f);
+                    const unsigned tf = tie[f];
+                    if (tn_before(pw, pt, r, tf) && tn_before(r, tf, nw, nt)) {
+                        nw = r;
+                        nt = tf;
+                    }
+                }
+                const unsigned nb =
+                    __reduce_max_sync(F, nw >= 0.0f ? __float_as_uint(nw) + 1u : 0u);
+                nt = __reduce_min_sync(
+                    F, nw >= 0.0f && __float_as_uint(nw) + 1u == nb ? nt : 0xffffffffu);
+                if (lane == from) {
+                    bw = nb ? __uint_as_float(nb - 1u) : -2.0f;
+                    bt = nt;
+                }
+            }
+        }
         __syncwarp();  // sel is complete
-        for (int k = lane; k < N; k += 32) wout[g * N + k] = (float)((double)sel[k] * scale);
+        // scale = total / kept, 1 when nothing was kept
+        const float as = fabsf(s), ak = fabsf(ks);
+        if (as > 1e-25f && as < 1e30f && ak > 1e-25f && ak < 1e30f) {
+            const float q = __fdiv_rn(s, ks);
+            const float rem = fmaf(-q, ks, s) + fmaf(-q, kc, c);
+            const float ql = __fdiv_rn(rem, ks);
+            for (int k = lane; k < N; k += 32) wout[g * N + k] = fmaf(sel[k], q, sel[k] * ql);
+        } else {  // near or beyond the ends of FP32's range, or not a number
+            double all = 0.0, kept = 0.0;
+            for (int e = lane; e < EE; e += 32) all += (double)win[e];
+            all = warp_sum_d(all);
+            for (int k = 0; k < N; ++k) kept += (double)sel[k];
+            const double scale = kept != 0.0 ? all / kept : 1.0;
+            for (int k = lane; k < N; k += 32) wout[g * N + k] = (float)((double)sel[k] * scale);
+        }
         __syncwarp();  // the window and sel are rewritten next
     }
 }
