@@ -423,7 +423,7 @@ int psf_matrix_set_spread_topn_bf16(psf_matrix *m, const psf_scanner *scanner,
 /* For a plan with top-N spreads (list-mode reconstruction, the next step of
  * Sec. 5): build the transpose of S -- for every measured LOR the source LORs
  * whose kept entries land on it, with their weights (plan-owned: 8 bytes per
- * kept tap, 12 bytes per LOR) -- with two passes over the taps (count, scan,
+ * kept tap, 12 bytes and a bit per LOR) -- with two passes over the taps (count, scan,
  * fill).  Afterwards S^T of an input with at most 1/16 nonzero entries (one
  * subset's counts or ratios) lists those entries and scatters from them with
  * FP32 atomics (the summation order varies between runs); denser inputs keep
@@ -579,6 +579,22 @@ int psf_em_update(float *x, const float *bp, const float *sens, float floor, int
  * does not synchronise. */
 int psf_mlem(const psf_matrix *m, const float *y, float *x, float *sens, int32_t given,
              int32_t iters, float *yhat, float *ratio, float *bp, void *stream);
+
+/* List-mode OSEM (the next step the paper names in Sec. 5), every sub-iteration
+ * enqueued by one call, for a top-N plan after psf_matrix_build_sparse_adjoint.
+ * The events (rows: device int64 [n_events] set rows, others skipped) are split
+ * into n_subsets consecutive subsets; `iters` times over the subsets
+ *   x <- x * sum_{e in subset} A_e^T / (A_e x) / (sens / n_subsets)
+ * where sens >= 1e-12 max(sens), else 0 -- the MLEM update on the subset's counts
+ * weighted by n_subsets.  x (device float [n_cols]): the start image when have_x,
+ * else it starts from 1 on the voxels the scanner sees.  sens (device float
+ * [n_cols]).  Scratch: counts (device float [n_rows], cleared here), list (device
+ * int32 [n_rows]), bp (device float [n_cols]).  Work in proportion to the
+ * subset's events; PSF_EINVAL when a subset may have more events than the set has
+ * rows (use the separate steps).  Does not synchronise. */
+int psf_osem(const psf_matrix *m, const int64_t *rows, int64_t n_events, int32_t n_subsets,
+             int32_t iters, float *x, int32_t have_x, const float *sens, float *counts,
+             int32_t *list, float *bp, void *stream);
 
 /*
  * Kernel timing -- instrumentation of the library, no counterpart in the

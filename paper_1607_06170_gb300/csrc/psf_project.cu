@@ -67,6 +67,7 @@ struct psf_matrix {
     float *tr_w;
     int32_t *tr_list;
     unsigned long long *tr_nz;
+    unsigned *tr_bits;  // a bit per row (psf_osem), 0 between calls
     // stencil form 5 (plan-owned): the LOR-space input packed into padded
     // ring-pair planes, and the class spreads re-laid out as one contiguous
     // slice per (transaxial class, partner offset); wpad_dirty after
@@ -2480,6 +2481,108 @@ __global__ void ts_scatter_kernel(const int32_t *__restrict__ list, const unsign
     }
 }
 
+// List-mode sub-iterations on a top-N plan with the transpose of S (psf_osem):
+// everything but the image is touched only where the subset's events are, so a
+// sub-iteration costs by its events, not by the set (the separate steps make
+// about 25 passes over LOR-space vectors of the whole set).
+//   osem_count  events -> counts per LOR, and the LORs they hit (a LOR is listed
+//               by the event that finds its count 0)
+//   osem_mark   the sources of the listed LORs, one bit each
+//   osem_list   the marked rows, in row order within a block's 8,192 (rows of one
+//               transaxial pair stay together), their q cleared, the bits too
+//   osem_ratio  per listed LOR: its projection from its sources, the ratio, and
+//               the ratio to its sources' q; its count is 0 again
+constexpr int OS_T = 256;
+
+__global__ void __launch_bounds__(OS_T) osem_count_kernel(
+    const int64_t *__restrict__ rows, int64_t n_events, int64_t n_rows, float weight,
+    float *__restrict__ counts, int32_t *__restrict__ list, unsigned long long *n_list) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (int64_t)blockIdx.x * OS_T + (threadIdx.x & ~31); b < n_events;
+         b += (int64_t)gridDim.x * OS_T) {
+        const int64_t i = b + lane, r = i < n_events ? rows[i] : -1;
+        const bool first = r >= 0 && r < n_rows && atomicAdd(counts + r, weight) == 0.0f;
+        const unsigned m = __ballot_sync(0xffffffffu, first);
+        unsigned long long at = 0;
+        if (lane == 0 && m) at = atomicAdd(n_list, (unsigned long long)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (first) list[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)r;
+    }
+}
+
+__global__ void __launch_bounds__(OS_T) osem_mark_kernel(const int32_t *__restrict__ list,
+                                                         const unsigned long long *n_list,
+                                                         const int64_t *__restrict__ ptr,
+                                                         const int32_t *__restrict__ src,
+                                                         unsigned *__restrict__ bits) {
+    const int64_t n = (int64_t)*n_list;
+    for (int64_t i = (int64_t)blockIdx.x * OS_T + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * OS_T) {
+        const int32_t m = list[i];
+        for (int64_t e = ptr[m], e1 = ptr[m + 1]; e < e1; ++e) {
+            const int32_t s = src[e];
+            atomicOr(bits + (s >> 5), 1u << (s & 31));
+        }
+    }
+}
+
+__global__ void __launch_bounds__(OS_T) osem_list_kernel(unsigned *__restrict__ bits,
+                                                         int64_t n_rows, float *__restrict__ q,
+                                                         int32_t *__restrict__ list,
+                                                         unsigned long long *n_list) {
+    __shared__ int warp_sum[OS_T / 32];
+    __shared__ unsigned long long base;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t nw = (n_rows + 31) / 32;
+    for (int64_t w0 = (int64_t)blockIdx.x * OS_T; w0 < nw; w0 += (int64_t)gridDim.x * OS_T) {
+        const int64_t w = w0 + t;
+        unsigned b = w < nw ? bits[w] : 0u;
+        if (b) bits[w] = 0u;
+        int incl = __popc(b);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        int before = 0, total = 0;
+        for (int k = 0; k < OS_T / 32; ++k) {
+            before += k < warp ? warp_sum[k] : 0;
+            total += warp_sum[k];
+        }
+        if (t == 0 && total) base = atomicAdd(n_list, (unsigned long long)total);
+        __syncthreads();
+        if (b) {
+            unsigned long long at = base + before + incl - __popc(b);
+            while (b) {
+                const int64_t r = 32 * w + (__ffs(b) - 1);
+                b &= b - 1;
+                list[at++] = (int32_t)r;
+                q[r] = 0.0f;
+            }
+        }
+        __syncthreads();  // warp_sum and base are rewritten
+    }
+}
+
+__global__ void __launch_bounds__(OS_T) osem_ratio_kernel(
+    const int32_t *__restrict__ list, const unsigned long long *n_list,
+    const int64_t *__restrict__ ptr, const int32_t *__restrict__ src, const float *__restrict__ w,
+    const float *__restrict__ p, float *__restrict__ counts, float *__restrict__ q) {
+    const int64_t n = (int64_t)*n_list;
+    for (int64_t i = (int64_t)blockIdx.x * OS_T + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * OS_T) {
+        const int32_t m = list[i];
+        const int64_t e0 = ptr[m], e1 = ptr[m + 1];
+        float yhat = 0.0f;
+        for (int64_t e = e0; e < e1; ++e) yhat = fmaf(w[e], p[src[e]], yhat);
+        const float ratio = yhat > 0.0f ? counts[m] / yhat : 0.0f;
+        counts[m] = 0.0f;
+        if (ratio != 0.0f)
+            for (int64_t e = e0; e < e1; ++e) atomicAdd(q + src[e], w[e] * ratio);
+    }
+}
+
 static int topn_s(const psf_matrix *m, const float *in, float *out, bool adjoint,
                   cudaStream_t st) {
     const size_t shm = sizeof(char4) * (size_t)m->E * m->E + sizeof(int32_t) * (m->ls.Nt + m->ls.NR + 2) +
@@ -3120,6 +3223,8 @@ static void drop_transpose(psf_matrix *m) {
     cudaFree(m->tr_src);
     cudaFree(m->tr_w);
     cudaFree(m->tr_list);
+    cudaFree(m->tr_bits);
+    m->tr_bits = nullptr;
     m->tr_ptr = nullptr;
     m->tr_src = nullptr;
     m->tr_w = nullptr;
@@ -3247,6 +3352,8 @@ extern "C" int psf_matrix_build_sparse_adjoint(psf_matrix *m, void *stream) {
     const int grid = (int)(need < (int64_t)sms * 8 ? need : (int64_t)sms * 8);
     int64_t *ptr = nullptr, *tiles = nullptr;
     int32_t *cur = nullptr, *src = nullptr, *list = nullptr;
+    unsigned *bits = nullptr;
+    const size_t bit_bytes = sizeof(unsigned) * ((n + 31) / 32);
     float *w = nullptr;
     int rc = PSF_OK;
     auto fail = [&](int code) {
@@ -3256,14 +3363,18 @@ extern "C" int psf_matrix_build_sparse_adjoint(psf_matrix *m, void *stream) {
         cudaFree(src);
         cudaFree(w);
         cudaFree(list);
+        cudaFree(bits);
         return code;
     };
     if (cudaMalloc(&ptr, sizeof(int64_t) * (n + 1)) != cudaSuccess ||
         cudaMalloc(&tiles, sizeof(int64_t) * scan_tile_count(n)) != cudaSuccess ||
         cudaMalloc(&cur, sizeof(int32_t) * n) != cudaSuccess ||
-        cudaMalloc(&list, sizeof(int32_t) * n + 2 * sizeof(unsigned long long)) != cudaSuccess)
+        cudaMalloc(&list, sizeof(int32_t) * (n + (n & 1)) + 2 * sizeof(unsigned long long)) !=
+            cudaSuccess ||
+        cudaMalloc(&bits, bit_bytes) != cudaSuccess)
         return fail(PSF_ECUDA);
     if (cudaMemsetAsync(ptr, 0, sizeof(int64_t) * (n + 1), st) != cudaSuccess ||
+        cudaMemsetAsync(bits, 0, bit_bytes, st) != cudaSuccess ||
         cudaMemsetAsync(cur, 0, sizeof(int32_t) * n, st) != cudaSuccess ||
         cudaFuncSetAttribute(topn_s_kernel<TS_COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)shm) != cudaSuccess ||
@@ -3306,6 +3417,7 @@ extern "C" int psf_matrix_build_sparse_adjoint(psf_matrix *m, void *stream) {
     m->tr_src = src;
     m->tr_w = w;
     m->tr_list = list;
+    m->tr_bits = bits;
     m->tr_nz = reinterpret_cast<unsigned long long *>(list + n + (n & 1));
     return PSF_OK;
 }
@@ -3323,6 +3435,7 @@ extern "C" int psf_matrix_destroy(psf_matrix *m) {
     cudaFree(m->tr_src);
     cudaFree(m->tr_w);
     cudaFree(m->tr_list);  // the nonzero count shares this allocation
+    cudaFree(m->tr_bits);
     cudaFree(m->pin);
     cudaFree(m->wpad);
     delete m;
@@ -3935,4 +4048,109 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
         if (!rc) rc = update(false, bp, fused && it + 1 < iters);
     }
     return rc;
+}
+
+// List-mode OSEM on a top-N plan with the transpose of S.
+extern "C" int psf_osem(const psf_matrix *m, const int64_t *rows, int64_t n_events,
+                        int32_t n_subsets, int32_t iters, float *x, int32_t have_x,
+                        const float *sens, float *counts, int32_t *list, float *bp,
+                        void *stream) {
+    PSF_RANGE("psf_osem");
+    if (!m || !x || !sens || !bp || n_events < 0 || n_subsets < 1 || iters < 0) return PSF_EINVAL;
+    if (m->topn <= 0 || !m->tr_ptr || !counts || !list || (n_events > 0 && !rows))
+        return PSF_EINVAL;
+    const int64_t n = m->n_rows, nv = m->n_cols;
+    if (n_events / n_subsets + 1 > n) return PSF_EINVAL;  // the list of hit LORs
+    cudaStream_t st = as_stream(stream);
+    int dev = 0, sms = 148;
+    PSF_TRY(cudaGetDevice(&dev));
+    PSF_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    unsigned *key = reinterpret_cast<unsigned *>(m->queue + 4);
+    unsigned long long *n_hit = m->tr_nz, *n_src = m->tr_nz + 1;
+    const int vgrid = grid_for(nv, PJ_T);
+    PSF_TRY(cudaMemsetAsync(key, 0, sizeof(unsigned), st));
+    PSF_TRY(cudaMemsetAsync(counts, 0, sizeof(float) * n, st));
+    PSF_TRY(cudaMemsetAsync(bp, 0, sizeof(float) * nv, st));
+    {
+        PSF_TIMED("mlem_sens_kernel", st);
+        mlem_sens_kernel<<<vgrid, PJ_T, 0, st>>>(nullptr, const_cast<float *>(sens), bp, nv, key);
+    }
+    PSF_LAUNCHED();
+    if (!have_x) {  // 1 on the voxels the scanner sees
+        PSF_TIMED("mlem_update_kernel", st);
+        mlem_update_kernel<true><<<vgrid, PJ_T, 0, st>>>(x, sens, bp, sens, key, nv, false);
+    }
+    PSF_LAUNCHED();
+    for (int it = 0; it < iters; ++it)
+        for (int j = 0; j < n_subsets; ++j) {
+            const int64_t e0 = n_events * j / n_subsets, e1 = n_events * (j + 1) / n_subsets;
+            PSF_TRY(cudaMemsetAsync(n_hit, 0, 2 * sizeof(unsigned long long), st));
+            if (e1 > e0) {
+                {
+                    PSF_TIMED("osem_count_kernel", st);
+                    osem_count_kernel<<<grid_for(e1 - e0, OS_T), OS_T, 0, st>>>(
+                        rows + e0, e1 - e0, n, (float)n_subsets, counts, m->tr_list, n_hit);
+                }
+                PSF_LAUNCHED();
+                {
+                    PSF_TIMED("osem_mark_kernel", st);
+                    osem_mark_kernel<<<grid_for(e1 - e0, OS_T), OS_T, 0, st>>>(
+                        m->tr_list, n_hit, m->tr_ptr, m->tr_src, m->tr_bits);
+                }
+                PSF_LAUNCHED();
+                {
+                    PSF_TIMED("osem_list_kernel", st);
+                    osem_list_kernel<<<grid_for((n + 31) / 32, OS_T), OS_T, 0, st>>>(
+                        m->tr_bits, n, m->q, list, n_src);
+                }
+                PSF_LAUNCHED();
+                int rc;
+                if (m->otf) {
+                    rc = otf_rows_fwd(m->otf_sc, m->otf_im, m->otf_ls, list, n_src, x, m->p,
+                                      m->status, st);
+                } else {
+                    rc = dispatch_dtype(m->dtype, [&](auto tag) -> int {
+                        using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
+                        {
+                            PSF_TIMED("csr_fwd_list_kernel", st);
+                            csr_fwd_list_kernel<VT><<<sms * 8, PJ_T, 0, st>>>(
+                                list, n_src, m->row_ptr, m->col, (const VT *)m->val, m->row_scale,
+                                x, m->p);
+                        }
+                        PSF_LAUNCHED();
+                        return PSF_OK;
+                    });
+                }
+                if (rc) return rc;
+                {
+                    PSF_TIMED("osem_ratio_kernel", st);
+                    osem_ratio_kernel<<<grid_for(e1 - e0, OS_T), OS_T, 0, st>>>(
+                        m->tr_list, n_hit, m->tr_ptr, m->tr_src, m->tr_w, m->p, counts, m->q);
+                }
+                PSF_LAUNCHED();
+                if (m->otf) {
+                    rc = otf_rows_back(m->otf_sc, m->otf_im, m->otf_ls, list, n_src, m->q, bp,
+                                       m->status, st);
+                } else {
+                    rc = dispatch_dtype(m->dtype, [&](auto tag) -> int {
+                        using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
+                        {
+                            PSF_TIMED("csr_back_list_kernel", st);
+                            csr_back_list_kernel<VT><<<sms * 8, PJ_T, 0, st>>>(
+                                list, n_src, 4 * n, m->row_ptr, m->col, (const VT *)m->val,
+                                m->row_scale, m->q, bp);
+                        }
+                        PSF_LAUNCHED();
+                        return PSF_OK;
+                    });
+                }
+                if (rc) return rc;
+            }
+            {
+                PSF_TIMED("mlem_update_kernel", st);
+                mlem_update_kernel<false><<<vgrid, PJ_T, 0, st>>>(x, bp, bp, sens, key, nv, true);
+            }
+            PSF_LAUNCHED();
+        }
+    return PSF_OK;
 }

@@ -34,7 +34,7 @@ FUNCTIONS = [
     "psf_matrix_check", "psf_matrix_build_sparse_adjoint", "psf_bin_spread_classes",
     "psf_set_wait_limit", "psf_matrix_create_otf", "psf_matrix_set_image",
     "psf_spread_topn_bf16", "psf_matrix_set_spread_topn_bf16", "psf_psf_rows_workspace",
-    "psf_psf_rows_merge", "psf_psf_rows_emit", "psf_mlem",
+    "psf_psf_rows_merge", "psf_psf_rows_emit", "psf_mlem", "psf_osem",
 ]
 
 
@@ -115,6 +115,7 @@ _SIGS = {
     "psf_psf_rows_workspace": (C.c_int, [_P, _P, _I64, _I32, _I32, _P]),
     "psf_psf_rows_merge": (C.c_int, [_P, _P, _P, _I64, _P, _I32, _I32, _P, _P, _I64, _P, _P]),
     "psf_mlem": (C.c_int, [_P, _P, _P, _P, _I32, _I32, _P, _P, _P, _P]),
+    "psf_osem": (C.c_int, [_P, _P, _I64, _I32, _I32, _P, _I32, _P, _P, _P, _P, _P]),
     "psf_psf_rows_emit": (C.c_int, [_P, _P, _I64, _I32, _P, _P, _P, _P, _P, _P]),
 }
 
@@ -598,6 +599,20 @@ class Matrix:
         yhat, ratio, bp = new(self.n_rows), new(self.n_rows), new(self.n_cols)
         _ok(lib().psf_mlem(self._h, _ptr(y), _ptr(x), _ptr(sens), given, int(iters), _ptr(yhat),
                            _ptr(ratio), _ptr(bp), _stream()), "psf_mlem")
+        return x
+
+    def osem(self, rows, n_subsets: int, iters: int, sens, x=None):
+        """`iters` list-mode OSEM iterations in one call (psf_osem): x, the start
+        image, is updated in place and returned (None: from the voxels the
+        scanner sees)."""
+        have_x = x is not None
+        new = lambda n, d=torch.float32: torch.empty(n, dtype=d, device=rows.device)
+        x = x if have_x else new(self.n_cols)
+        # kept until the call returns: scratch of the enqueued sub-iterations
+        counts, lst, bp = new(self.n_rows), new(self.n_rows, torch.int32), new(self.n_cols)
+        _ok(lib().psf_osem(self._h, _ptr(rows), rows.numel(), int(n_subsets), int(iters), _ptr(x),
+                           int(have_x), _ptr(sens), _ptr(counts), _ptr(lst), _ptr(bp),
+                           _stream()), "psf_osem")
         return x
 
     def __del__(self):

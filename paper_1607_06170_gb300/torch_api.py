@@ -98,12 +98,16 @@ def listmode_osem(matrix, rows, n_subsets: int, iters: int = 1, x0=None, sens=No
     subset's events hit --, psf_em_ratio, psf_back, psf_em_update).
     Voxels with sens < 1e-12 * max(sens) are held at zero.  With top-N spreads
     and sparse_adjoint, the plan's transpose of S is built once so that S^T of
-    a subset's counts and ratios scatters from their nonzero entries."""
+    a subset's counts and ratios scatters from their nonzero entries; subsets of
+    at most a sixteenth of the rows then go through psf_osem, which touches
+    LOR-space data only where the events are."""
     n_ev = rows.numel()
     if sparse_adjoint and matrix.topn > 0:
         matrix.build_sparse_adjoint()
     if sens is None:
         sens = matrix.sensitivity(device=rows.device)
+    if sparse_adjoint and matrix.topn > 0 and n_ev // n_subsets + 1 <= matrix.n_rows // 16:
+        return matrix.osem(rows, n_subsets, iters, sens, None if x0 is None else x0.clone())
     floor = 1e-12 * float(sens.max())
     if x0 is None:
         x = torch.ones_like(sens)

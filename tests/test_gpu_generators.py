@@ -223,3 +223,42 @@ def test_pair_streamed_projections(P, ring3d, dtype, case):
     for g, o in zip(got, want):
         # sums of the same positive products in another order: up to ~2e4 per voxel
         assert_close(g.cpu(), o.cpu(), 2e-5, 1e-6 * float(o.abs().max()), case)
+
+
+@pytest.mark.parametrize("plan", ["stored", "bf16 rows and weights", "traced"])
+@pytest.mark.parametrize("n_ev,n_sub", [(4000, 4), (37, 1), (3, 5)])
+def test_osem_by_events(P, ring3d, plan, n_ev, n_sub):
+    """List-mode OSEM through psf_osem against the separate steps (a plan without
+    the transpose of S): events outside the set, LORs hit several times, subsets
+    without events, a given start image."""
+    from paper_1607_06170_gb300.torch_api import listmode_osem
+
+    w, W, rows = ring3d
+    s, ls, im = w["scanner"], w["lors"], w["image"]
+    nv = im["nx"] * im["ny"] * im["nz"]
+    idx, wk = P.spread_topn(W, *w["window"], 5)
+    wk, wsc = P.spread_topn_bf16(wk) if plan.startswith("bf16") else (wk, None)
+
+    def make():
+        if plan == "traced":
+            M = P.Matrix.traced(s, im, ls)
+        else:
+            ptr, col, val, sc = rows["bf16" if plan.startswith("bf16") else "f32"]
+            M = P.Matrix(ptr, col, val, nv, row_scale=sc)
+        return M.set_spread_topn(s, ls, *w["window"], idx, wk, scale=wsc)
+
+    M, R = make(), make()
+    rng = np.random.default_rng(n_ev)
+    ev = rng.choice(rng.integers(0, M.n_rows, max(n_ev // 2, 1)), n_ev)
+    ev[::17] = -1
+    ev = torch.from_numpy(ev.astype(np.int64)).cuda()
+    x0 = torch.from_numpy(I.random_image(im, 7, 0.5, 1.5).reshape(-1)).cuda()
+    for start in (None, x0):
+        P.timing_enable(True)
+        got = listmode_osem(M, ev, n_sub, 2, x0=start)
+        ran = set(P.timing_read())
+        P.timing_enable(False)
+        assert "osem_ratio_kernel" in ran
+        want = listmode_osem(R, ev, n_sub, 2, x0=start, sparse_adjoint=False)
+        # products of up to eight sub-iterations of reordered FP32 sums
+        assert_close(got.cpu(), want.cpu(), 5e-5, 1e-6 * float(want.max()) + 1e-30, "OSEM image")
