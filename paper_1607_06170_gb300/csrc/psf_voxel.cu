@@ -14,16 +14,16 @@
 namespace psf {
 
 constexpr int VH_T = 256;
-constexpr int VH_P = 4;                 // pixels of a CTA (fewer for sets with many rows)
-constexpr int VH_MAX_ROWS = 16384;      // one pixel's column in shared memory
-constexpr int VH_COL_BYTES = 96 * 1024; // columns of a CTA's pixels
+constexpr int VH_P = 12;             // most pixels of a CTA
+constexpr int VH_MAX_ROWS = 16384;   // one pixel's column in shared memory
 
 struct VhGeom {
     int R, Nb, Pt;
     double radius, wt, pt, width;  // width: transaxial block width
-    double edge;                   // half the side of the ring polygon
+    double u_lo, u_hi;             // the side of the ring polygon in cells, off its ends
     double to_u, u0;               // face coordinate -> cell lattice: st * to_u + u0
     double Pp, iPp;                // cells per crystal pitch and its inverse
+    bool whole;                    // no gaps: crystal i spans whole cells [i Pt, i Pt + Pt)
 };
 
 // What one end of a line needs of the block whose face plane it crosses: the
@@ -31,7 +31,7 @@ struct VhGeom {
 // another block than the pixel before it, not per pixel.
 struct VhBlock {
     int b;           // -1: none yet
-    double idn, dt;  // 1 / (direction . normal), tangential direction component
+    double idn, du;  // 1 / (direction . normal), cells per unit of path along the face
     int ent, ent1;   // table entries of sub-position 0: this block, the next one
     int sgt;         // travel direction along the face
     float cratio;    // cos(alpha) / cos(beta)
@@ -44,7 +44,7 @@ struct VhBlock {
 template <bool STAGED>
 struct VhFrame {
     int R;
-    const double *cs, *pn, *pt;
+    const double *cs, *pn, *pu;
     double cx, cy;
     __device__ __forceinline__ void trig(int b, double &c, double &s) const {
         if (STAGED) {
@@ -60,22 +60,23 @@ struct VhFrame {
         trig(b, c, s);
         return cx * c + cy * s;
     }
-    __device__ __forceinline__ double tangential(int b) const {
-        if (STAGED) return pt[b];
+    // tangential coordinate in cells of the face lattice
+    __device__ __forceinline__ double cells(const VhGeom &g, int b) const {
+        if (STAGED) return pu[b];
         double c, s;
         trig(b, c, s);
-        return cy * c - cx * s;
+        return (cy * c - cx * s) * g.to_u + g.u0;
     }
 };
 
 template <bool STAGED>
-__device__ __forceinline__ void vh_block(const Scan &sc, const Tab &tb, const VhFrame<STAGED> &f,
-                                         int b, double dx, double dy, VhBlock &k) {
+__device__ __forceinline__ void vh_block(const VhGeom &g, const Scan &sc, const Tab &tb,
+                                         const VhFrame<STAGED> &f, int b, double dx, double dy, VhBlock &k) {
     double cb, sb;
     f.trig(b, cb, sb);
     k.b = b;
     k.idn = 1.0 / (dx * cb + dy * sb);
-    k.dt = dy * cb - dx * sb;
+    k.du = (dy * cb - dx * sb) * g.to_u;
     // the response's angles, as end_response forms them (no axial component)
     const float fx = (float)dx, fy = (float)dy;
     float fs, fc;
@@ -155,34 +156,42 @@ __device__ __forceinline__ VhHit vh_entry(const VhGeom &g, const Scan &sc, const
     h.n = 0;
     h.x0 = h.p0 = h.x1 = h.p1 = 0;
     h.w = 1.0f;
-    double st = 0.0;
+    double u = 0.0;
     auto hits = [&]() {  // within the side of block k.b, off its ends
         const double t = (g.radius - f.normal(k.b)) * k.idn;
-        st = f.tangential(k.b) + t * k.dt;
-        return k.idn > 0.0 && fabs(st) < g.edge * (1.0 - 1e-9);
+        u = f.cells(g, k.b) + t * k.du;
+        return k.idn > 0.0 && u > g.u_lo && u < g.u_hi;
     };
     if (!(inside && k.b >= 0 && hits())) {
         int b = STAGED && inside ? vh_guess(g, csf, f.pn, (float)dx, (float)dy) : -1;
-        if (b >= 0 && b != k.b) vh_block(sc, tb, f, b, dx, dy, k);
+        if (b >= 0 && b != k.b) vh_block(g, sc, tb, f, b, dx, dy, k);
         if (b < 0 || !hits()) {
             b = vh_exit(g, f, dx, dy);
             if (b < 0) return h;
-            if (b != k.b) vh_block(sc, tb, f, b, dx, dy, k);
+            if (b != k.b) vh_block(g, sc, tb, f, b, dx, dy, k);
             hits();
         }
     }
     // cells of the face lattice: crystal i spans cells [i Pp, i Pp + Pt)
-    const double u = st * g.to_u + g.u0, ur = rint(u);
-    const bool on = fabs(u - ur) < 1e-9;
+    const double ur = rint(u), off = u - ur;
+    const bool on = fabs(off) < 1e-9;
     h.w = on ? 0.5f : 1.0f;
 #pragma unroll 1
     for (int side = 0; side < (on ? 2 : 1); ++side) {
-        const double uu = on ? ur - 0.5 + side : u;
-        const int i = (int)floor(uu * g.iPp);
-        if (i < 0 || i >= g.Nb) continue;
-        const double cell = uu - i * g.Pp;
-        if (cell >= g.Pt) continue;  // in the gap after crystal i
-        const int p = (int)floor(cell);
+        int i, p;
+        if (g.whole) {  // the lattice cell below (or beside) the hit, in integers
+            const int cell = (int)ur - (on ? 1 - side : off < 0.0 ? 1 : 0);
+            if (cell < 0 || cell >= g.Nb * g.Pt) continue;
+            i = cell / g.Pt;
+            p = cell - i * g.Pt;
+        } else {
+            const double uu = on ? ur - 0.5 + side : u;
+            i = (int)floor(uu * g.iPp);
+            if (i < 0 || i >= g.Nb) continue;
+            const double cell = uu - i * g.Pp;
+            if (cell >= g.Pt) continue;  // in the gap after crystal i
+            p = (int)floor(cell);
+        }
         if (h.n == 0) {
             h.x0 = i;
             h.p0 = p;
@@ -232,9 +241,11 @@ __device__ __forceinline__ void vh_response(const Scan &sc, const Tab &tb,
 // sectors).  The FP64 work bounds it (2 lanes a clock on an SM): a line's
 // direction is one FP64 sine and cosine for its P pixels, its block's normal
 // component and angles are found once per block, the blocks' trigonometry and
-// the pixels' block coordinates once per CTA, which leaves about 12 FP64
-// operations per line end and pixel.  RING2D, 720 lines: 7.03 -> 0.47 ms
-// (a CTA per pixel that found all of this per line: 16 FP64 sines a line end).
+// the pixels' block coordinates (in cells of the face lattice) once per CTA,
+// which leaves 6 FP64 operations per line end and pixel.  RING2D, 720 lines:
+// 7.03 -> 0.37 ms (a CTA per pixel that found all of this per line: 16 FP64
+// sines a line end).  Neighbouring lines stay in a warp: they cross the same
+// blocks (lines k / 32 apart in a warp: 0.57 ms, 9 of 32 lanes at work).
 // split > 1 (few lines): split threads share a line, each with P / split pixels.
 template <int WT, bool STAGED>
 __global__ void __launch_bounds__(VH_T, WT <= 3 ? 3 : 2) voxel_homog_kernel(VhGeom g, Scan sc, Tab tb,
@@ -246,8 +257,8 @@ __global__ void __launch_bounds__(VH_T, WT <= 3 ? 3 : 2) voxel_homog_kernel(VhGe
     const int SR = STAGED ? g.R : 0;                     // blocks with tables
     double *cs = reinterpret_cast<double *>(vh_raw);     // [SR][2] block cosine, sine
     double *pn = cs + 2 * SR;                            // [P][SR] pixel . normal
-    double *ptan = pn + P * SR;                          // [P][SR] pixel . tangent
-    float2 *csf = reinterpret_cast<float2 *>(ptan + P * SR);  // [SR]
+    double *pu = pn + P * SR;                            // [P][SR] its cells along the face
+    float2 *csf = reinterpret_cast<float2 *>(pu + P * SR);  // [SR]
     float *vh_col = reinterpret_cast<float *>(csf + SR);      // [P][stride]
     int32_t *tp_start = reinterpret_cast<int32_t *>(vh_col + P * stride);
     int32_t *rp_start = tp_start + ls.Nt + 1;
@@ -288,7 +299,7 @@ __global__ void __launch_bounds__(VH_T, WT <= 3 ? 3 : 2) voxel_homog_kernel(VhGe
             double cx, cy;
             pixel(v0 + p, cx, cy);
             pn[j] = cx * cs[2 * b] + cy * cs[2 * b + 1];
-            ptan[j] = cy * cs[2 * b] - cx * cs[2 * b + 1];
+            pu[j] = (cy * cs[2 * b] - cx * cs[2 * b + 1]) * g.to_u + g.u0;
             if (!(pn[j] < g.radius)) inside[p] = 0;
         }
         __syncthreads();
@@ -302,7 +313,7 @@ __global__ void __launch_bounds__(VH_T, WT <= 3 ? 3 : 2) voxel_homog_kernel(VhGe
             const int pe = (part + 1) * per < np ? (part + 1) * per : np;
 #pragma unroll 1
             for (int p = part * per; p < pe; ++p) {
-                VhFrame<STAGED> f{g.R, cs, pn + p * SR, ptan + p * SR, 0.0, 0.0};
+                VhFrame<STAGED> f{g.R, cs, pn + p * SR, pu + p * SR, 0.0, 0.0};
                 if (!STAGED) pixel(v0 + p, f.cx, f.cy);
                 const bool in = inside[p];
                 const VhHit h1 = vh_entry(g, sc, tb, f, csf, in, cth, sth, k1b);
@@ -382,30 +393,45 @@ extern "C" int psf_voxel_homog(const psf_scanner *scanner, const psf_table_desc 
     g.wt = scanner->xtal_w_t;
     g.pt = scanner->xtal_w_t + scanner->gap_t;
     g.width = scanner->nt_block * scanner->xtal_w_t + (scanner->nt_block - 1) * scanner->gap_t;
-    g.edge = g.radius * tan(M_PI / g.R);
     g.to_u = g.Pt / g.wt;
     g.u0 = 0.5 * g.width / g.wt * g.Pt;
+    const double edge = g.radius * tan(M_PI / g.R) * (1.0 - 1e-9) * g.to_u;
+    g.u_lo = g.u0 - edge;
+    g.u_hi = g.u0 + edge;
     g.Pp = g.Pt * g.pt / g.wt;
     g.iPp = 1.0 / g.Pp;
+    g.whole = g.pt == g.wt;
     cudaStream_t st = as_stream(stream);
-    const int stride = (int)((ls.ntp + 31) / 32 * 32 + 8);  // the pixels' columns 8 banks apart
-    int P = VH_P;
-    while (P > 1 && sizeof(float) * P * stride > VH_COL_BYTES) P /= 2;
-    auto bytes = [&](int SR) {
-        return sizeof(double) * SR * (2 + 2 * P) + sizeof(float2) * SR + sizeof(float) * P * stride +
-               sizeof(int32_t) * (ls.Nt + ls.NR + 2 + P);
-    };
-    size_t shm = bytes(g.R);
-    const bool staged = shm <= 200 * 1024;
-    if (!staged) {  // thousands of blocks: no tables
-        P = 1;
-        shm = bytes(0);
-    }
-    const int split = k <= VH_T / 4 && P >= 4 ? 4 : k <= VH_T / 2 && P >= 2 ? 2 : 1;
-    const int64_t nvox = (int64_t)im.nx * im.ny;
     int dev = 0, sms = 148;
     PSF_TRY(cudaGetDevice(&dev));
     PSF_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t nvox = (int64_t)im.nx * im.ny;
+    const int stride = (int)((ls.ntp + 31) / 32 * 32 + 8);  // the pixels' columns 8 banks apart
+    auto bytes = [&](int P, int SR) {
+        return sizeof(double) * SR * (2 + 2 * P) + sizeof(float2) * SR + sizeof(float) * P * stride +
+               sizeof(int32_t) * (ls.Nt + ls.NR + 2 + P);
+    };
+    // Pixels of a CTA: a line costs an SM's FP64 pipe about 3 units and each of
+    // its pixels one, the SM's CTAs share the pipe, and whole waves of them run;
+    // the fewest units (RING2D: 9 pixels, one wave, 0.37 ms; 4 pixels, three
+    // waves, 0.47 ms).
+    int P = 0;
+    double best = 1e300;
+    for (int p = 1; p <= VH_P; ++p) {
+        const size_t b = bytes(p, g.R);
+        if (b > 200 * 1024) break;
+        const int per_sm = b <= 74 * 1024 ? 3 : b <= 112 * 1024 ? 2 : 1;
+        const int64_t groups = (nvox + p - 1) / p, at_once = (int64_t)sms * per_sm;
+        const double units = (double)((groups + at_once - 1) / at_once) * (3 + p) * per_sm;
+        if (units < best) {
+            best = units;
+            P = p;
+        }
+    }
+    const bool staged = P > 0;
+    if (!staged) P = 1;  // thousands of blocks: no tables
+    const size_t shm = bytes(P, staged ? g.R : 0);
+    const int split = k <= VH_T / 4 && P >= 4 ? 4 : k <= VH_T / 2 && P >= 2 ? 2 : 1;
     const int64_t groups = (nvox + P - 1) / P;
     const int grid = (int)(groups < (int64_t)sms * 16 ? groups : (int64_t)sms * 16);
     auto launch = [&](auto kernel) -> int {
