@@ -278,8 +278,7 @@ def kernel_model(name, s, t, ls, Wt, Wa, n_lors, n_cls, nnz, nv, vb=4):
         # column + value, row_ptr, two LOR values, image pair
         return "hbm", ent + 16.0 * n_lors + 8.0 * nv, "GB/s"
     if name == "spread_q_kernel":  # one FMA per sub-LOR and quadrant entry pair
-        # of the classes the kernel computes (one per orbit of the two reflections):
-        # the definition's work, of which the kernel's runs leave about an eighth
+        # of the classes the kernel computes (one per orbit of the two reflections)
         nsub = (t["n_sub_t"] * t["n_sub_a"]) ** 2
         return "alu", 2.0 * n_comp_classes(s, ls) * nsub * ((Wt + 1) * (Wa + 1)) ** 2, "TFLOP/s"
     if name.startswith("stencil"):  # one FMA per (output LOR, source LOR) pair

@@ -125,38 +125,13 @@ struct GapConst {
     const float *tanT, *tanB, *tanA;  // [Kt - 1], [Kt - 1], [Ka - 1] (shared memory)
 };
 
-// The tangents, from the host: FP64 tangents in every CTA (and t2 in every
-// thread) took a fifth of a planar ring's spreads (32 -> 24 us for 64 sub-LORs
-// each).  n = 0: more nodes than fit a kernel argument, found by the CTA.
-struct NodeTans {
-    float t2;
-    int n;
-    float t[256];
-};
-
-inline NodeTans make_nodetans(const Scan &sc, const Tab &tb) {
-    NodeTans k;
-    const double st = (double)tb.dt, sa = (double)tb.da, g = (double)sc.two_pi_R;
-    const double half_pi = 1.5707963267948966;
-    k.t2 = (float)tan(g);
-    k.n = 2 * (int64_t)tb.Kt + tb.Ka <= 256 ? 2 * tb.Kt + tb.Ka : 0;
-    for (int j = 0; j < k.n; ++j) {
-        const double b = j < tb.Kt       ? (j + 0.5) * st
-                         : j < 2 * tb.Kt ? (j - tb.Kt + 0.5) * st + g
-                                         : (j - 2 * tb.Kt + 0.5) * sa;
-        k.t[j] = b < half_pi ? (float)tan(b) : INFINITY;
-    }
-    return k;
-}
-
 // Tangent tables in shared memory (2 * Kt + Ka floats); call with every
 // thread of the CTA, then synchronise.
-__device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb, const NodeTans &nt,
-                                                  float *tabs) {
+__device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb, float *tabs) {
     GapConst k;
     k.c2 = cosf(sc.two_pi_R);
     k.s2 = sc.sin_two_pi_R;
-    k.t2 = nt.t2;
+    k.t2 = (float)tan((double)sc.two_pi_R);
     k.ipt = 1.0f / sc.pt;
     k.ipa = 1.0f / sc.pa;
     k.iwt = 1.0f / sc.wt;
@@ -165,8 +140,7 @@ __device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb,
     float *tT = tabs, *tB = tabs + tb.Kt, *tA = tabs + 2 * tb.Kt;
     const double st = (double)tb.dt, sa = (double)tb.da, g = (double)sc.two_pi_R;
     const double half_pi = 1.5707963267948966;
-    for (int j = threadIdx.x; j < nt.n; j += blockDim.x) tabs[j] = nt.t[j];
-    for (int j = threadIdx.x; j < 2 * tb.Kt + tb.Ka && !nt.n; j += blockDim.x) {
+    for (int j = threadIdx.x; j < 2 * tb.Kt + tb.Ka; j += blockDim.x) {
         double b;
         float* dst;
         if (j < tb.Kt) { b = (j + 0.5) * st; dst = tT + j; }
@@ -187,9 +161,7 @@ __device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb,
 __device__ __forceinline__ int node_by_tan(const float *tab, int K, float opp, float adj,
                                            int k0) {
     int k = k0 < 0 ? 0 : (k0 > K - 1 ? K - 1 : k0);
-#pragma unroll 1
     while (k < K - 1 && adj * tab[k] <= opp) ++k;
-#pragma unroll 1
     while (k > 0 && adj * tab[k - 1] > opp) --k;
     return k;
 }
@@ -206,156 +178,14 @@ __device__ __forceinline__ float atan_seed(float y, float x) {
     return above ? 1.57079633f - a : a;
 }
 
-// The response of end_response() in three parts with a compile-time window, so
-// that a caller does each of them as seldom as its inputs change: the side
-// (the transaxial direction: node, sub-position and gap crossing), the node
-// (the polar node, and where a gap crosser meets block1 axially) and the rows
-// (the table values, into a quadrant array that stays in registers: every
-// index is static after unrolling).  The trigonometry of the gap path comes
-// from the direction components (cos a = vn/h, tan theta = |dz|/h,
-// cos(a - 2pi/R) by the angle-difference formula), the nearest nodes from
-// tangent tables, and divisions by constants are products with reciprocals.
-// Same quantity: Sec. 2.1.1 table lookup for block0 and Sec. 2.1.2 Eq. 2, 4, 5
+// The response of end_response() with a compile-time window: the quadrant
+// array stays in registers (every index is static after unrolling), the
+// trigonometry of the gap path comes from the direction components
+// (cos a = vn/h, tan theta = |dz|/h, cos(a - 2pi/R) by the angle-difference
+// formula), the nearest nodes come from tangent tables and divisions by
+// constants are products with reciprocals.  The response is the same
+// quantity: Sec. 2.1.1 table lookup for block0 and Sec. 2.1.2 Eq. 2, 4, 5
 // for block1.
-struct QSide {
-    float ih, h, run;  // (end_gap_cell: run with the axial sign of travel)
-    int sgt, row0;   // travel sign; (kt * Ka) * Pt + iu: table rows of block0 are row0 + ka * Pt
-    int row1, m;     // the same for block1, and its first crystal reached
-    int edge;        // crystals of block0 beyond the entry one
-    bool gap;        // beta = alpha - 2 pi/R > 0: block1 through the corner gap
-};
-
-__device__ __forceinline__ QSide end_side(const Scan &sc, const Tab &tb, const GapConst &k, int i,
-                                          int p, float s_entry, float vn, float vt) {
-    QSide e;
-    e.sgt = vt >= 0.0f ? 1 : -1;
-    const float avt = fabsf(vt);
-    // (explicit products and sums: the nodes decided from them are the same
-    // bits wherever this is inlined)
-    const float h2 = fmaf(vn, vn, vt * vt);
-    e.ih = rsqrtf(h2);
-    e.h = h2 * e.ih;
-    const int iu = e.sgt > 0 ? p : tb.Pt - 1 - p;
-    // nearest nodes: count of node boundaries (j + 1/2) * step at or below
-    // the angle, seeded from the approximate angle
-    const float alpha = atan_seed(avt, vn);
-    const int kt = node_by_tan(k.tanT, tb.Kt, avt, vn, f2i_rd(fmaf(alpha, tb.inv_dt, 0.5f)));
-    e.row0 = kt * tb.Ka * tb.Pt + iu;
-    e.edge = e.sgt > 0 ? sc.Nb - 1 - i : i;
-    e.gap = avt > vn * k.t2;
-    e.run = 0.0f;
-    e.m = e.row1 = 0;
-    if (e.gap) {
-        const float nu = sc.half_w - e.sgt * s_entry;
-        const float ca = vn * e.ih, sa = avt * e.ih;
-        const float icb = 1.0f / fmaf(ca, k.c2, sa * k.s2);
-        const float AP1 = sc.sigma + ca * icb * (sc.sigma + nu);
-        const float qq = fmaxf(AP1 - sc.gt, 0.0f);
-        e.m = f2i_rd(qq * k.ipt);
-        const float f = qq - e.m * sc.pt;
-        const float u1 = f < sc.wt ? (sc.wt - f) * k.iwt : 0.0f;
-        const int iu1 = max(min(f2i_rd(u1 * tb.Pt), tb.Pt - 1), 0);
-        e.run = (sc.sigma + nu) * sc.sin_two_pi_R * icb;
-        const int kt1 = node_by_tan(k.tanB, tb.Kt, avt, vn,
-                                    f2i_rd(fmaf(alpha - sc.two_pi_R, tb.inv_dt, 0.5f)));
-        e.row1 = kt1 * tb.Ka * tb.Pt + iu1;
-    }
-    return e;
-}
-
-// Polar node of a photon that climbs adz over the side's transaxial run h, and
-// where its count starts.
-__device__ __forceinline__ int polar_seed(const Tab &tb, const QSide &e, float adz) {
-    return f2i_rd(fmaf(atan_seed(adz, e.h), tb.inv_da, 0.5f));
-}
-__device__ __forceinline__ int end_polar(const Tab &tb, const GapConst &k, const QSide &e, float adz) {
-    return node_by_tan(k.tanA, tb.Ka, adz, e.h, polar_seed(tb, e, adz));
-}
-
-// Crystal ring (high half, from the entry ring on; far ones at +-2^14) and axial
-// sub-position (low half) at which a gap crosser enters block1.  In the order of travel through block1's lattice, so
-// monotone in adz, like end_polar().
-__device__ __forceinline__ int end_gap_cell(const Scan &sc, const Tab &tb, const GapConst &k,
-                                            const QSide &e, float z_entry, float adz, int sga,
-                                            int ring) {
-    const float z1 = z_entry + e.run * (adz * e.ih);
-    const float zl = z1 - k.zbase;
-    int k1 = f2i_rd(zl * k.ipa);
-    const float fa = zl - k1 * sc.pa;
-    float v1;
-    if (fa <= sc.wa) {
-        v1 = sga > 0 ? fa * k.iwa : (sc.wa - fa) * k.iwa;
-    } else {
-        if (sga > 0) k1 += 1;
-        v1 = 0.0f;
-    }
-    const int iv1 = max(min(f2i_rd(v1 * tb.Pa), tb.Pa - 1), 0);
-    return (max(min(k1, ring + 16384), ring - 16384) - ring) * 65536 + iv1;
-}
-
-// The table values of a photon (polar node ka, axial sub-position iv in the
-// direction of travel, sga; gap crossers: cell of end_gap_cell()) added to the
-// quadrant array q and, in FP64, to the total es (null: not wanted).
-template <int WT, int WA>
-__device__ __forceinline__ void end_rows(const Scan &sc, const Tab &tb, const float *__restrict__ T,
-                                         const double *__restrict__ eta, const QSide &e, int ka,
-                                         int iv, int cell, int sga,
-                                         float (&q)[(WT + 1) * (WA + 1)], double *es) {
-    constexpr int W1 = WA + 1;
-    const int MM = tb.Mt * tb.Ma;
-    // table offsets fit 32 bits (the descriptor holds at most 2^28 values)
-    const int ent = (e.row0 + ka * tb.Pt) * tb.Pa + iv;
-    const float *Tb = T + ent * MM;
-    const int nx0 = min(e.edge, tb.Mt - 1);
-    if (WA % 2 == 1 && WA < tb.Ma && (tb.Ma & 1) == 0) {
-        // rows of an even length start 8-byte aligned: load z pairs
-#pragma unroll
-        for (int x = 0; x <= WT; ++x)
-            if (x <= nx0) {
-#pragma unroll
-                for (int z = 0; z <= WA; z += 2) {
-                    const float2 v = __ldg(reinterpret_cast<const float2 *>(Tb + x * tb.Ma + z));
-                    q[x * W1 + z] += v.x;
-                    q[x * W1 + z + 1] += v.y;
-                }
-            }
-    } else {
-        const int nz0 = tb.Ma - 1;
-#pragma unroll
-        for (int x = 0; x <= WT; ++x)
-#pragma unroll
-            for (int z = 0; z <= WA; ++z)
-                if (x <= nx0 && z <= nz0) q[x * W1 + z] += ldg(Tb + x * tb.Ma + z);
-    }
-    double t = 0.0;
-    if (es) t = ldg(eta + ent * (tb.Mt + 1) + min(e.edge + 1, tb.Mt));
-    if (e.gap && (es || e.edge < WT)) {
-        const int ent1 = (e.row1 + ka * tb.Pt) * tb.Pa + (cell & 65535);
-        const float *T1 = T + ent1 * MM;
-        if (es) {
-            const double *E1 = eta + ent1 * (tb.Mt + 1);
-            t += ldg(E1 + min(e.m + 1 + sc.Nb, tb.Mt)) - ldg(E1 + min(e.m + 1, tb.Mt));
-        }
-        const int dzq0 = sga * (cell >> 16);
-        // block1 crystals enter the window only from an entry crystal within
-        // WT of the block edge (the same for every sub-LOR of the LOR)
-        if (e.edge < WT) {
-#pragma unroll
-            for (int X = 0; X <= WT; ++X) {
-                const int j = X - e.edge - 1, x = e.m + 1 + j;  // block1 crystal j, table column x
-                if (j < 0 || j >= sc.Nb || x >= tb.Mt) continue;
-#pragma unroll
-                for (int Z = 0; Z <= WA; ++Z) {
-                    const int z = Z - dzq0;
-                    if (z >= 0 && z < tb.Ma) q[X * W1 + Z] += ldg(T1 + x * tb.Ma + z);
-                }
-            }
-        }
-    }
-    if (es) *es += t;
-}
-
-// The response of one photon: all three parts.
 template <int WT, int WA>
 struct QResp {
     float q[(WT + 1) * (WA + 1)];
@@ -368,16 +198,96 @@ __device__ __forceinline__ void end_resp_q(const Scan &sc, const Tab &tb, const 
                                            const double *__restrict__ eta, int i, int ring,
                                            int p, int q, float s_entry, float z_entry, float vn,
                                            float vt, float dz, QResp<WT, WA> &r) {
+    constexpr int W1 = WA + 1;
+    const int sgt = vt >= 0.0f ? 1 : -1;
     const int sga = dz >= 0.0f ? 1 : -1;
 #pragma unroll
-    for (int j = 0; j < (WT + 1) * (WA + 1); ++j) r.q[j] = 0.0f;
-    r.eta = 0.0;
-    QSide e = end_side(sc, tb, k, i, p, s_entry, vn, vt);
-    e.run *= sga;
-    const float adz = fabsf(dz);
-    const int ka = end_polar(tb, k, e, adz);
-    const int cell = e.gap ? end_gap_cell(sc, tb, k, e, z_entry, adz, sga, ring) : 0;
-    end_rows<WT, WA>(sc, tb, T, eta, e, ka, sga > 0 ? q : tb.Pa - 1 - q, cell, sga, r.q, &r.eta);
+    for (int j = 0; j < (WT + 1) * W1; ++j) r.q[j] = 0.0f;
+    const float avt = fabsf(vt), adz = fabsf(dz);
+    const float h2 = vn * vn + vt * vt;
+    const float ih = rsqrtf(h2);
+    const float h = h2 * ih;
+    const int iu = sgt > 0 ? p : tb.Pt - 1 - p;
+    const int iv = sga > 0 ? q : tb.Pa - 1 - q;
+    // nearest nodes: count of node boundaries (j + 1/2) * step at or below
+    // the angle, seeded from the approximate angle
+    const float alpha = atan_seed(avt, vn);
+    const int kt = node_by_tan(k.tanT, tb.Kt, avt, vn, f2i_rd(fmaf(alpha, tb.inv_dt, 0.5f)));
+    const int ka = node_by_tan(k.tanA, tb.Ka, adz, h,
+                               f2i_rd(fmaf(atan_seed(adz, h), tb.inv_da, 0.5f)));
+    const int MM = tb.Mt * tb.Ma;
+    // table offsets fit 32 bits (the descriptor holds at most 2^28 values)
+    const int ent = ((kt * tb.Ka + ka) * tb.Pt + iu) * tb.Pa + iv;
+    const float *Tb = T + ent * MM;
+    const int edge = sgt > 0 ? sc.Nb - 1 - i : i;  // crystals of block0 beyond the entry one
+    const int nx0 = min(edge, tb.Mt - 1);
+    if (WA % 2 == 1 && WA < tb.Ma && (tb.Ma & 1) == 0) {
+        // rows of an even length start 8-byte aligned: load z pairs
+#pragma unroll
+        for (int x = 0; x <= WT; ++x)
+            if (x <= nx0) {
+#pragma unroll
+                for (int z = 0; z <= WA; z += 2) {
+                    const float2 v = __ldg(reinterpret_cast<const float2 *>(Tb + x * tb.Ma + z));
+                    r.q[x * W1 + z] = v.x;
+                    r.q[x * W1 + z + 1] = v.y;
+                }
+            }
+    } else {
+        const int nz0 = tb.Ma - 1;
+#pragma unroll
+        for (int x = 0; x <= WT; ++x)
+#pragma unroll
+            for (int z = 0; z <= WA; ++z)
+                if (x <= nx0 && z <= nz0) r.q[x * W1 + z] = ldg(Tb + x * tb.Ma + z);
+    }
+    double e = ldg(eta + ent * (tb.Mt + 1) + min(edge + 1, tb.Mt));
+    if (avt > vn * k.t2) {  // beta = alpha - 2 pi/R > 0: block1 through the corner gap
+        const float nu = sc.half_w - sgt * s_entry;
+        const float ca = vn * ih, sa = avt * ih;
+        const float icb = 1.0f / (ca * k.c2 + sa * k.s2);
+        const float AP1 = sc.sigma + ca * icb * (sc.sigma + nu);
+        const float qq = fmaxf(AP1 - sc.gt, 0.0f);
+        const int m = f2i_rd(qq * k.ipt);
+        const float f = qq - m * sc.pt;
+        const float u1 = f < sc.wt ? (sc.wt - f) * k.iwt : 0.0f;
+        const int iu1 = max(min(f2i_rd(u1 * tb.Pt), tb.Pt - 1), 0);
+        const float run = (sc.sigma + nu) * sc.sin_two_pi_R * icb;
+        const float z1 = z_entry + sga * run * (adz * ih);
+        const float zl = z1 - k.zbase;
+        int k1 = f2i_rd(zl * k.ipa);
+        const float fa = zl - k1 * sc.pa;
+        float v1;
+        if (fa <= sc.wa) {
+            v1 = sga > 0 ? fa * k.iwa : (sc.wa - fa) * k.iwa;
+        } else {
+            if (sga > 0) k1 += 1;
+            v1 = 0.0f;
+        }
+        const int iv1 = max(min(f2i_rd(v1 * tb.Pa), tb.Pa - 1), 0);
+        const int kt1 = node_by_tan(k.tanB, tb.Kt, avt, vn,
+                                    f2i_rd(fmaf(alpha - sc.two_pi_R, tb.inv_dt, 0.5f)));
+        const int ent1 = ((kt1 * tb.Ka + ka) * tb.Pt + iu1) * tb.Pa + iv1;
+        const float *T1 = T + ent1 * MM;
+        const double *E1 = eta + ent1 * (tb.Mt + 1);
+        e += ldg(E1 + min(m + 1 + sc.Nb, tb.Mt)) - ldg(E1 + min(m + 1, tb.Mt));
+        const int dzq0 = sga * (k1 - ring);
+        // block1 crystals enter the window only from an entry crystal within
+        // WT of the block edge (the same for every sub-LOR of the LOR)
+        if (edge < WT) {
+#pragma unroll
+            for (int X = 0; X <= WT; ++X) {
+                const int j = X - edge - 1, x = m + 1 + j;  // block1 crystal j, table column x
+                if (j < 0 || j >= sc.Nb || x >= tb.Mt) continue;
+#pragma unroll
+                for (int Z = 0; Z <= WA; ++Z) {
+                    const int z = Z - dzq0;
+                    if (z >= 0 && z < tb.Ma) r.q[X * W1 + Z] += ldg(T1 + x * tb.Ma + z);
+                }
+            }
+        }
+    }
+    r.eta = e;
 }
 
 }  // namespace psf

@@ -219,31 +219,26 @@ static size_t spread_smem(const Tab &tb, int Wt, int Wa) {
 }
 
 
-// K3 for the common windows (3 crystals to a side, axially 0, 2 or 3).  A LOR's sub-LORs are not
-// evaluated one by one: the transaxial half of a response depends on the
-// transaxial sub-positions (p1, p2) alone, and for one such pair the axial half
-// (polar nodes, the cells that gap crossers meet) is a step function of the
-// axial ones (q1, q2): seen from one q, two or three steps at most, as a rule,
-// over the other end's.  So each q's few different rows ("variants") are
-// evaluated once, and sum_{q1,q2} r1 (x) r2 is, over the runs of q2 in which
-// r1(q1) stays, r1 (x) (sum_q2 r2): about 25 table rows and 12 outer products a
-// pair for its Pa^2 sub-LORs (64).  A warp takes a 4 x 4 tile of pairs: first a
-// lane the transaxial side of a pair's end, then, a few pairs at a time, a lane an
-// end's q: the steps, its variants into shared memory, the runs' sums (two lanes to a
-// q1), and the outer products with 16 lanes owning RB x CB blocks of the Q x Q
-// quadrant product.  Pairs with different signs of travel land in different
-// quadrants of the window: a pass for each pattern of signs.  Sums have a fixed
-// order (FP32, deterministic); the totals that normalise them are FP64.  Bound
-// by issue; warps are at different places of the code, which therefore has one
-// copy of each part (with the sums of pairs without steps formed apart, 150 KB
-// of code: 10 of 16 cycles of a warp went by without an instruction).  RING3D's
-// 21,744 orbit classes x 4096 sub-LORs: 4.65 -> 3.2 ms (a sub-LOR per lane,
-// 4096 outer products a LOR).
-constexpr int SQ_T = 128;
-constexpr int SQ_WARPS = SQ_T / 32;
-constexpr int SQ_V = 3;  // most variants of a row that are staged (more: fewer q at a time)
-constexpr int SQ_R = 16 * SQ_V;  // most sums of a batch: 16 lanes' runs
-constexpr int SQ_S = 7;   // words of a staged side
+// K3 with a compile-time window (the common windows).  A warp evaluates 32
+// sub-LORs at a time, one per lane, into warp-private rows of shared memory,
+// then accumulates their outer products r1 (x) r2: each half-warp takes every
+// other staged sub-LOR, its 16 lanes owning fixed RB x CB blocks of the Q x Q
+// quadrant-local product (two shared-memory reads per 16 FMA).  Sub-LORs with
+// different travel patterns land in different quadrants of the window, so
+// each pattern present in the LOR gets its own register accumulator ("slot");
+// a pre-pass finds the patterns present and a LOR with more than SQ_SLOTS
+// patterns is done in several passes, each evaluating the responses of only
+// its patterns' sub-LORs.  The per-warp accumulators are summed in a fixed
+// order at the end of each pass (FP32, deterministic), folded into the window,
+// and normalised with FP64 totals.  One slot (a pass per pattern) leaves the
+// registers for three CTAs per SM, which hides more latency than the extra
+// passes over the sub-LOR directions cost (22.1 ms against 24.2 ms with four
+// slots at two CTAs per SM, 3D ring classes).
+constexpr int SQ_SLOTS = 1;
+constexpr int SQ_WARPS = SP_THREADS / 32;
+constexpr int SQ_TA_LOG = 3, SQ_TB_LOG = 2;  // sub-LOR tile of a warp: 8 x 4
+constexpr int SQ_TA = 1 << SQ_TA_LOG, SQ_TB = 1 << SQ_TB_LOG;
+static_assert(SQ_TA * SQ_TB == 32, "one sub-LOR per lane");
 
 template <int WT, int WA>
 struct SqShape {
@@ -254,12 +249,16 @@ struct SqShape {
     // alternate staged sub-LORs and are summed at the end of a pass
     static constexpr int RB = (Q + 3) / 4;
     static constexpr int CB = (Q + 3) / 4;
-    // floats from one staged row to the next: 16-byte parts, an odd number of
-    // them, so that eight lanes storing a part each hit distinct banks
-    static constexpr int QS = RB % 2 ? 4 * RB : 4 * RB + 4;
+    // row stride of the staged responses: covers every lane's reads, 16-byte
+    // rows, and an odd number of 16-byte units so 8 lanes storing 16 bytes
+    // each hit distinct banks; then rows r and r + 4 (the two halves' rows at
+    // one step) lie 16 banks apart
+    static constexpr int QR = 4 * RB;
+    static constexpr int QS = ((QR + 3) / 4) % 2 == 0 ? ((QR + 3) / 4) * 4 + 4 : ((QR + 3) / 4) * 4;
+    static_assert((4 * QS) % 32 == 16 || QR <= 8, "halves' rows 16 banks apart");
 };
 
-// A lane's operands of a staged row.
+// One staged sub-LOR's operands of a lane: RB entries of r1, CB of r2.
 template <int N>
 __device__ __forceinline__ void load_n(const float *p, float (&v)[N]) {
     if constexpr (N == 4) {
@@ -268,394 +267,269 @@ __device__ __forceinline__ void load_n(const float *p, float (&v)[N]) {
         v[1] = w.y;
         v[2] = w.z;
         v[3] = w.w;
+    } else if constexpr (N == 2) {
+        const float2 w = *reinterpret_cast<const float2 *>(p);
+        v[0] = w.x;
+        v[1] = w.y;
     } else {
 #pragma unroll
         for (int i = 0; i < N; ++i) v[i] = p[i];
     }
 }
 
-// n rows of R2, with the rows of R1 that `at` names (in floats), into the
-// accumulator: each half-warp takes every other one.
-template <class S>
-__device__ __forceinline__ void acc_rows(float (&acc)[S::RB][S::CB], const float *R1, const int *at,
-                                         const float *R2, int n, int h, int rb, int cb) {
-    R1 += rb * S::RB;
-    R2 += h * S::QS + cb * S::CB;
-#pragma unroll 2
-    for (int row = h; row < n; row += 2) {
-        float a[S::RB], b[S::CB];
-        load_n<S::RB>(R1 + at[row], a);
-        load_n<S::CB>(R2, b);
-        R2 += 2 * S::QS;
+template <int RB, int CB>
+__device__ __forceinline__ void load_ab(const float *ra, const float *rbp, float (&a)[RB],
+                                        float (&b)[CB]) {
+    load_n<RB>(ra, a);
+    load_n<CB>(rbp, b);
+}
+
+// Staged row of a half-warp at step k (0..15): the halves take rows r and
+// r + 4 of each group of eight.
+__device__ __forceinline__ int half_row(int k, int h) { return ((k >> 2) << 3) + (k & 3) + (h << 2); }
+
+// All 32 staged sub-LORs of a warp into one accumulator (same slot): each
+// half-warp takes 16 of them.
+template <int RB, int CB, int QS>
+__device__ __forceinline__ void acc_all32(float (&acc)[RB][CB], const float *ra,
+                                          const float *rbp, int h) {
+#pragma unroll 8
+    for (int k = 0; k < 16; ++k) {
+        float a[RB], b[CB];
+        const int row = half_row(k, h);
+        load_ab<RB, CB>(ra + row * QS, rbp + row * QS, a, b);
 #pragma unroll
-        for (int i = 0; i < S::RB; ++i)
+        for (int i = 0; i < RB; ++i)
 #pragma unroll
-            for (int j = 0; j < S::CB; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int j = 0; j < CB; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
 }
 
-// A lane's half of a run's sum into its place.
-template <class S, int PH>
-__device__ __forceinline__ void put_sum(float *R, int half, const float4 (&sum)[PH]) {
+// A response into its staging row (16-byte aligned when Q is a multiple of 4).
+template <int Q>
+__device__ __forceinline__ void stage_row(float *dst, const float (&q)[Q]) {
+    if constexpr (Q % 4 == 0) {
 #pragma unroll
-    for (int k = 0; k < PH; ++k)
-        if (half * PH + k < S::Q / 4) reinterpret_cast<float4 *>(R)[half * PH + k] = sum[k];
-}
-
-// Shared words of a warp, in order: variant rows [SQ_V][32][QS], sums
-// [SQ_R][QS], variants' totals [SQ_V][32] (FP64), sides [SQ_S][32], steps [32],
-// sums' r1 [SQ_R], pairs [16].
-template <class S>
-__host__ __device__ constexpr int spread_q_words() {
-    return (SQ_V * 32 + SQ_R) * S::QS + 2 * SQ_V * 32 + SQ_S * 32 + 32 + SQ_R + 16;
+        for (int k = 0; k < Q; k += 4)
+            *reinterpret_cast<float4 *>(dst + k) = make_float4(q[k], q[k + 1], q[k + 2], q[k + 3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) dst[k] = q[k];
+    }
 }
 
 template <int WT, int WA>
 static size_t spread_q_smem(const Tab &tb) {
     using S = SqShape<WT, WA>;
-    size_t b = sizeof(float) * SQ_WARPS * spread_q_words<S>();
-    b += sizeof(double) * 2 * SQ_WARPS;            // FP64 partial totals
-    b += sizeof(float) * 2 * (4 * tb.Pt + tb.Pa);  // sub-position centres
-    b += sizeof(int) * 4;                          // sign masks, the LOR
-    b += sizeof(float) * (2 * tb.Kt + tb.Ka);      // node tangents
-    return b;
+    const int NP = tb.Pt * tb.Pa;
+    size_t b = sizeof(double) * 2 * SQ_WARPS;                       // FP64 partial totals
+    b += sizeof(int) * 20;                                           // pattern mask, slots
+    b += sizeof(float) * SQ_WARPS * 2 * 32 * S::QS;                  // staged responses
+    b += sizeof(float) * S::E * S::E;                                // window
+    b += sizeof(float) * 2 * NP * 4;                                 // sub-position centres
+    b += sizeof(float) * (2 * tb.Kt + tb.Ka);                        // node tangents
+    return b + 64;
 }
 
-// queue: the next LOR to take (null: strided)
 template <int WT, int WA>
-__global__ void __launch_bounds__(SQ_T, 4) spread_q_kernel(
-    Scan sc, Tab tb, const __grid_constant__ NodeTans tans, const float *__restrict__ T,
-    const double *__restrict__ eta, const int32_t *__restrict__ lors, int64_t n_lors, int wt, int wa,
-    int norm, float *__restrict__ out, const int32_t *__restrict__ sym, unsigned *queue) {
+__global__ void __launch_bounds__(SP_THREADS, 3) spread_q_kernel(
+    Scan sc, Tab tb, const float *__restrict__ T, const double *__restrict__ eta,
+    const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
+    const int32_t *__restrict__ sym) {
     using S = SqShape<WT, WA>;
-    constexpr int Q = S::Q, RB = S::RB, CB = S::CB, QS = S::QS;
-    const int W2a = 2 * wa + 1, E = (2 * wt + 1) * W2a;
+    constexpr int Q = S::Q, E = S::E, RB = S::RB, CB = S::CB, QS = S::QS;
+    constexpr int W2a = 2 * WA + 1;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int Pt = tb.Pt, Pa = tb.Pa;
-    const int nsub = Pt * Pa * Pt * Pa;
+    const int NP = tb.Pt * tb.Pa;
+    const int nsub = NP * NP;
+    double *red = reinterpret_cast<double *>(smraw);                 // [2][SQ_WARPS]
+    int *ipat = reinterpret_cast<int *>(red + 2 * SQ_WARPS);        // [0] mask, [1] npat, [4..19] slot pattern
+    float *Rw = reinterpret_cast<float *>(ipat + 20);               // [warps][2][32][QS]
+    float *pts = Rw + SQ_WARPS * 2 * 32 * QS;                       // [2][NP][4]
+    float *wwin = pts + 2 * NP * 4;                                 // [E*E]
+    float *part = Rw;  // [warps][SQ_SLOTS][Q*Q], reuses the staging rows at the end of a LOR
+    static_assert(SQ_WARPS * SQ_SLOTS * Q * Q <= SQ_WARPS * 2 * 32 * QS, "part fits the staging rows");
+    static_assert(QS % 4 == 0 && (2 * 8 * SQ_WARPS + 4 * 20) % 16 == 0,
+                  "staging rows and sub-position centres start 16-byte aligned");
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    float *all = reinterpret_cast<float *>(smraw);
-    constexpr int WORDS = spread_q_words<S>();
-    static_assert(WORDS % 4 == 0 && QS % 4 == 0 && SQ_R % 4 == 0, "16-byte and 8-byte alignment");
-    float *Rv = all + warp * WORDS, *Rs = Rv + SQ_V * 32 * QS;
-    double *Es = reinterpret_cast<double *>(Rs + SQ_R * QS);
-    float *side = reinterpret_cast<float *>(Es + SQ_V * 32);
-    unsigned *steps = reinterpret_cast<unsigned *>(side + SQ_S * 32);
-    int *row1 = reinterpret_cast<int *>(steps + 32), *pairs = row1 + SQ_R;
-    // of all warps
-    double *red = reinterpret_cast<double *>(all + SQ_WARPS * WORDS);  // [2][SQ_WARPS]
-    float4 *pts = reinterpret_cast<float4 *>(red + 2 * SQ_WARPS);      // [2][Pt]: x, y, face
-    float *zs = reinterpret_cast<float *>(pts + 2 * Pt);               // [2][Pa]
-    // signs of travel: [0] transaxial, [1] axial; [2] the LOR
-    int *masks = reinterpret_cast<int *>(zs + 2 * Pa);
-    float *tabs = reinterpret_cast<float *>(masks + 4);
-    const float *part = all;  // [Q*Q] of each warp, over its variant rows
-    static_assert(Q * Q <= SQ_V * 32 * QS, "part fits the staged rows");
+    float *R1w = Rw + warp * 2 * 32 * QS, *R2w = R1w + 32 * QS;
     const int hw = lane >> 4, rb = (lane >> 2) & 3, cb = lane & 3;
-    const unsigned below = (1u << lane) - 1u;
-    const bool need_eta = norm == PSF_NORM_EFF;
-    // s = 2^lg: axial sub-positions of an end in a batch, nq batches to an end
-    int lg = 0;
-    while (lg < 4 && (1 << lg) < Pa) ++lg;
-    const int s = 1 << lg, nq = (Pa + s - 1) >> lg;
-    const GapConst gk = make_gapconst(sc, tb, tans, tabs);
-    for (int64_t lor = blockIdx.x;; lor += gridDim.x) {
-        __syncthreads();  // the LOR before: its readers of the shared arrays are done
-        if (queue) {
-            if (t == 0) masks[2] = (int)atomicAdd(queue, 1u);
-            __syncthreads();
-            lor = (unsigned)masks[2];
-        }
-        if (lor >= n_lors) break;
-        if (sym && sym[lor] >= 0) continue;  // an image of another class under the mirrors
+    const GapConst gk = make_gapconst(sc, tb, wwin + E * E);  // visible after the first barrier
+    for (int k = t; k < SQ_WARPS * 2 * 32 * QS; k += SP_THREADS) Rw[k] = 0.0f;
+    for (int64_t lor = blockIdx.x; lor < n_lors; lor += gridDim.x) {
         const int id1 = lors[2 * lor], id2 = lors[2 * lor + 1];
         const int ring1 = id1 / sc.Nt, c1 = id1 - ring1 * sc.Nt;
         const int ring2 = id2 / sc.Nt, c2 = id2 - ring2 * sc.Nt;
+        if (sym && sym[lor] >= 0) continue;  // an image of another class under the mirrors
         const int b1 = c1 / sc.Nb, i1 = c1 - b1 * sc.Nb;
         const int b2 = c2 / sc.Nb, i2 = c2 - b2 * sc.Nb;
         float *o = out + lor * (int64_t)E * E;
         const int nc = sc.Nt * sc.NR;
-#pragma unroll 1
-        for (int k = t; k < E * E; k += SQ_T) o[k] = 0.0f;
-        if (b1 == b2 || id1 < 0 || id2 < 0 || id1 >= nc || id2 >= nc) continue;
+        __syncthreads();  // previous LOR's readers of pts / wwin / part are done
+        if (b1 == b2 || id1 < 0 || id2 < 0 || id1 >= nc || id2 >= nc) {
+            for (int k = t; k < E * E; k += SP_THREADS) o[k] = 0.0f;
+            continue;
+        }
         float sb1, cb1, sb2, cb2;
         sincospif(2.0f * b1 / sc.R, &sb1, &cb1);
         sincospif(2.0f * b2 / sc.R, &sb2, &cb2);
-#pragma unroll 1
-        for (int k = t; k < 2 * Pt; k += SQ_T) {
-            const int end = k / Pt, p = k - end * Pt;
+        for (int k = t; k < 2 * NP; k += SP_THREADS) {
+            const int end = k / NP, sp = k - end * NP;
+            const int p = sp / tb.Pa, q = sp - p * tb.Pa;
+            const int i = end ? i2 : i1, ring = end ? ring2 : ring1;
             const float cbk = end ? cb2 : cb1, sbk = end ? sb2 : sb1;
-            const float u = (end ? i2 : i1) - 0.5f * (sc.Nb - 1);
-            const float se = fmaf(u, sc.pt, ((p + 0.5f) / Pt - 0.5f) * sc.wt);
-            pts[k] = make_float4(fmaf(sc.radius, cbk, -(se * sbk)), fmaf(sc.radius, sbk, se * cbk),
-                                 se, 0.0f);
+            const float se = (i - 0.5f * (sc.Nb - 1)) * sc.pt + ((p + 0.5f) / tb.Pt - 0.5f) * sc.wt;
+            const float ze = sc.z0 + ring * sc.pa + ((q + 0.5f) / tb.Pa - 0.5f) * sc.wa;
+            reinterpret_cast<float4 *>(pts)[k] =
+                make_float4(sc.radius * cbk - se * sbk, sc.radius * sbk + se * cbk, ze, se);
         }
-#pragma unroll 1
-        for (int k = t; k < 2 * Pa; k += SQ_T) {
-            const int end = k / Pa, q = k - end * Pa;
-            zs[k] = sc.z0 + (end ? ring2 : ring1) * sc.pa + ((q + 0.5f) / Pa - 0.5f) * sc.wa;
-        }
-        if (t < 2) masks[t] = 0;
+        for (int k = t; k < E * E; k += SP_THREADS) wwin[k] = 0.0f;
+        if (t == 0) ipat[0] = 0;
         __syncthreads();
-        // signs of travel of a transaxial pair: -1 (a photon leaves the ring
-        // the wrong way), else end 1's times 2 plus end 2's (1: forwards)
-        auto pair_dirs = [&](int p1, int p2, float &vn1, float &vt1, float &vn2, float &vt2) {
-            const float4 P1 = pts[p1], P2 = pts[Pt + p2];
-            const float dx = P1.x - P2.x, dy = P1.y - P2.y;
+        // pre-pass: the travel patterns present among the valid sub-LORs
+        unsigned mine = 0;
+        for (int s = t; s < nsub; s += SP_THREADS) {
+            const int s1 = s / NP, s2 = s - s1 * NP;
+            const float4 P1 = reinterpret_cast<const float4 *>(pts)[s1];
+            const float4 P2 = reinterpret_cast<const float4 *>(pts)[NP + s2];
+            const float dx = P1.x - P2.x, dy = P1.y - P2.y, dz = P1.z - P2.z;
+            float vn1, vt1, vn2, vt2;
             end_dir(dx, dy, cb1, sb1, vn1, vt1);
             end_dir(-dx, -dy, cb2, sb2, vn2, vt2);
-            if (!(vn1 > 0.0f && vn2 > 0.0f)) return -1;
-            return ((vt1 >= 0.0f) << 1) | (vt2 >= 0.0f);
-        };
-        auto axial_signs = [](float dz) { return ((dz >= 0.0f) << 1) | (-dz >= 0.0f); };
-        unsigned mt = 0, ma = 0;
-#pragma unroll 1
-        for (int k = t; k < Pt * Pt; k += SQ_T) {
-            float vn1, vt1, vn2, vt2;
-            const int s = pair_dirs(k / Pt, k % Pt, vn1, vt1, vn2, vt2);
-            if (s >= 0) mt |= 1u << s;
+            if (vn1 > 0.0f && vn2 > 0.0f)
+                mine |= 1u << (((vt1 >= 0.0f) << 3) | ((dz >= 0.0f) << 2) | ((vt2 >= 0.0f) << 1) |
+                               (-dz >= 0.0f));
         }
-#pragma unroll 1
-        for (int k = t; k < Pa * Pa; k += SQ_T) ma |= 1u << axial_signs(zs[k / Pa] - zs[Pa + k % Pa]);
-        mt = __reduce_or_sync(0xffffffffu, mt);
-        ma = __reduce_or_sync(0xffffffffu, ma);
-        if (lane == 0 && mt) atomicOr(masks, (int)mt);
-        if (lane == 0 && ma) atomicOr(masks + 1, (int)ma);
+        mine = __reduce_or_sync(0xffffffffu, mine);
+        if (lane == 0 && mine) atomicOr(ipat, (int)mine);
         __syncthreads();
-        const unsigned tsigns = masks[0], asigns = masks[1];
-        const bool one_sign = __popc(asigns) == 1;
-        // a warp's pairs are a 4 x 4 tile: its table reads hit about 4 + 4 rows
-        const int nt = (Pt + 3) >> 2;
-        const int sub = nt * nt < SQ_WARPS ? SQ_WARPS : 1;  // warps that share a tile
-        const int end = (lane >> lg) & 1, ring = end ? ring2 : ring1;
-        int np = 0;
-        const bool once = __popc(tsigns) * __popc(asigns) == 1;  // one pass
-        // the pass's sums over the warps, with their places in the window: within
-        // one pattern the quadrant-to-window map is one-to-one, so no two
-        // threads meet
-        auto each_sum = [&](int ts, int as, auto f) {
-            const int g1 = ts >> 1 ? 1 : -1, g2 = ts & 1 ? 1 : -1;
-            const int a1 = as >> 1 ? 1 : -1, a2 = as & 1 ? 1 : -1;
-#pragma unroll 1
-            for (int e = t; e < Q * Q; e += SQ_T) {
-                const int e1 = e / Q, e2 = e - e1 * Q;
-                const int x1 = e1 / (WA + 1), z1 = e1 - x1 * (WA + 1);
-                const int x2 = e2 / (WA + 1), z2 = e2 - x2 * (WA + 1);
-                if (x1 > wt || x2 > wt || z1 > wa || z2 > wa) continue;
-                float sum = 0.0f;
+        const unsigned present = (unsigned)ipat[0];
+        // a warp takes the sub-LORs of a tile of SQ_TA end-1 by SQ_TB end-2
+        // sub-positions: its table reads then hit about SQ_TA + SQ_TB rows
+        // instead of 33 for a run of 32 end-2 positions (17.3 ms against
+        // 22.1 ms on the 3D ring classes; 4 x 8 18.3, 16 x 2 18.1, 32 x 1 21.3)
+        const int ntb = (NP + SQ_TB - 1) >> SQ_TB_LOG;
+        const int ntile = ((NP + SQ_TA - 1) >> SQ_TA_LOG) * ntb;
+        const int npat = __popc(present);
+        double sfull = 0.0;
+        for (int pass = 0; pass * SQ_SLOTS < npat; ++pass) {
+            float acc[SQ_SLOTS][RB][CB];
 #pragma unroll
-                for (int w = 0; w < SQ_WARPS; ++w) sum += part[w * WORDS + e];
-                f(((g1 * x1 + wt) * W2a + a1 * z1 + wa) * E + (g2 * x2 + wt) * W2a + a2 * z2 + wa,
-                  sum);
-            }
-        };
-        double sfull = 0.0, swin = 0.0;
-#pragma unroll 1
-        for (int pass = 0; pass < 16; ++pass) {
-            const int ts = pass >> 2, as = pass & 3;  // (uniform over the CTA)
-            if (!((tsigns >> ts) & 1) || !((asigns >> as) & 1)) continue;
-            const int sga = (end ? as & 1 : as >> 1) ? 1 : -1;
-            float acc[RB][CB];
+            for (int a = 0; a < SQ_SLOTS; ++a)
 #pragma unroll
-            for (int i = 0; i < RB; ++i)
+                for (int i = 0; i < RB; ++i)
 #pragma unroll
-                for (int j = 0; j < CB; ++j) acc[i][j] = 0.0f;
-#pragma unroll 1
-            for (int u = warp; u < nt * nt * sub; u += SQ_WARPS) {
-                const int tile = u / sub;
-                // a lane: the transaxial side of an end of a pair
-                {
-                    const int p1 = tile / nt * 4 + ((lane & 15) >> 2);
-                    const int p2 = tile % nt * 4 + (lane & 3);
-                    bool in = p1 < Pt && p2 < Pt;
+                    for (int j = 0; j < CB; ++j) acc[a][i][j] = 0.0f;
+            for (int tile = warp; tile < ntile; tile += SQ_WARPS) {
+                const int ta = tile / ntb;
+                const int s1 = (ta << SQ_TA_LOG) + (lane >> SQ_TB_LOG);
+                const int s2 = ((tile - ta * ntb) << SQ_TB_LOG) + (lane & (SQ_TB - 1));
+                int slot = -1;
+                if (s1 < NP && s2 < NP) {
+                    const float4 P1 = reinterpret_cast<const float4 *>(pts)[s1];
+                    const float4 P2 = reinterpret_cast<const float4 *>(pts)[NP + s2];
+                    const float dx = P1.x - P2.x, dy = P1.y - P2.y, dz = P1.z - P2.z;
                     float vn1, vt1, vn2, vt2;
-                    if (in) in = pair_dirs(p1, p2, vn1, vt1, vn2, vt2) == ts;
-                    const unsigned ins = __ballot_sync(0xffffffffu, in) & 0xffffu;
-                    if (in) {
-                        const QSide e = end_side(sc, tb, gk, hw ? i2 : i1, hw ? p2 : p1,
-                                                 pts[hw ? Pt + p2 : p1].z, hw ? vn2 : vn1,
-                                                 hw ? vt2 : vt1);
-                        side[lane] = e.ih;
-                        side[32 + lane] = e.h;
-                        side[64 + lane] = e.run;
-                        side[96 + lane] = __int_as_float(e.row0);
-                        side[128 + lane] = __int_as_float(e.row1);
-                        side[160 + lane] = __int_as_float(e.m);
-                        side[192 + lane] = __int_as_float(2 * e.edge + e.gap);
-                        if (lane < 16) pairs[__popc(ins & below)] = lane;
+                    end_dir(dx, dy, cb1, sb1, vn1, vt1);
+                    end_dir(-dx, -dy, cb2, sb2, vn2, vt2);
+                    if (vn1 > 0.0f && vn2 > 0.0f) {
+                        const int P = ((vt1 >= 0.0f) << 3) | ((dz >= 0.0f) << 2) |
+                                      ((vt2 >= 0.0f) << 1) | (-dz >= 0.0f);
+                        // slot = rank of the pattern among those present
+                        const int sl = __popc(present & ((1u << P) - 1u)) - pass * SQ_SLOTS;
+                        if (sl >= 0 && sl < SQ_SLOTS) {
+                            slot = sl;
+                            QResp<WT, WA> r;
+                            end_resp_q<WT, WA>(sc, tb, gk, T, eta, i1, ring1, s1 / tb.Pa,
+                                               s1 % tb.Pa, P1.w, P1.z, vn1, vt1, dz, r);
+                            const double e1 = r.eta;
+                            stage_row<Q>(R1w + lane * QS, r.q);
+                            end_resp_q<WT, WA>(sc, tb, gk, T, eta, i2, ring2, s2 / tb.Pa,
+                                               s2 % tb.Pa, P2.w, P2.z, vn2, vt2, -dz, r);
+                            stage_row<Q>(R2w + lane * QS, r.q);
+                            sfull += e1 * r.eta;
+                        }
                     }
-                    np = __popc(ins);
                 }
                 __syncwarp();
-                // a lane: an end's q of a pair, against s of the other end's
-#pragma unroll 1
-                for (int b0 = u % sub * (16 >> lg); b0 < np; b0 += sub * (16 >> lg)) {
-                    const int slot = b0 + (lane >> (lg + 1));
-                    const bool in = slot < np;
-                    QSide e = {};
-                    if (in) {
-                        const int l = pairs[slot] + 16 * end;
-                        e.ih = side[l];
-                        e.h = side[32 + l];
-                        e.run = sga * side[64 + l];
-                        e.row0 = __float_as_int(side[96 + l]);
-                        e.row1 = __float_as_int(side[128 + l]);
-                        e.m = __float_as_int(side[160 + l]);
-                        e.edge = __float_as_int(side[192 + l]) >> 1;
-                        e.gap = __float_as_int(side[192 + l]) & 1;
-                    }
-                    const bool gap = e.gap && (need_eta || e.edge < WT);
-                    // the squares of s x s of (q1, q2)
-#pragma unroll 1
-                    for (int square = 0; square < nq * nq; ++square) {
-                        const int o1 = square / nq * s, o2 = square % nq * s;  // its first q1, q2
-                        const int q = (end ? o2 : o1) + (lane & (s - 1));
-                        const float zq = q < Pa ? zs[end * Pa + q] : 0.0f;
-                        const int ox = end ? o1 : o2;
-                        const float *zx = zs + (1 - end) * Pa + ox;  // the other end's
-                        // first members of the variants, members
-                        unsigned starts = 0, members = 0;
-                        int ka = 0;
-                        if (in && q < Pa) {
-                            int kl = 0, cl = 0;
-                            ka = polar_seed(tb, e, fabsf(zq - zx[0]));
-                            float lo = 1.0f, hi = 0.0f;  // adz of node ka: [lo, hi)
-                            const int nx = min(s, Pa - ox);
-#pragma unroll 1
-                            for (int j = 0; j < nx; ++j) {
-                                const float d = zq - zx[j], adz = fabsf(d);
-                                if (!one_sign && axial_signs(end ? -d : d) != as) continue;
-                                if (!(adz >= lo && adz < hi)) {
-                                    ka = node_by_tan(gk.tanA, tb.Ka, adz, e.h, ka);
-                                    lo = ka > 0 ? e.h * gk.tanA[ka - 1] : 0.0f;
-                                    hi = ka < tb.Ka - 1 ? e.h * gk.tanA[ka] : CUDART_INF_F;
-                                }
-                                const int c = gap ? end_gap_cell(sc, tb, gk, e, zq, adz, sga, ring) : 0;
-                                if (members == 0 || ka != kl || c != cl) starts |= 1u << j;
-                                members |= 1u << j;
-                                kl = ka;
-                                cl = c;
-                            }
-                        }
-                        // in pieces of step x step, in which no lane has more
-                        // variants than are staged (two at most in 2 x 2)
-                        int step = s;
-                        while (step > 2) {
-                            bool few = true;
-                            for (int j = 0; j < s; j += step) {
-                                const unsigned m = members & (((1u << step) - 1u) << j);
-                                few = few && __popc((starts & m) | (m & -m)) <= SQ_V;
-                            }
-                            if (__all_sync(0xffffffffu, few)) break;
-                            step >>= 1;
-                        }
-#pragma unroll 1
-                        for (int piece = 0; piece < (s / step) * (s / step); ++piece) {
-                            const int f1 = piece / (s / step) * step, f2 = piece % (s / step) * step;
-                            const int fo = end ? f2 : f1, fx = end ? f1 : f2;
-                            const bool act = (lane & (s - 1)) >= fo && (lane & (s - 1)) < fo + step;
-                            const unsigned mem = act ? members & (((1u << step) - 1u) << fx) : 0;
-                            const unsigned st = (starts & mem) | (mem & -mem);
-                            const int nv = __popc(st);
-                            const int nmax = __reduce_max_sync(0xffffffffu, nv);
-                            __syncwarp();  // the rows before are read
-                            steps[lane] = st;
-                            unsigned rest = st;
-#pragma unroll 1
-                            for (int v = 0; v < nmax; ++v) {
-                                if (v >= nv) continue;
-                                const float adz = fabsf(zq - zx[__ffs(rest) - 1]);
-                                rest &= rest - 1;
-                                ka = node_by_tan(gk.tanA, tb.Ka, adz, e.h, ka);
-                                float r[Q];
-                                double es = 0.0;
+                const float *ra = R1w + rb * RB, *rbp = R2w + cb * CB;
+                const int s0 = __shfl_sync(0xffffffffu, slot, 0);
+                if (__all_sync(0xffffffffu, slot == s0)) {
+                    // common case: one travel pattern for the whole warp
 #pragma unroll
-                                for (int k = 0; k < Q; ++k) r[k] = 0.0f;
-                                end_rows<WT, WA>(
-                                    sc, tb, T, eta, e, ka, sga > 0 ? q : Pa - 1 - q,
-                                    gap ? end_gap_cell(sc, tb, gk, e, zq, adz, sga, ring) : 0, sga, r,
-                                    need_eta ? &es : nullptr);
-                                float4 *dst = reinterpret_cast<float4 *>(Rv + (v * 32 + lane) * QS);
+                    for (int sl = 0; sl < SQ_SLOTS; ++sl)
+                        if (s0 == sl) acc_all32<RB, CB, QS>(acc[sl], ra, rbp, hw);
+                } else {
+#pragma unroll 4
+                    for (int k = 0; k < 16; ++k) {
+                        const int row = half_row(k, hw);
+                        const int sk = __shfl_sync(0xffffffffu, slot, row);
+                        if (sk < 0) continue;
+                        float a[RB], b[CB];
+                        load_ab<RB, CB>(ra + row * QS, rbp + row * QS, a, b);
 #pragma unroll
-                                for (int k = 0; k < Q / 4; ++k)
-                                    dst[k] = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
-                                Es[v * 32 + lane] = es;
+                        for (int sl = 0; sl < SQ_SLOTS; ++sl)
+                            if (sk == sl) {
+#pragma unroll
+                                for (int i = 0; i < RB; ++i)
+#pragma unroll
+                                    for (int j = 0; j < CB; ++j)
+                                        acc[sl][i][j] = fmaf(a[i], b[j], acc[sl][i][j]);
                             }
-                            __syncwarp();
-                            // runs: lanes l1 (of end 1) and l1 + s share q1
-                            const int l1 = lane & ~s, l2 = l1 + s - (lane & (s - 1));
-                            const unsigned st1 = __shfl_sync(0xffffffffu, st, l1);
-                            const unsigned mem1 = __shfl_sync(0xffffffffu, mem, l1);
-                            const unsigned upto = (2u << (lane & (s - 1))) - 1u;
-                            int at = 0;
-                            float *pos[SQ_V];
-#pragma unroll
-                            for (int v = 0; v < SQ_V; ++v) {
-                                const unsigned m = __ballot_sync(0xffffffffu, end == 0 && nv > v);
-                                const int p = at + __popc(m & ((1u << l1) - 1u));
-                                pos[v] = Rs + p * QS;
-                                at += __popc(m);
-                                if (end == 0 && nv > v) row1[p] = (v * 32 + lane) * QS;
-                            }
-                            if (need_eta)
-#pragma unroll 1
-                                for (int j = f2 + end; j < f2 + step; j += 2)
-                                    if ((mem1 >> j) & 1) {
-                                        const int v1 = __popc(st1 & ((2u << j) - 1u)) - 1;
-                                        const int v2 = __popc(steps[l2 + j] & upto) - 1;
-                                        sfull += Es[v1 * 32 + l1] * Es[v2 * 32 + l2 + j];
-                                    }
-                            constexpr int PARTS = Q / 4, PH = (PARTS + 1) / 2;
-                            float4 sum[PH];
-                            int v = -1;
-#pragma unroll 1
-                            for (int j = f2; j < f2 + step; ++j) {
-                                if ((st1 >> j) & 1) {
-                                    if (v >= 0) put_sum<S>(v == 0 ? pos[0] : pos[1], end, sum);
-                                    ++v;
-#pragma unroll
-                                    for (int k = 0; k < PH; ++k) sum[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                                }
-                                if ((mem1 >> j) & 1) {
-                                    const float4 *src = reinterpret_cast<const float4 *>(
-                                        Rv + ((__popc(steps[l2 + j] & upto) - 1) * 32 + l2 + j) * QS);
-#pragma unroll
-                                    for (int k = 0; k < PH; ++k) {
-                                        if (end * PH + k >= PARTS) continue;
-                                        const float4 x = src[end * PH + k];
-                                        sum[k].x += x.x;
-                                        sum[k].y += x.y;
-                                        sum[k].z += x.z;
-                                        sum[k].w += x.w;
-                                    }
-                                }
-                            }
-                            if (v >= 0)
-                                put_sum<S>(v == 0 ? pos[0] : v == 1 ? pos[1] : pos[2], end, sum);
-                            __syncwarp();
-                            acc_rows<S>(acc, Rv, row1, Rs, at, hw, rb, cb);
-                        }
                     }
                 }
-                __syncwarp();  // the sides and rows are read
+                __syncwarp();
             }
-            // per-warp accumulators (the two halves summed) -> part
+            // per-warp accumulators (the two halves summed) -> part, then fold
+            // into the window
 #pragma unroll
-            for (int i = 0; i < RB; ++i)
+            for (int sl = 0; sl < SQ_SLOTS; ++sl)
 #pragma unroll
-                for (int j = 0; j < CB; ++j) {
-                    acc[i][j] += __shfl_xor_sync(0xffffffffu, acc[i][j], 16);
-                    const int e1 = rb * RB + i, e2 = cb * CB + j;
-                    if (hw == 0 && e1 < Q && e2 < Q) Rv[e1 * Q + e2] = acc[i][j];
-                }
+                for (int i = 0; i < RB; ++i)
+#pragma unroll
+                    for (int j = 0; j < CB; ++j)
+                        acc[sl][i][j] += __shfl_xor_sync(0xffffffffu, acc[sl][i][j], 16);
             __syncthreads();
-            each_sum(ts, as, [&](int at, float v) {
-                swin += (double)v;
-                if (!once) o[at] += v;
-            });
-            __syncthreads();  // the next pass may meet these entries; part aliases the staged rows
+            if (hw == 0) {
+#pragma unroll
+                for (int sl = 0; sl < SQ_SLOTS; ++sl)
+#pragma unroll
+                    for (int i = 0; i < RB; ++i)
+#pragma unroll
+                        for (int j = 0; j < CB; ++j) {
+                            const int e1 = rb * RB + i, e2 = cb * CB + j;
+                            if (e1 < Q && e2 < Q)
+                                part[(warp * SQ_SLOTS + sl) * Q * Q + e1 * Q + e2] = acc[sl][i][j];
+                        }
+            }
+            __syncthreads();
+            const int nsl = min(SQ_SLOTS, npat - pass * SQ_SLOTS);
+            // fold slot by slot, in pattern order: within one pattern the
+            // quadrant-to-window map is one-to-one, so no two threads meet
+            unsigned rest = present;
+            for (int c = 0; c < pass * SQ_SLOTS; ++c) rest &= rest - 1u;
+            for (int sl = 0; sl < nsl; ++sl) {
+                const int P = __ffs(rest) - 1;
+                rest &= rest - 1u;
+                const int g1 = (P >> 3) & 1 ? 1 : -1, a1 = (P >> 2) & 1 ? 1 : -1;
+                const int g2 = (P >> 1) & 1 ? 1 : -1, a2 = P & 1 ? 1 : -1;
+                for (int e = t; e < Q * Q; e += SP_THREADS) {
+                    const int e1 = e / Q, e2 = e - e1 * Q;
+                    const int x1 = e1 / (WA + 1), z1 = e1 - x1 * (WA + 1);
+                    const int x2 = e2 / (WA + 1), z2 = e2 - x2 * (WA + 1);
+                    const int w1 = (g1 * x1 + WT) * W2a + (a1 * z1 + WA);
+                    const int w2 = (g2 * x2 + WT) * W2a + (a2 * z2 + WA);
+                    float sum = 0.0f;
+#pragma unroll
+                    for (int w = 0; w < SQ_WARPS; ++w) sum += part[(w * SQ_SLOTS + sl) * Q * Q + e];
+                    wwin[w1 * E + w2] += sum;
+                }
+                __syncthreads();  // the next slot may meet these entries; part aliases the staging rows
+            }
         }
-        // FP64 totals: sfull over sub-LORs, sw over the window
+        // FP64 totals: sfull over sub-LORs, sw over the accumulated window
+        double swin = 0.0;
+        for (int wc = t; wc < E * E; wc += SP_THREADS) swin += (double)wwin[wc];
         sfull = warp_sum_d(sfull);
         swin = warp_sum_d(swin);
         if (lane == 0) {
@@ -669,20 +543,11 @@ __global__ void __launch_bounds__(SQ_T, 4) spread_q_kernel(
             sf += red[w];
             sw += red[SQ_WARPS + w];
         }
-        double scale = 1.0;
-        if (norm == PSF_NORM_UNIT && sw > 0.0)
-            scale = 1.0 / sw;  // total = 1
-        else if (norm == PSF_NORM_EFF && sw > 0.0)
-            scale = sf / (sw * nsub);  // total = mean eta1 eta2
-        else
-            scale = 1.0 / nsub;  // mean
+        double scale = 1.0 / nsub;                                       // NONE: mean
+        if (norm == PSF_NORM_EFF && sw > 0.0) scale = sf / (sw * nsub);    // total = mean eta1 eta2
+        if (norm == PSF_NORM_UNIT && sw > 0.0) scale = 1.0 / sw;           // total = 1
         const float fs = (float)scale;
-        if (once) {
-            each_sum(__ffs(tsigns) - 1, __ffs(asigns) - 1, [&](int at, float v) { o[at] = v * fs; });
-        } else {
-#pragma unroll 1
-            for (int k = t; k < E * E; k += SQ_T) o[k] *= fs;
-        }
+        for (int k = t; k < E * E; k += SP_THREADS) o[k] = wwin[k] * fs;
     }
 }
 
@@ -693,21 +558,21 @@ __global__ void __launch_bounds__(SQ_T, 4) spread_q_kernel(
 // does not travel to, so the window is one small product sum_s r1_s (x) r2_s
 // whatever the travel patterns, each lane owning a few of its entries (fixed
 // order over s).  Responses and node decisions are spread_q_kernel's.  Bound by
-// latency: RING2D, 2,016 LORs of 16 sub-LORs: 70 -> 15 us between events (about
-// 5 us of which are the events'; 18 us with the node tangents found by the CTAs).
+// latency: RING2D, 2,016 LORs of 16 sub-LORs: 70 -> 18 us
+// between events (about 5 us of which are the events').
 constexpr int SPL_T = 128;
 constexpr int SPL_NSUB = 64;  // most sub-LORs: above, a warp's serial chunks lose to a CTA
 
 template <int WT, int G>
 __global__ void __launch_bounds__(SPL_T) spread_planar_kernel(
-    Scan sc, Tab tb, const __grid_constant__ NodeTans tans, const float *__restrict__ T,
-    const double *__restrict__ eta, const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
+    Scan sc, Tab tb, const float *__restrict__ T, const double *__restrict__ eta,
+    const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
     const int32_t *__restrict__ sym) {
     constexpr int E = 2 * WT + 1, OWN = (E * E + G - 1) / G, NG = SPL_T / G;
     constexpr int RS = (2 * E) | 1;  // odd: the lanes' rows start in different banks
     extern __shared__ float spl_tabs[];          // node tangents
     __shared__ float R[NG][G][RS];                // a chunk's responses at both ends
-    const GapConst gk = make_gapconst(sc, tb, tans, spl_tabs);
+    const GapConst gk = make_gapconst(sc, tb, spl_tabs);
     __syncthreads();
     const int t = threadIdx.x, grp = t / G, l = t % G;
     const unsigned mask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << ((t & 31) / G * G);
@@ -809,7 +674,7 @@ static int launch_spread_planar(const Scan &sc, const Tab &tb, const float *T, c
     {
         PSF_TIMED("spread_planar_kernel", st);
         spread_planar_kernel<WT, G><<<(int)(need < cap ? need : cap), SPL_T, shm, st>>>(
-            sc, tb, make_nodetans(sc, tb), T, eta, lors, n_lors, norm, out, sym);
+            sc, tb, T, eta, lors, n_lors, norm, out, sym);
     }
     PSF_LAUNCHED();
     return PSF_OK;
@@ -817,8 +682,8 @@ static int launch_spread_planar(const Scan &sc, const Tab &tb, const float *T, c
 
 template <int WT, int WA>
 static int launch_spread_q(const Scan &sc, const Tab &tb, const float *T, const double *eta,
-                           const int32_t *lors, int64_t n_lors, int wt, int wa, int norm, float *out,
-                           const int32_t *sym, unsigned *queue, cudaStream_t st) {
+                           const int32_t *lors, int64_t n_lors, int norm, float *out,
+                           const int32_t *sym, cudaStream_t st) {
     const size_t shm = spread_q_smem<WT, WA>(tb);
     if (shm > 200 * 1024) return PSF_EINVAL;
     PSF_TRY(cudaFuncSetAttribute(spread_q_kernel<WT, WA>,
@@ -826,14 +691,15 @@ static int launch_spread_q(const Scan &sc, const Tab &tb, const float *T, const 
     int dev = 0, sms = 148, per_sm = 0;
     PSF_TRY(cudaGetDevice(&dev));
     PSF_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    PSF_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, spread_q_kernel<WT, WA>, SQ_T,
-                                                          shm));
+    PSF_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, spread_q_kernel<WT, WA>,
+                                                          SP_THREADS, shm));
     if (per_sm < 1) per_sm = 1;
     const int64_t cap = (int64_t)sms * per_sm;
+    const int64_t grid = n_lors < cap ? n_lors : cap;
     {
         PSF_TIMED("spread_q_kernel", st);
-        spread_q_kernel<WT, WA><<<(int)(n_lors < cap ? n_lors : cap), SQ_T, shm, st>>>(
-            sc, tb, make_nodetans(sc, tb), T, eta, lors, n_lors, wt, wa, norm, out, sym, queue);
+        spread_q_kernel<WT, WA><<<(int)grid, SP_THREADS, shm, st>>>(sc, tb, T, eta, lors, n_lors,
+                                                                    norm, out, sym);
     }
     PSF_LAUNCHED();
     return PSF_OK;
@@ -876,7 +742,6 @@ __global__ void spread_sym_kernel(LorSet ls, int32_t *__restrict__ sym) {
     __syncthreads();
     const int D = 2 * ls.Dm + 1;
     const int64_t n_cls = ls.ntp_cls * D;
-    if (blockIdx.x == 0 && threadIdx.x == 0) sym[n_cls] = 0;  // the spread kernel's queue
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cls;
          c += (int64_t)gridDim.x * blockDim.x) {
         const int64_t tp = c / D;
@@ -945,7 +810,7 @@ __global__ void spread_mirror_kernel(int64_t n_cls, int Wt, int Wa,
 static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, const float *table,
                       const double *eta, const int32_t *lors, int64_t n_lors, int32_t half_t,
                       int32_t half_a, int32_t norm, float *spread, const int32_t *sym,
-                      unsigned *queue, cudaStream_t st) {
+                      cudaStream_t st) {
     Scan sc;
     Tab tb;
     int rc = make_scan(scanner, &sc);
@@ -958,6 +823,10 @@ static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, co
     if (n_lors == 0) return PSF_OK;
     if (!table || !eta || !lors || !spread) return PSF_EINVAL;
     if (tb.Pt * tb.Pa > 1024) return PSF_EINVAL;
+    if (half_t == 3 && half_a == 3)
+        return launch_spread_q<3, 3>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
+    if (half_t == 3 && half_a == 2)
+        return launch_spread_q<3, 2>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
     const int nsub = tb.Pt * tb.Pa * tb.Pt * tb.Pa;
     if (half_t == 3 && half_a == 0 && nsub <= SPL_NSUB && 2 * tb.Kt + tb.Ka <= 4096)
         return nsub <= 16
@@ -966,11 +835,7 @@ static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, co
                    : launch_spread_planar<3, 32>(sc, tb, table, eta, lors, n_lors, norm, spread,
                                                  sym, st);
     if (half_t == 3 && half_a == 0)
-        return launch_spread_q<3, 0>(sc, tb, table, eta, lors, n_lors, half_t, half_a, norm, spread,
-                                     sym, queue, st);
-    if (half_t == 3 && (half_a == 2 || half_a == 3))
-        return launch_spread_q<3, 3>(sc, tb, table, eta, lors, n_lors, half_t, half_a, norm, spread,
-                                     sym, queue, st);
+        return launch_spread_q<3, 0>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
     size_t shm = spread_smem(tb, half_t, half_a);
     if (shm > 200 * 1024) return PSF_EINVAL;
     PSF_TRY(cudaFuncSetAttribute(spread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -996,7 +861,7 @@ extern "C" int psf_bin_spread(const psf_scanner *scanner, const psf_table_desc *
                               float *spread, void *stream) {
     PSF_RANGE("psf_bin_spread");
     return bin_spread(scanner, desc, table, eta, lors, n_lors, half_t, half_a, norm, spread,
-                      nullptr, nullptr, as_stream(stream));
+                      nullptr, as_stream(stream));
 }
 
 extern "C" int psf_bin_spread_classes(const psf_scanner *scanner, const psf_table_desc *desc,
@@ -1014,8 +879,7 @@ extern "C" int psf_bin_spread_classes(const psf_scanner *scanner, const psf_tabl
     if (!class_lors || !spread) return PSF_EINVAL;
     cudaStream_t st = as_stream(stream);
     int32_t *sym = nullptr;
-    // and the next class to compute: of a CTA's share, uneven parts are images
-    PSF_TRY(cudaMallocAsync(&sym, sizeof(int32_t) * (n_cls + 1), st));
+    PSF_TRY(cudaMallocAsync(&sym, sizeof(int32_t) * n_cls, st));
     int dev = 0, sms = 148;
     rc = cudaGetDevice(&dev) != cudaSuccess ||
                  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess
@@ -1030,7 +894,7 @@ extern "C" int psf_bin_spread_classes(const psf_scanner *scanner, const psf_tabl
     // the smallest class of each orbit through the spread kernel ...
     if (!rc)
         rc = bin_spread(scanner, desc, table, eta, class_lors, n_cls, half_t, half_a, norm,
-                        spread, sym, reinterpret_cast<unsigned *>(sym + n_cls), st);
+                        spread, sym, st);
     // ... the others as its images
     if (!rc) {
         PSF_TIMED("spread_mirror_kernel", st);

@@ -145,26 +145,6 @@ def test_planar_spreads(P, orc, n_sub, norm):
     assert_close(got[sure], want[sure], 1e-5, (1e-6 * scale + 1e-30)[sure], "planar spreads")
 
 
-@pytest.mark.parametrize("n_sub", [(4, 1), (5, 3), (3, 8), (2, 20)])
-@pytest.mark.parametrize("window,norm", [((3, 3), 1), ((3, 2), 2), ((3, 0), 0)])
-def test_spreads_by_axial_steps(P, orc, n_sub, window, norm):
-    """Spreads with pairs of sub-positions that leave lanes and tile corners
-    idle, axial ones that fill no batch, one and two, ring differences with
-    both signs of travel, and a window inside the widest."""
-    w = I.workload("RING3D_SMALL")
-    s, t = w["scanner"], dict(w["table"], n_sub_t=n_sub[0], n_sub_a=n_sub[1])
-    T, eta = P.response_build(s, t)
-    To, _ = orc.table_build(s, t)
-    L = I.workload_lors(w)
-    L = L[np.random.default_rng(5).permutation(len(L))[:400]]
-    got = P.bin_spread(s, t, T, eta, torch.from_numpy(L).cuda(), *window, norm=norm).cpu().numpy()
-    want = orc.spread(s, t, To, L, *window, norm=norm)
-    sure = orc.tie_margin(s, t, To, L) > 1e-5
-    assert sure.mean() > 0.3
-    scale = np.abs(want).reshape(len(L), -1).max(1)[:, None, None]
-    assert_close(got[sure], want[sure], 1e-5, (1e-6 * scale + 1e-30)[sure], "spreads")
-
-
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("start", ["nothing", "sens", "x0", "both"])
 @pytest.mark.parametrize("iters", [0, 1, 3])
