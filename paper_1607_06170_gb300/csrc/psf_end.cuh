@@ -125,13 +125,38 @@ struct GapConst {
     const float *tanT, *tanB, *tanA;  // [Kt - 1], [Kt - 1], [Ka - 1] (shared memory)
 };
 
+// The tangents, from the host: FP64 tangents in every CTA (and t2 in every
+// thread) took a fifth of a planar ring's spreads (32 -> 24 us for 64 sub-LORs
+// each).  n = 0: more nodes than fit a kernel argument, found by the CTA.
+struct NodeTans {
+    float t2;
+    int n;
+    float t[256];
+};
+
+inline NodeTans make_nodetans(const Scan &sc, const Tab &tb) {
+    NodeTans k;
+    const double st = (double)tb.dt, sa = (double)tb.da, g = (double)sc.two_pi_R;
+    const double half_pi = 1.5707963267948966;
+    k.t2 = (float)tan(g);
+    k.n = 2 * (int64_t)tb.Kt + tb.Ka <= 256 ? 2 * tb.Kt + tb.Ka : 0;
+    for (int j = 0; j < k.n; ++j) {
+        const double b = j < tb.Kt       ? (j + 0.5) * st
+                         : j < 2 * tb.Kt ? (j - tb.Kt + 0.5) * st + g
+                                         : (j - 2 * tb.Kt + 0.5) * sa;
+        k.t[j] = b < half_pi ? (float)tan(b) : INFINITY;
+    }
+    return k;
+}
+
 // Tangent tables in shared memory (2 * Kt + Ka floats); call with every
 // thread of the CTA, then synchronise.
-__device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb, float *tabs) {
+__device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb, const NodeTans &nt,
+                                                  float *tabs) {
     GapConst k;
     k.c2 = cosf(sc.two_pi_R);
     k.s2 = sc.sin_two_pi_R;
-    k.t2 = (float)tan((double)sc.two_pi_R);
+    k.t2 = nt.t2;
     k.ipt = 1.0f / sc.pt;
     k.ipa = 1.0f / sc.pa;
     k.iwt = 1.0f / sc.wt;
@@ -140,7 +165,8 @@ __device__ __forceinline__ GapConst make_gapconst(const Scan &sc, const Tab &tb,
     float *tT = tabs, *tB = tabs + tb.Kt, *tA = tabs + 2 * tb.Kt;
     const double st = (double)tb.dt, sa = (double)tb.da, g = (double)sc.two_pi_R;
     const double half_pi = 1.5707963267948966;
-    for (int j = threadIdx.x; j < 2 * tb.Kt + tb.Ka; j += blockDim.x) {
+    for (int j = threadIdx.x; j < nt.n; j += blockDim.x) tabs[j] = nt.t[j];
+    for (int j = threadIdx.x; j < 2 * tb.Kt + tb.Ka && !nt.n; j += blockDim.x) {
         double b;
         float* dst;
         if (j < tb.Kt) { b = (j + 0.5) * st; dst = tT + j; }

@@ -233,7 +233,12 @@ static size_t spread_smem(const Tab &tb, int Wt, int Wa) {
 // and normalised with FP64 totals.  One slot (a pass per pattern) leaves the
 // registers for three CTAs per SM, which hides more latency than the extra
 // passes over the sub-LOR directions cost (22.1 ms against 24.2 ms with four
-// slots at two CTAs per SM, 3D ring classes).
+// slots at two CTAs per SM, 3D ring classes).  The classes that are computed lie
+// unevenly among their images, so the CTAs take the next one from a queue: 4.65 ->
+// 4.43 ms for RING3D's 21,744 of 84,227.  (Sums by axial steps -- a response
+// evaluated once per step of its polar node or gap cell, outer products of sums --
+// take 3.2 ms, but round the last bits otherwise, and by these a truncation ranks
+// the mirror images of an entry: 4.5 % of the kept indices changed.)
 constexpr int SQ_SLOTS = 1;
 constexpr int SQ_WARPS = SP_THREADS / 32;
 constexpr int SQ_TA_LOG = 3, SQ_TB_LOG = 2;  // sub-LOR tile of a warp: 8 x 4
@@ -333,9 +338,9 @@ static size_t spread_q_smem(const Tab &tb) {
 
 template <int WT, int WA>
 __global__ void __launch_bounds__(SP_THREADS, 3) spread_q_kernel(
-    Scan sc, Tab tb, const float *__restrict__ T, const double *__restrict__ eta,
-    const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
-    const int32_t *__restrict__ sym) {
+    Scan sc, Tab tb, const __grid_constant__ NodeTans tans, const float *__restrict__ T,
+    const double *__restrict__ eta, const int32_t *__restrict__ lors, int64_t n_lors, int norm,
+    float *__restrict__ out, const int32_t *__restrict__ sym, unsigned *queue) {
     using S = SqShape<WT, WA>;
     constexpr int Q = S::Q, E = S::E, RB = S::RB, CB = S::CB, QS = S::QS;
     constexpr int W2a = 2 * WA + 1;
@@ -354,9 +359,19 @@ __global__ void __launch_bounds__(SP_THREADS, 3) spread_q_kernel(
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     float *R1w = Rw + warp * 2 * 32 * QS, *R2w = R1w + 32 * QS;
     const int hw = lane >> 4, rb = (lane >> 2) & 3, cb = lane & 3;
-    const GapConst gk = make_gapconst(sc, tb, wwin + E * E);  // visible after the first barrier
+    const GapConst gk = make_gapconst(sc, tb, tans, wwin + E * E);  // visible after the first barrier
     for (int k = t; k < SQ_WARPS * 2 * 32 * QS; k += SP_THREADS) Rw[k] = 0.0f;
-    for (int64_t lor = blockIdx.x; lor < n_lors; lor += gridDim.x) {
+    __shared__ unsigned taken;
+    // queue: the next LOR to take (null: strided); of a CTA's share, uneven
+    // parts are images of others
+    for (int64_t lor = blockIdx.x;; lor += gridDim.x) {
+        if (queue) {
+            __syncthreads();
+            if (t == 0) taken = atomicAdd(queue, 1u);
+            __syncthreads();
+            lor = taken;
+        }
+        if (lor >= n_lors) break;
         const int id1 = lors[2 * lor], id2 = lors[2 * lor + 1];
         const int ring1 = id1 / sc.Nt, c1 = id1 - ring1 * sc.Nt;
         const int ring2 = id2 / sc.Nt, c2 = id2 - ring2 * sc.Nt;
@@ -558,21 +573,21 @@ __global__ void __launch_bounds__(SP_THREADS, 3) spread_q_kernel(
 // does not travel to, so the window is one small product sum_s r1_s (x) r2_s
 // whatever the travel patterns, each lane owning a few of its entries (fixed
 // order over s).  Responses and node decisions are spread_q_kernel's.  Bound by
-// latency: RING2D, 2,016 LORs of 16 sub-LORs: 70 -> 18 us
-// between events (about 5 us of which are the events').
+// latency: RING2D, 2,016 LORs of 16 sub-LORs: 70 -> 15 us between events (about
+// 5 us of which are the events'; 18 us with the node tangents found by the CTAs).
 constexpr int SPL_T = 128;
 constexpr int SPL_NSUB = 64;  // most sub-LORs: above, a warp's serial chunks lose to a CTA
 
 template <int WT, int G>
 __global__ void __launch_bounds__(SPL_T) spread_planar_kernel(
-    Scan sc, Tab tb, const float *__restrict__ T, const double *__restrict__ eta,
-    const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
+    Scan sc, Tab tb, const __grid_constant__ NodeTans tans, const float *__restrict__ T,
+    const double *__restrict__ eta, const int32_t *__restrict__ lors, int64_t n_lors, int norm, float *__restrict__ out,
     const int32_t *__restrict__ sym) {
     constexpr int E = 2 * WT + 1, OWN = (E * E + G - 1) / G, NG = SPL_T / G;
     constexpr int RS = (2 * E) | 1;  // odd: the lanes' rows start in different banks
     extern __shared__ float spl_tabs[];          // node tangents
     __shared__ float R[NG][G][RS];                // a chunk's responses at both ends
-    const GapConst gk = make_gapconst(sc, tb, spl_tabs);
+    const GapConst gk = make_gapconst(sc, tb, tans, spl_tabs);
     __syncthreads();
     const int t = threadIdx.x, grp = t / G, l = t % G;
     const unsigned mask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << ((t & 31) / G * G);
@@ -674,7 +689,7 @@ static int launch_spread_planar(const Scan &sc, const Tab &tb, const float *T, c
     {
         PSF_TIMED("spread_planar_kernel", st);
         spread_planar_kernel<WT, G><<<(int)(need < cap ? need : cap), SPL_T, shm, st>>>(
-            sc, tb, T, eta, lors, n_lors, norm, out, sym);
+            sc, tb, make_nodetans(sc, tb), T, eta, lors, n_lors, norm, out, sym);
     }
     PSF_LAUNCHED();
     return PSF_OK;
@@ -683,7 +698,7 @@ static int launch_spread_planar(const Scan &sc, const Tab &tb, const float *T, c
 template <int WT, int WA>
 static int launch_spread_q(const Scan &sc, const Tab &tb, const float *T, const double *eta,
                            const int32_t *lors, int64_t n_lors, int norm, float *out,
-                           const int32_t *sym, cudaStream_t st) {
+                           const int32_t *sym, unsigned *queue, cudaStream_t st) {
     const size_t shm = spread_q_smem<WT, WA>(tb);
     if (shm > 200 * 1024) return PSF_EINVAL;
     PSF_TRY(cudaFuncSetAttribute(spread_q_kernel<WT, WA>,
@@ -698,8 +713,8 @@ static int launch_spread_q(const Scan &sc, const Tab &tb, const float *T, const 
     const int64_t grid = n_lors < cap ? n_lors : cap;
     {
         PSF_TIMED("spread_q_kernel", st);
-        spread_q_kernel<WT, WA><<<(int)grid, SP_THREADS, shm, st>>>(sc, tb, T, eta, lors, n_lors,
-                                                                    norm, out, sym);
+        spread_q_kernel<WT, WA><<<(int)grid, SP_THREADS, shm, st>>>(
+            sc, tb, make_nodetans(sc, tb), T, eta, lors, n_lors, norm, out, sym, queue);
     }
     PSF_LAUNCHED();
     return PSF_OK;
@@ -742,6 +757,7 @@ __global__ void spread_sym_kernel(LorSet ls, int32_t *__restrict__ sym) {
     __syncthreads();
     const int D = 2 * ls.Dm + 1;
     const int64_t n_cls = ls.ntp_cls * D;
+    if (blockIdx.x == 0 && threadIdx.x == 0) sym[n_cls] = 0;  // the spread kernel's queue
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cls;
          c += (int64_t)gridDim.x * blockDim.x) {
         const int64_t tp = c / D;
@@ -827,7 +843,7 @@ __global__ void spread_mirror_kernel(int64_t n_cls, int Wt, int Wa,
 static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, const float *table,
                       const double *eta, const int32_t *lors, int64_t n_lors, int32_t half_t,
                       int32_t half_a, int32_t norm, float *spread, const int32_t *sym,
-                      cudaStream_t st) {
+                      unsigned *queue, cudaStream_t st) {
     Scan sc;
     Tab tb;
     int rc = make_scan(scanner, &sc);
@@ -841,9 +857,11 @@ static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, co
     if (!table || !eta || !lors || !spread) return PSF_EINVAL;
     if (tb.Pt * tb.Pa > 1024) return PSF_EINVAL;
     if (half_t == 3 && half_a == 3)
-        return launch_spread_q<3, 3>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
+        return launch_spread_q<3, 3>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, queue,
+                                     st);
     if (half_t == 3 && half_a == 2)
-        return launch_spread_q<3, 2>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
+        return launch_spread_q<3, 2>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, queue,
+                                     st);
     const int nsub = tb.Pt * tb.Pa * tb.Pt * tb.Pa;
     if (half_t == 3 && half_a == 0 && nsub <= SPL_NSUB && 2 * tb.Kt + tb.Ka <= 4096)
         return nsub <= 16
@@ -852,7 +870,8 @@ static int bin_spread(const psf_scanner *scanner, const psf_table_desc *desc, co
                    : launch_spread_planar<3, 32>(sc, tb, table, eta, lors, n_lors, norm, spread,
                                                  sym, st);
     if (half_t == 3 && half_a == 0)
-        return launch_spread_q<3, 0>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, st);
+        return launch_spread_q<3, 0>(sc, tb, table, eta, lors, n_lors, norm, spread, sym, queue,
+                                     st);
     size_t shm = spread_smem(tb, half_t, half_a);
     if (shm > 200 * 1024) return PSF_EINVAL;
     PSF_TRY(cudaFuncSetAttribute(spread_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -878,7 +897,7 @@ extern "C" int psf_bin_spread(const psf_scanner *scanner, const psf_table_desc *
                               float *spread, void *stream) {
     PSF_RANGE("psf_bin_spread");
     return bin_spread(scanner, desc, table, eta, lors, n_lors, half_t, half_a, norm, spread,
-                      nullptr, as_stream(stream));
+                      nullptr, nullptr, as_stream(stream));
 }
 
 extern "C" int psf_bin_spread_classes(const psf_scanner *scanner, const psf_table_desc *desc,
@@ -896,7 +915,8 @@ extern "C" int psf_bin_spread_classes(const psf_scanner *scanner, const psf_tabl
     if (!class_lors || !spread) return PSF_EINVAL;
     cudaStream_t st = as_stream(stream);
     int32_t *sym = nullptr;
-    PSF_TRY(cudaMallocAsync(&sym, sizeof(int32_t) * n_cls, st));
+    // and the next class to compute
+    PSF_TRY(cudaMallocAsync(&sym, sizeof(int32_t) * (n_cls + 1), st));
     int dev = 0, sms = 148;
     rc = cudaGetDevice(&dev) != cudaSuccess ||
                  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess
@@ -911,7 +931,7 @@ extern "C" int psf_bin_spread_classes(const psf_scanner *scanner, const psf_tabl
     // the smallest class of each orbit through the spread kernel ...
     if (!rc)
         rc = bin_spread(scanner, desc, table, eta, class_lors, n_cls, half_t, half_a, norm,
-                        spread, sym, st);
+                        spread, sym, reinterpret_cast<unsigned *>(sym + n_cls), st);
     // ... the others as its images
     if (!rc) {
         PSF_TIMED("spread_mirror_kernel", st);
