@@ -2036,6 +2036,7 @@ namespace psf {
 
 // Images and windows the dense merge takes.
 static bool merge_ok(const Scan &sc, const Img &im, int half_t, int half_a) {
+    if (half_t < 0 || half_a < 0) return false;
     const int64_t E = (2 * (int64_t)half_t + 1) * (2 * (int64_t)half_a + 1);
     return (int64_t)im.nx * im.ny * im.nz <= 49152 && E * E <= 2401 &&
            (int64_t)sc.Nt * sc.NR <= 4096;
@@ -2316,7 +2317,7 @@ extern "C" int psf_psf_rows_workspace(const psf_scanner *scanner, const psf_imag
     if (rc) return rc;
     rc = make_img(image, &im);
     if (rc) return rc;
-    if (!bytes || n_lors < 0 || half_t < 0 || half_a < 0) return PSF_EINVAL;
+    if (!bytes || n_lors < 0) return PSF_EINVAL;
     if (!merge_ok(sc, im, half_t, half_a)) return PSF_EINVAL;
     const MergeSpace sp = merge_space(sc, im, n_lors);
     *bytes = n_lors > 0 && sp.total <= MERGE_SPACE_MAX ? (int64_t)sp.total : 0;
@@ -2334,9 +2335,7 @@ extern "C" int psf_psf_rows_merge(const psf_scanner *scanner, const psf_image *i
     if (rc) return rc;
     rc = make_img(image, &im);
     if (rc) return rc;
-    if (!nnz_out || !row_ptr || !lors || !spread || !workspace || n_lors < 1 || half_t < 0 ||
-        half_a < 0)
-        return PSF_EINVAL;
+    if (!nnz_out || !row_ptr || !lors || !spread || !workspace || n_lors < 1) return PSF_EINVAL;
     if (!merge_ok(sc, im, half_t, half_a)) return PSF_EINVAL;
     const MergeSpace sp = merge_space(sc, im, n_lors);
     if (sp.total > MERGE_SPACE_MAX || bytes < (int64_t)sp.total ||
