@@ -32,17 +32,26 @@ def sensitivity(matrix, n_rows: int, device="cuda"):
     return matrix.sensitivity(device=device)
 
 
+def _library_projections(matrix):
+    """Is it a psf.Matrix with the library's projections?  The one-call forms
+    (psf_mlem, psf_osem) project inside the library: an object of another type,
+    or one that brings its own forward or back (a normalisation, an attenuation),
+    goes step by step through its methods."""
+    return type(matrix) is psf.Matrix and vars(matrix).keys().isdisjoint(
+        ("forward", "forward_masked", "back", "back_sens", "sensitivity"))
+
+
 def mlem(matrix, y, iters: int = 10, x0=None, sens=None, graph: bool = False):
     """MLEM (Sec. 3): sens = A^T 1; x <- x * A^T(y / A x) / sens.
 
     Voxels with sens < 1e-12 * max(sens) are held at zero, and 0/0 in the
-    ratio is zero.  All steps are library kernels, enqueued by one call
-    (psf_mlem).  With graph=True the `iters` iterations (psf_forward,
+    ratio is zero.  All steps are library kernels, for a psf.Matrix enqueued by
+    one call (psf_mlem).  With graph=True the `iters` iterations (psf_forward,
     psf_em_ratio, psf_back, psf_em_update) are captured once in a CUDA graph
     (after one uncaptured iteration on a copy, which sets up the kernels' launch
     attributes) and replayed as one launch.
     """
-    if not graph:
+    if not graph and _library_projections(matrix):
         return matrix.mlem(y, iters, None if x0 is None else x0.clone(), sens)
     yhat = torch.empty_like(y)
     ratio = torch.empty_like(y)
@@ -75,6 +84,10 @@ def mlem(matrix, y, iters: int = 10, x0=None, sens=None, graph: bool = False):
         matrix.back(ratio, out=bp)
         psf.em_update(xi, bp, sens, floor)
 
+    if not graph:
+        for _ in range(iters):
+            iteration(x)
+        return x
     if iters == 0:
         return x
     iteration(x.clone())  # uncaptured warm-up on a scratch copy
@@ -99,14 +112,15 @@ def listmode_osem(matrix, rows, n_subsets: int, iters: int = 1, x0=None, sens=No
     Voxels with sens < 1e-12 * max(sens) are held at zero.  With top-N spreads
     and sparse_adjoint, the plan's transpose of S is built once so that S^T of
     a subset's counts and ratios scatters from their nonzero entries; subsets of
-    at most a sixteenth of the rows then go through psf_osem, which touches
-    LOR-space data only where the events are."""
+    at most a sixteenth of the rows then go through psf_osem (a psf.Matrix),
+    which touches LOR-space data only where the events are."""
     n_ev = rows.numel()
     if sparse_adjoint and matrix.topn > 0:
         matrix.build_sparse_adjoint()
     if sens is None:
         sens = matrix.sensitivity(device=rows.device)
-    if sparse_adjoint and matrix.topn > 0 and n_ev // n_subsets + 1 <= matrix.n_rows // 16:
+    if (sparse_adjoint and matrix.topn > 0 and _library_projections(matrix)
+            and n_ev // n_subsets + 1 <= matrix.n_rows // 16):
         return matrix.osem(rows, n_subsets, iters, sens, None if x0 is None else x0.clone())
     floor = 1e-12 * float(sens.max())
     if x0 is None:
