@@ -8,6 +8,7 @@ process has no GPU the calls raise.
 from __future__ import annotations
 
 import ctypes as C
+import operator
 import os
 import threading
 
@@ -597,8 +598,8 @@ class Matrix:
         sens = new(self.n_cols) if sens is None else sens
         # kept until the call returns: scratch of the enqueued iterations
         yhat, ratio, bp = new(self.n_rows), new(self.n_rows), new(self.n_cols)
-        _ok(lib().psf_mlem(self._h, _ptr(y), _ptr(x), _ptr(sens), given, int(iters), _ptr(yhat),
-                           _ptr(ratio), _ptr(bp), _stream()), "psf_mlem")
+        _ok(lib().psf_mlem(self._h, _ptr(y), _ptr(x), _ptr(sens), given, operator.index(iters),
+                           _ptr(yhat), _ptr(ratio), _ptr(bp), _stream()), "psf_mlem")
         return x
 
     def osem(self, rows, n_subsets: int, iters: int, sens, x=None):
@@ -610,9 +611,9 @@ class Matrix:
         x = x if have_x else new(self.n_cols)
         # kept until the call returns: scratch of the enqueued sub-iterations
         counts, lst, bp = new(self.n_rows), new(self.n_rows, torch.int32), new(self.n_cols)
-        _ok(lib().psf_osem(self._h, _ptr(rows), rows.numel(), int(n_subsets), int(iters), _ptr(x),
-                           int(have_x), _ptr(sens), _ptr(counts), _ptr(lst), _ptr(bp),
-                           _stream()), "psf_osem")
+        _ok(lib().psf_osem(self._h, _ptr(rows), rows.numel(), operator.index(n_subsets),
+                           operator.index(iters), _ptr(x), int(have_x), _ptr(sens), _ptr(counts),
+                           _ptr(lst), _ptr(bp), _stream()), "psf_osem")
         return x
 
     def __del__(self):

@@ -51,7 +51,7 @@ def mlem(matrix, y, iters: int = 10, x0=None, sens=None, graph: bool = False):
     (after one uncaptured iteration on a copy, which sets up the kernels' launch
     attributes) and replayed as one launch.
     """
-    if not graph and _library_projections(matrix):
+    if not graph and _library_projections(matrix) and iters >= 0:
         return matrix.mlem(y, iters, None if x0 is None else x0.clone(), sens)
     yhat = torch.empty_like(y)
     ratio = torch.empty_like(y)
@@ -120,7 +120,7 @@ def listmode_osem(matrix, rows, n_subsets: int, iters: int = 1, x0=None, sens=No
     if sens is None:
         sens = matrix.sensitivity(device=rows.device)
     if (sparse_adjoint and matrix.topn > 0 and _library_projections(matrix)
-            and n_ev // n_subsets + 1 <= matrix.n_rows // 16):
+            and iters >= 0 and n_subsets > 0 and n_ev // n_subsets + 1 <= matrix.n_rows // 16):
         return matrix.osem(rows, n_subsets, iters, sens, None if x0 is None else x0.clone())
     floor = 1e-12 * float(sens.max())
     if x0 is None:
