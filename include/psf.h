@@ -516,7 +516,10 @@ int psf_matrix_set_stencil_form(psf_matrix *m, int32_t form);
  * access, so any rows give the same result up to FP32 summation order.  Used
  * by default once declared where a pair's cells mostly fit
  * (psf_matrix_autotune times it against the other forms; psf_matrix_set_launch
- * switches psf_forward and psf_back to the launch it sets).  Host only; checks
+ * switches psf_forward and psf_back to the launch it sets).  A tuned choice is
+ * kept over later psf_matrix_set_spread(_topn) and psf_matrix_set_image calls and
+ * applies while the plan allows the form; otherwise the row launches run.  Host
+ * only; checks
  * the division constants it derives over the grid's range (PSF_EDEBUG if one
  * fails). */
 int psf_matrix_set_image(psf_matrix *m, const psf_image *image);

@@ -87,6 +87,7 @@ struct psf_matrix {
     unsigned img_zm;  // column / (nx * ny) = umulhi(column, img_zm) >> img_zk
     int img_zk;
     // is a direction (forward, back) pair-streamed: 0 where it fits, 1 no, 2 yes
+    // (where the plan allows it: a new spread or image may not)
     int stream_form[2];
 };
 
@@ -2773,13 +2774,15 @@ static int rows_pair_stream(const psf_matrix *m, const float *in, const float *i
     });
 }
 
-// Is a direction (0 forward, 1 back) pair-streamed: as timed, else where it fits.
+// Is a direction (0 forward, 1 back) pair-streamed: where the plan as it is now
+// allows it (the spreads or the image may be others than those it was timed
+// with), as timed, else where it fits.
 static bool use_pair_stream(const psf_matrix *m, int dir) {
-    if (m->stream_form[dir]) return m->stream_form[dir] == 2;
+    if (m->stream_form[dir] == 1) return false;
     PairGrid g{};
     int sms = 0;
     bool fits = false;
-    return pair_grid(m, 1, &g, &sms, &fits) && fits;
+    return pair_grid(m, 1, &g, &sms, &fits) && (m->stream_form[dir] == 2 || fits);
 }
 
 static int rows_fwd_with(const psf_matrix *m, const float *x, float *y, int chunk, int threads,
@@ -3632,18 +3635,19 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
                 m->wq_chunk = bc;
                 m->wq_threads = bt;
             }
-            // against the pair-streamed form, where the plan allows it
+            // against the pair-streamed form, where the plan allows it (a plan that
+            // allows it only later takes it where it fits)
             PairGrid sg{};
             int ssms = 0;
             bool sfits = false;
-            m->stream_form[dir] = 1;
+            m->stream_form[dir] = 0;
             if (pair_grid(m, 1, &sg, &ssms, &sfits)) {
                 for (int rep = 0; rep < 3 && !rc; ++rep) {
                     float ms = 0.0f;
                     if (cudaEventRecord(e0, st) != cudaSuccess) rc = PSF_ECUDA;
                     m->stream_form[dir] = 2;
                     if (!rc) rc = dir == 0 ? rows_fwd(m, x, y, st) : rows_back(m, y, x, st);
-                    m->stream_form[dir] = 1;
+                    m->stream_form[dir] = 1;  // the row launches, unless found slower
                     if (!rc && (cudaEventRecord(e1, st) != cudaSuccess ||
                                 cudaEventSynchronize(e1) != cudaSuccess ||
                                 cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
@@ -3683,7 +3687,7 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
             int bf = 0;
             for (int f = 1; f < 3; ++f)
                 if (best[f] < best[bf]) bf = f;
-            if (!rc) m->pair_form = bf == 0 ? 1 : forms[bf];
+            if (!rc) m->pair_form = bf == 0 && patch ? 1 : forms[bf];
         }
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
@@ -3876,15 +3880,15 @@ extern "C" int psf_back_sens(const psf_matrix *m, const float *y, float *x, floa
         int rc = rows_back(m, qa, sens, st);
         return rc ? rc : rows_back(m, qb, x, st);
     }
-    // pair form 0: the per-pair shared-memory kernel where the plan allows it,
-    // else the back projection's launch (form 1: that launch, kept by the
-    // autotuner)
+    // pair form 0: the pair-streamed kernel where it fits, -3: where the plan as
+    // it is now allows it, else the back projection's launch (form 1: that
+    // launch, kept by the autotuner)
     int form = m->pair_form;
-    if (form == 0) {
+    if (form == 0 || form == -3) {
         PairGrid g{};
         int sms = 0;
         bool fits = false;
-        form = pair_grid(m, 2, &g, &sms, &fits) && fits ? -3 : 0;
+        form = pair_grid(m, 2, &g, &sms, &fits) && (form == -3 || fits) ? -3 : 0;
     } else if (form == 1) {
         form = 0;
     }
