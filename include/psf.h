@@ -578,8 +578,11 @@ int psf_em_update(float *x, const float *bp, const float *sens, float floor, int
  * written to it; bit 1, x (device float [n_cols]) holds the start image, else it
  * starts from 1 on the voxels the scanner sees (the sensitivity then comes with
  * the first back-projection).  yhat, ratio (device float [n_rows]) and bp
- * (device float [n_cols]) are scratch.  The floor stays on the device: the call
- * does not synchronise. */
+ * (device float [n_cols]) are scratch.  The floor stays on the device, in yhat:
+ * the call does not synchronise.  With sens given, a plan without spreads (at any
+ * launch but the work queue's) is only read: calls on several streams or threads
+ * may share it, each with scratch of its own.  Other calls use the plan's scratch,
+ * as psf_forward, psf_back and psf_back_sens do then. */
 int psf_mlem(const psf_matrix *m, const float *y, float *x, float *sens, int32_t given,
              int32_t iters, float *yhat, float *ratio, float *bp, void *stream);
 
@@ -594,7 +597,8 @@ int psf_mlem(const psf_matrix *m, const float *y, float *x, float *sens, int32_t
  * [n_cols]).  Scratch: counts (device float [n_rows], cleared here), list (device
  * int32 [n_rows]), bp (device float [n_cols]).  Work in proportion to the
  * subset's events; PSF_EINVAL when a subset may have more events than the set has
- * rows (use the separate steps).  Does not synchronise. */
+ * rows (use the separate steps).  Uses the plan's scratch, as every projection of
+ * a plan with spreads does: one call at a time on a plan.  Does not synchronise. */
 int psf_osem(const psf_matrix *m, const int64_t *rows, int64_t n_events, int32_t n_subsets,
              int32_t iters, float *x, int32_t have_x, const float *sens, float *counts,
              int32_t *list, float *bp, void *stream);

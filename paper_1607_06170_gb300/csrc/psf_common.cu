@@ -172,8 +172,9 @@ __global__ void lorset_list_kernel(LorSet ls, int32_t *lors, bool classes) {
 }
 
 // ------------------------------------------------------------ MLEM steps
-__global__ void em_ratio_kernel(const float *__restrict__ y, const float *__restrict__ yh,
-                                float *__restrict__ r, int64_t n) {
+// (yh may be r: psf_mlem takes the ratio in place)
+__global__ void em_ratio_kernel(const float *__restrict__ y, const float *yh, float *r,
+                                int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         float d = yh[i];

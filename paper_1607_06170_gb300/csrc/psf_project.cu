@@ -3158,8 +3158,8 @@ extern "C" int psf_matrix_create(psf_matrix **out, int64_t n_rows, int64_t n_col
     m->tr_w = nullptr;
     m->tr_list = nullptr;
     m->tr_nz = nullptr;
-    // row counters [2], the status word, the stencil's pair counter and the
-    // key of the largest sensitivity, one allocation
+    // row counters [2], the status word, the stencil's pair counter and
+    // psf_osem's key of the largest sensitivity, one allocation
     if (cudaMalloc(&m->queue, 5 * sizeof(unsigned long long)) != cudaSuccess) {
         delete m;
         return PSF_ECUDA;
@@ -3972,7 +3972,12 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
     cudaStream_t st = as_stream(stream);
     const bool have_sens = given & 1, have_x = given & 2;
     const int64_t nv = m->n_cols, n = m->n_rows;
-    unsigned *key = reinterpret_cast<unsigned *>(m->queue + 4);
+    // The key of the largest sensitivity lives in the caller's scratch for as long
+    // as the iterations need it (the projection goes to `ratio` and becomes the
+    // ratio in place, so yhat is free): calls that share a plan on several streams
+    // each have their own.  A plan without rows has no such scratch.
+    unsigned *key = reinterpret_cast<unsigned *>(yhat);
+    if (n == 0) PSF_TRY(cudaMallocAsync(&key, sizeof(unsigned), st));
     const int vgrid = grid_for(nv, PJ_T), rgrid = grid_for(n * 32, PJ_T);
     // three launches an iteration for stored rows at the grid-stride launches
     // (a tuned plan keeps its own kernels)
@@ -3989,8 +3994,8 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
     };
     auto to_ratio = [&](bool ones) -> int {
         if (!fused) {
-            const int rc = psf_forward(m, x, yhat, stream);
-            return rc ? rc : psf_em_ratio(y, yhat, ratio, n, stream);
+            const int rc = psf_forward(m, x, ratio, stream);
+            return rc ? rc : psf_em_ratio(y, ratio, ratio, n, stream);
         }
         return dispatch_dtype(m->dtype, [&](auto tag) -> int {
             using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
@@ -4018,39 +4023,44 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
                       ones ? mlem_update_kernel<true> : mlem_update_kernel<false>, vgrid, x, factor,
                       bp, sens, key, nv, clear);
     };
-    int rc = PSF_OK;
-    if (!have_x && !have_sens && iters > 0) {
-        // first iteration from an image of ones: its forward projection equals
-        // that of ones on the voxels the scanner sees (the others' columns are
-        // zero), so A^T 1 comes with the first back-projection
-        if (fused) {
-            rc = to_ratio(true);
-            if (!rc) rc = back(true);
-            if (!rc) rc = sens_key(true);
-        } else {
-            {
-                PSF_TIMED("fill_kernel", st);
-                fill_kernel<<<vgrid, PJ_T, 0, st>>>(x, 1.0f, nv);
+    auto iterate = [&]() -> int {
+        int rc = PSF_OK;
+        if (!have_x && !have_sens && iters > 0) {
+            // first iteration from an image of ones: its forward projection equals
+            // that of ones on the voxels the scanner sees (the others' columns are
+            // zero), so A^T 1 comes with the first back-projection
+            if (fused) {
+                rc = to_ratio(true);
+                if (!rc) rc = back(true);
+                if (!rc) rc = sens_key(true);
+            } else {
+                {
+                    PSF_TIMED("fill_kernel", st);
+                    fill_kernel<<<vgrid, PJ_T, 0, st>>>(x, 1.0f, nv);
+                }
+                PSF_LAUNCHED();
+                rc = to_ratio(false);
+                if (!rc) rc = psf_back_sens(m, ratio, bp, sens, stream);
+                if (!rc) rc = sens_key(false);
             }
-            PSF_LAUNCHED();
-            rc = to_ratio(false);
-            if (!rc) rc = psf_back_sens(m, ratio, bp, sens, stream);
+            --iters;
+            if (!rc) rc = update(true, bp, fused && iters > 0);
+        } else {
+            if (!have_sens) rc = psf_sensitivity(m, sens, stream);
             if (!rc) rc = sens_key(false);
+            // 1 on the voxels the scanner sees; a given image stays as it is
+            if (!rc && !have_x) rc = update(true, sens, false);
+            if (!rc && fused && iters > 0) PSF_TRY(cudaMemsetAsync(bp, 0, sizeof(float) * nv, st));
         }
-        --iters;
-        if (!rc) rc = update(true, bp, fused && iters > 0);
-    } else {
-        if (!have_sens) rc = psf_sensitivity(m, sens, stream);
-        if (!rc) rc = sens_key(false);
-        // 1 on the voxels the scanner sees; a given image stays as it is
-        if (!rc && !have_x) rc = update(true, sens, false);
-        if (!rc && fused && iters > 0) PSF_TRY(cudaMemsetAsync(bp, 0, sizeof(float) * nv, st));
-    }
-    for (int it = 0; it < iters && !rc; ++it) {
-        rc = to_ratio(false);
-        if (!rc) rc = fused ? back(false) : psf_back(m, ratio, bp, stream);
-        if (!rc) rc = update(false, bp, fused && it + 1 < iters);
-    }
+        for (int it = 0; it < iters && !rc; ++it) {
+            rc = to_ratio(false);
+            if (!rc) rc = fused ? back(false) : psf_back(m, ratio, bp, stream);
+            if (!rc) rc = update(false, bp, fused && it + 1 < iters);
+        }
+        return rc;
+    };
+    const int rc = iterate();
+    if (n == 0) cudaFreeAsync(key, st);
     return rc;
 }
 
