@@ -64,11 +64,13 @@ __device__ __forceinline__ void tn_warp(float &s, float &c) {
 // do; those (a handful) rank themselves against each other.  Windows with more
 // than 32 such entries (ties, or no N positive pieces) and N above 32 take the
 // entries one after the other, each from the piece that holds the next.  Totals
-// and scale are pairs of FP32 numbers (FP64 beyond their range: the FP64 pipe
-// would cost more than all the rest).  RING3D, N = 5, 84,227 windows, 809 MB:
-// 0.27 ms (1.52 ms when every rank was another pass over the window in 64-bit
-// keys with a CTA barrier, 0.40 ms when each was taken from its piece in turn,
-// with FP64 totals).
+// and scale are pairs of FP32 numbers where no weight is negative (nothing
+// cancels, so they keep 2^-46 of the total, and total / kept is 1 .. EE / N) and
+// within FP32's range, else FP64 (whose pipe would cost more than all the rest).
+// RING3D, N = 5, 84,227 windows, 809 MB: 0.26 ms (1.52 ms when every rank was
+// another pass over the window in 64-bit keys with a CTA barrier, 0.40 ms when
+// each was taken from its piece in turn, with FP64 totals; the pieces' largest
+// weights as floats, not bits: 0.27 ms).
 __global__ void __launch_bounds__(TN_W * 32) topn_kernel(const float *__restrict__ spread,
                                                          int64_t n, int Wt, int Wa, int N,
                                                          int piece, int32_t *__restrict__ idx,
@@ -107,18 +109,24 @@ __global__ void __launch_bounds__(TN_W * 32) topn_kernel(const float *__restrict
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
-        // the lane's piece: its sum and its largest weight (0 for none positive)
+        // the lane's piece: its sum and its largest weight (0 for none positive), by
+        // the weights' bits, which order as they do unless one is negative (or not
+        // a number): then above infinity's, and that window's are compared again
         const float *mine = win + lane * piece;
         uint64_t s2 = 0, c2 = 0;
-        float bw = 0.0f;
+        unsigned top = __float_as_uint(mine[piece - 1]);
 #pragma unroll 4
         for (int j = 0; j + 1 < piece; j += 2) {
             const float w = mine[j], v = mine[j + 1];
             tn_add2(s2, c2, w, v);
-            bw = fmaxf(bw, fmaxf(w, v));
+            top = max(top, max(__float_as_uint(w), __float_as_uint(v)));
         }
-        bw = fmaxf(bw, mine[piece - 1]);
-        bw = bw > 0.0f ? bw : 0.0f;
+        const bool mixed = __any_sync(F, top > 0x7f800000u);
+        float bw = __uint_as_float(top);
+        if (mixed) {
+            bw = 0.0f;
+            for (int j = 0; j < piece; ++j) bw = fmaxf(bw, mine[j]);
+        }
         float s, c, sb, cb;
         asm("mov.b64 {%0, %1}, %2;" : "=f"(s), "=f"(sb) : "l"(s2));
         asm("mov.b64 {%0, %1}, %2;" : "=f"(c), "=f"(cb) : "l"(c2));
@@ -225,13 +233,12 @@ __global__ void __launch_bounds__(TN_W * 32) topn_kernel(const float *__restrict
         }
         __syncwarp();  // sel is complete
         // scale = total / kept, 1 when nothing was kept
-        const float as = fabsf(s), ak = fabsf(ks);
-        if (as > 1e-25f && as < 1e30f && ak > 1e-25f && ak < 1e30f) {
+        if (!mixed && s > 1e-25f && s < 1e30f && ks > 1e-25f && ks < 1e30f) {
             const float q = __fdiv_rn(s, ks);
             const float rem = fmaf(-q, ks, s) + fmaf(-q, kc, c);
             const float ql = __fdiv_rn(rem, ks);
             for (int k = lane; k < N; k += 32) wout[g * N + k] = fmaf(sel[k], q, sel[k] * ql);
-        } else {  // near or beyond the ends of FP32's range, or not a number
+        } else {  // a negative weight, an end of FP32's range, or not a number
             double all = 0.0, kept = 0.0;
             for (int e = lane; e < EE; e += 32) all += (double)win[e];
             all = warp_sum_d(all);
