@@ -282,11 +282,14 @@ int psf_sysmat_rows(const psf_scanner *scanner, const psf_image *image, const in
  *    image, window or scanner.
  *  psf_psf_rows_merge: merges the rows into the workspace (device, 16-byte
  *    aligned), writes row_ptr and *nnz_out (host); synchronises `stream` once.
- *    PSF_ECAPACITY when the merged rows do not fit the workspace.
+ *    PSF_ECAPACITY when the merged rows do not fit the workspace (use
+ *    psf_sysmat_rows: the workspace then lacks the rows that found no room).
  *  psf_psf_rows_emit: writes col, val and row_scale (dtype as in
  *    psf_sysmat_rows; room for *nnz_out entries) from that workspace and
  *    row_ptr, after a psf_psf_rows_merge of the same scanner, image and n_lors
- *    on the same stream.  Does not synchronise.
+ *    on the same stream that returned PSF_OK (after PSF_ECAPACITY the rows that
+ *    found no room are left unwritten).  PSF_EINVAL for an image, scanner or
+ *    n_lors that psf_psf_rows_merge refuses.  Does not synchronise.
  */
 int psf_psf_rows_workspace(const psf_scanner *scanner, const psf_image *image, int64_t n_lors,
                            int32_t half_t, int32_t half_a, int64_t *bytes);

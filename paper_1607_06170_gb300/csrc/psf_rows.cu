@@ -930,7 +930,8 @@ __global__ void __launch_bounds__(256) merge_kernel(Scan sc, int nvox, const int
 }
 
 // Merged rows from where the merge put them to the CSR arrays, in the value
-// format: a warp per row.
+// format: a warp per row.  (A row that found no room, off < 0, has no entries to
+// write.)
 template <typename VT>
 __global__ void __launch_bounds__(256) merge_emit_kernel(
     int64_t n, const int64_t *__restrict__ row_ptr, const int64_t *__restrict__ off,
@@ -941,7 +942,7 @@ __global__ void __launch_bounds__(256) merge_emit_kernel(
     for (int64_t m = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); m < n;
          m += (int64_t)gridDim.x * 8) {
         const int64_t a = row_ptr[m], from = off[m];
-        const int len = (int)(row_ptr[m + 1] - a);
+        const int len = from < 0 ? 0 : (int)(row_ptr[m + 1] - a);
         float inv = 1.0f;
         if (row_scale) {
             const float scale = rmax[m] > 0.0f ? rmax[m] : 1.0f;
@@ -2359,9 +2360,12 @@ extern "C" int psf_psf_rows_emit(const psf_scanner *scanner, const psf_image *im
     if (n_lors < 1 || !row_ptr || !workspace || !col || !val) return PSF_EINVAL;
     if (dtype < PSF_F32 || dtype > PSF_F16) return PSF_EINVAL;
     if ((dtype == PSF_F32) != (row_scale == nullptr)) return PSF_EINVAL;
-    return merge_emit(merge_space(sc, im, n_lors),
-                      static_cast<const unsigned char *>(workspace), n_lors, dtype, row_ptr, col,
-                      val, row_scale, as_stream(stream));
+    if (!merge_ok(sc, im, 0, 0)) return PSF_EINVAL;  // (of any window)
+    const MergeSpace sp = merge_space(sc, im, n_lors);
+    if (sp.total > MERGE_SPACE_MAX || (reinterpret_cast<uintptr_t>(workspace) & 15))
+        return PSF_EINVAL;
+    return merge_emit(sp, static_cast<const unsigned char *>(workspace), n_lors, dtype, row_ptr,
+                      col, val, row_scale, as_stream(stream));
 }
 
 // ------------------------------------------------ no-allocation entry point

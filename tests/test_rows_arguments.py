@@ -32,3 +32,19 @@ def test_psf_rows_refuse_windows(L, half):
     assert lib.psf_psf_rows_workspace(s, i, 5, *half, C.byref(room)) == EINVAL
     assert lib.psf_psf_rows_merge(s, i, DEV, 5, DEV, *half, DEV, DEV, 1 << 30, C.byref(nnz),
                                   None) == EINVAL
+
+
+@pytest.mark.parametrize("nx,rings,n", [(64, 1, 1 << 22), (256, 1, 5), (64, 80, 5)])
+def test_psf_rows_emit_refuses_what_merge_refuses(L, nx, rings, n):
+    """A list too long for a workspace, an image of too many voxels, a scanner of
+    too many crystals."""
+    w = I.workload("RING2D")
+    sc = L.scanner(dict(w["scanner"], na_block=rings))
+    im = L.image(I.image(nx, nx, 1, 1.0, 1.0, 1.0))
+    s, i, nnz, room = C.byref(sc), C.byref(im), C.c_int64(), C.c_int64(-1)
+    lib = L.lib()
+    rc = lib.psf_psf_rows_workspace(s, i, n, 3, 0, C.byref(room))
+    assert rc == EINVAL or (rc == 0 and room.value == 0)
+    assert lib.psf_psf_rows_merge(s, i, DEV, n, DEV, 3, 0, DEV, DEV, 1 << 40, C.byref(nnz),
+                                  None) == EINVAL
+    assert lib.psf_psf_rows_emit(s, i, n, L.PSF_F32, DEV, DEV, DEV, DEV, None, None) == EINVAL
