@@ -454,9 +454,9 @@ int psf_matrix_destroy(psf_matrix *m);
  * and, where psf_matrix_set_image allows it, the pair-streamed form,
  * on all-ones vectors, and keeps the fastest for psf_forward / psf_back of
  * this plan (chunk_out / threads_out name the fastest of the others); the pair
- * back-projection of psf_back_sens takes the faster of
- * the back launch and the bulk-staged kernel (psf_back keeps launches that
- * skip rows with y = 0, which a bulk-staged pass cannot); for a
+ * back-projection of psf_back_sens takes the fastest of the back launch, the
+ * bulk-staged kernel (not a choice of psf_back: it cannot skip rows with y = 0)
+ * and the forms by transaxial pair that psf_matrix_set_image allows; for a
  * factored plan with full-window spreads it also times the staged forms of the
  * LOR-space spread stencil in each direction and keeps the fastest (call it after
  * psf_matrix_set_spread; the candidates are forms 3, 4 and, when it fits, 5).
@@ -517,8 +517,10 @@ int psf_matrix_set_stencil_form(psf_matrix *m, int32_t form);
  * cells are read from its direct-plane row of the middle ring; an entry whose
  * voxel is not among them, or past the shared-memory capacity, takes the global
  * access, so any rows give the same result up to FP32 summation order.  Used
- * by default once declared where a pair's cells mostly fit
- * (psf_matrix_autotune times it against the other forms; psf_matrix_set_launch
+ * by default once declared where a pair's cells mostly fit beside a table of a
+ * byte per (x, y); psf_back_sens on wider images finds the cells by their y rows
+ * instead (psf_matrix_autotune times them against the other forms;
+ * psf_matrix_set_launch
  * switches psf_forward and psf_back to the launch it sets).  A tuned choice is
  * kept over later psf_matrix_set_spread(_topn) and psf_matrix_set_image calls and
  * applies while the plan allows the form; otherwise the row launches run.  Host

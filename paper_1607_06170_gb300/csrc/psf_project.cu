@@ -82,10 +82,13 @@ struct psf_matrix {
     psf::Img otf_im;
     psf::LorSet otf_ls;
     // the voxel grid of the columns (psf_matrix_set_image); enables the
-    // pair-streamed projections (psf_back_sens: pair form -3)
+    // pair-streamed projections (psf_back_sens: pair form -3) and the pair back-
+    // projection of wide images (pair form -4)
     int img_nx, img_ny, img_nz;
     unsigned img_zm;  // column / (nx * ny) = umulhi(column, img_zm) >> img_zk
     int img_zk;
+    unsigned dv_xy_m, dv_x_m;  // the multiply-shift forms of the divisions by
+    int dv_xy_k, dv_x_k;       // nx * ny and nx over the grid's own range
     // is a direction (forward, back) pair-streamed: 0 where it fits, 1 no, 2 yes
     // (where the plan allows it: a new spread or image may not)
     int stream_form[2];
@@ -2711,22 +2714,37 @@ static int bk_table(psf_matrix *m, cudaStream_t st) {
 
 }  // namespace psf
 
+#include "psf_pair_runs.cuh"
 #include "psf_pair_stream.cuh"
 
 namespace psf {
 
-// The pair-streamed form of a plan (a factored plan over the full set with its
-// image declared): its grid, and whether a pair's cells mostly fit -- the longest
-// side of the image -- so that it is the default.
-static bool pair_grid(const psf_matrix *m, int vectors, PairGrid *g, int *sms, bool *fits) {
+// Does the plan allow the projections by transaxial pair (a factored plan over the
+// full set with its image declared)?  With the device's SMs and shared memory.
+static bool pair_plan(const psf_matrix *m, int *sms, int *optin) {
     if (!m->factored || m->topn > 0 || m->otf || m->img_nz <= 0 || m->n_rows == 0) return false;
     if (m->n_rows != m->ls.ntp * m->ls.nrp) return false;
-    int dev = 0, optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-            cudaSuccess)
-        return false;
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
+               cudaSuccess;
+}
+
+// The ring pair whose row lists a transaxial pair's cells: the direct plane of the
+// middle ring.
+static int pair_cell_row(const LorSet &ls) {
+    const int rm = ls.NR / 2;
+    int64_t jm = 0;
+    for (int r = 0; r < rm; ++r) jm += ls.rp_count(r);
+    return (int)(jm + (rm - ls.rp_lo(rm)));
+}
+
+// The pair-streamed form of a plan: its grid, and whether a pair's cells mostly
+// fit -- the longest side of the image -- so that it is the default.
+static bool pair_grid(const psf_matrix *m, int vectors, PairGrid *g, int *sms, bool *fits) {
+    int optin = 0;
+    if (!pair_plan(m, sms, &optin)) return false;
     const int64_t nxy = (int64_t)m->img_nx * m->img_ny;
     if (nxy < 4 || nxy > optin || m->n_cols >= (1ll << 30)) return false;
     g->nx = m->img_nx;
@@ -2736,13 +2754,58 @@ static bool pair_grid(const psf_matrix *m, int vectors, PairGrid *g, int *sms, b
     g->nrp = (int)m->ls.nrp;
     g->zm = m->img_zm;
     g->zk = m->img_zk;
-    const int rm = m->ls.NR / 2;  // the direct-plane row of the middle ring lists the cells
-    int64_t jm = 0;
-    for (int r = 0; r < rm; ++r) jm += m->ls.rp_count(r);
-    g->jm = (int)(jm + (rm - m->ls.rp_lo(rm)));
+    g->jm = pair_cell_row(m->ls);
     if (!pair_layout(*g, vectors, (size_t)optin - 256)) return false;  // + static shared memory
     *fits = g->cap >= g->nx && g->cap >= g->ny;
     return true;
+}
+
+// The pair back-projection of wide images: its grid and shared memory.
+static bool runs_grid(const psf_matrix *m, RunsGrid *g, int *sms, size_t *shm) {
+    int optin = 0;
+    if (!pair_plan(m, sms, &optin)) return false;
+    g->nx = m->img_nx;
+    g->ny = m->img_ny;
+    g->nz = m->img_nz;
+    g->nxy = m->img_nx * m->img_ny;
+    g->dxy.m = m->dv_xy_m;
+    g->dxy.k = m->dv_xy_k;
+    g->dx.m = m->dv_x_m;
+    g->dx.k = m->dv_x_k;
+    g->jm = pair_cell_row(m->ls);
+    g->cap = 0;
+    const size_t fixed = runs_smem_bytes(*g, (int)m->ls.nrp) + 512;  // + static shared memory
+    if ((size_t)optin <= fixed) return false;
+    const size_t cell = sizeof(float2) * (size_t)g->nz + sizeof(int);
+    const size_t cap = ((size_t)optin - fixed) / cell / 4 * 4;
+    g->cap = cap < 32767 ? (int)cap : 32764;  // a cell index and a run length in 16 bits
+    *shm = runs_smem_bytes(*g, (int)m->ls.nrp);
+    return g->cap >= 32;
+}
+
+// How psf_back_sens back-projects a pair when nothing was timed: streamed where a
+// pair's cells fit beside the byte table, by y rows where the table takes their
+// room (both sides measured at csr_back_pair_runs_kernel), else 0, row by row.
+static int default_pair_form(const psf_matrix *m) {
+    PairGrid g{};
+    RunsGrid r{};
+    int sms = 0;
+    size_t shm = 0;
+    bool fits = false;
+    if (pair_grid(m, 2, &g, &sms, &fits) && fits) return -3;
+    return runs_grid(m, &r, &sms, &shm) ? -4 : 0;
+}
+
+// Does the plan as it is now allow a pair form that was timed on it earlier?
+static bool pair_form_ok(const psf_matrix *m, int form) {
+    PairGrid g{};
+    RunsGrid r{};
+    int sms = 0;
+    size_t shm = 0;
+    bool fits = false;
+    return form == -3   ? pair_grid(m, 2, &g, &sms, &fits)
+           : form == -4 ? runs_grid(m, &r, &sms, &shm)
+                        : true;
 }
 
 // One pair-streamed projection (the outputs of the back-projections are added
@@ -3599,6 +3662,7 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
         if (!rc) {
             fill_kernel<<<grid_for(m->n_cols, 256), 256, 0, st>>>(x, 1.0f, m->n_cols);
             fill_kernel<<<grid_for(m->n_rows, 256), 256, 0, st>>>(y, 1.0f, m->n_rows);
+            fill_kernel<<<grid_for(m->n_rows, 256), 256, 0, st>>>(m->q, 1.0f, m->n_rows);
             if (cudaGetLastError() != cudaSuccess) rc = PSF_ECUDA;
         }
         for (int dir = 0; dir < 2 && !rc; ++dir) {
@@ -3660,23 +3724,20 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
                 if (!rc && bc == -4) m->stream_form[dir] = 2;
             }
         }
-        // the pair back-projection of psf_back_sens: the back launch or the
-        // bulk-staged kernel (the single back keeps the row-skipping launches:
-        // a bulk-staged pass streams every chunk whatever y holds)
+        // the pair back-projection of psf_back_sens: the back launch, the
+        // bulk-staged kernel (not for the single back: it streams every chunk
+        // whatever y holds) or a form by transaxial pair
         m->pair_form = 0;
-        PairGrid pg{};
-        int psms = 0;
-        bool pfits = false;
-        const bool patch = pair_grid(m, 2, &pg, &psms, &pfits);
+        const bool patch = pair_form_ok(m, -3) || pair_form_ok(m, -4);
         if ((bulk || patch) && !rc) {
-            const int forms[3] = {0, -2, -3};
-            float best[3] = {1e30f, 1e30f, 1e30f};
-            for (int f = 0; f < 3 && !rc; ++f) {
-                if ((f == 1 && !bulk) || (f == 2 && !patch)) continue;
+            const int forms[4] = {0, -2, -3, -4};
+            float best[4] = {1e30f, 1e30f, 1e30f, 1e30f};
+            for (int f = 0; f < 4 && !rc; ++f) {
+                if ((f == 1 && !bulk) || !pair_form_ok(m, forms[f])) continue;
                 for (int rep = 0; rep < 3 && !rc; ++rep) {
                     float ms = 0.0f;
                     if (cudaEventRecord(e0, st) != cudaSuccess) rc = PSF_ECUDA;
-                    if (!rc) rc = rows_back_pair(m, y, y, forms[f], st);
+                    if (!rc) rc = rows_back_pair(m, y, m->q, forms[f], st);
                     if (!rc && (cudaEventRecord(e1, st) != cudaSuccess ||
                                 cudaEventSynchronize(e1) != cudaSuccess ||
                                 cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
@@ -3685,7 +3746,7 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
                 }
             }
             int bf = 0;
-            for (int f = 1; f < 3; ++f)
+            for (int f = 1; f < 4; ++f)
                 if (best[f] < best[bf]) bf = f;
             if (!rc) m->pair_form = bf == 0 && patch ? 1 : forms[bf];
         }
@@ -3757,6 +3818,20 @@ extern "C" int psf_matrix_set_image(psf_matrix *m, const psf_image *image) {
     for (int64_t z = 0; z < im.nz && l >= 2; ++z)
         for (int64_t n = z * nxy; n < nv && n <= (z + 1) * nxy - 1; n += nxy > 1 ? nxy - 1 : 1)
             if ((int64_t)(((unsigned long long)n * zm) >> (30 + l)) != z) return PSF_EDEBUG;
+    const DivMagic a = div_magic((unsigned)nxy, (unsigned long long)nv),
+                   b = div_magic((unsigned)im.nx, (unsigned long long)nxy);
+    if (nv <= (1ll << 26)) {  // (checked at the quotients' steps, as above)
+        for (int64_t z = 0; z < im.nz; ++z)
+            if (a.div((unsigned)(z * nxy)) != z || a.div((unsigned)((z + 1) * nxy - 1)) != z)
+                return PSF_EDEBUG;
+        for (int64_t y = 0; y < im.ny; ++y)
+            if (b.div((unsigned)(y * im.nx)) != y || b.div((unsigned)((y + 1) * im.nx - 1)) != y)
+                return PSF_EDEBUG;
+    }
+    m->dv_xy_m = a.m;
+    m->dv_xy_k = a.k;
+    m->dv_x_m = b.m;
+    m->dv_x_k = b.k;
     m->img_zm = (unsigned)zm;
     m->img_zk = l - 2;
     m->img_nx = im.nx;
@@ -3880,18 +3955,11 @@ extern "C" int psf_back_sens(const psf_matrix *m, const float *y, float *x, floa
         int rc = rows_back(m, qa, sens, st);
         return rc ? rc : rows_back(m, qb, x, st);
     }
-    // pair form 0: the pair-streamed kernel where it fits, -3: where the plan as
-    // it is now allows it, else the back projection's launch (form 1: that
-    // launch, kept by the autotuner)
+    // the form that was timed (1: the back projection's launch), where the plan as
+    // it is now allows it; nothing timed, or that form refused: the default
     int form = m->pair_form;
-    if (form == 0 || form == -3) {
-        PairGrid g{};
-        int sms = 0;
-        bool fits = false;
-        form = pair_grid(m, 2, &g, &sms, &fits) && (form == -3 || fits) ? -3 : 0;
-    } else if (form == 1) {
-        form = 0;
-    }
+    if (form == 0 || !pair_form_ok(m, form)) form = default_pair_form(m);
+    if (form == 1) form = 0;
     int rc = rows_back_pair(m, qa, qb, form, st);
     if (rc) return rc;
     {
@@ -3904,14 +3972,39 @@ extern "C" int psf_back_sens(const psf_matrix *m, const float *y, float *x, floa
 
 namespace psf {
 
-// img2 = A^T (qa, qb) as an interleaved pair: form -3 the pair-streamed
-// kernel, -2 the bulk-staged kernel, else the pair kernel at
+// The pair back-projection of wide images, into img2 (cleared by the caller).
+static int rows_back_runs(const psf_matrix *m, const float *qa, const float *qb,
+                          cudaStream_t st) {
+    RunsGrid g{};
+    int sms = 0;
+    size_t shm = 0;
+    if (!runs_grid(m, &g, &sms, &shm)) return PSF_EINVAL;
+    PSF_TRY(cudaMemsetAsync(m->queue + 3, 0, sizeof(unsigned long long), st));  // pair counter
+    return dispatch_dtype(m->dtype, [&](auto tag) -> int {
+        using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
+        PSF_TRY(cudaFuncSetAttribute(csr_back_pair_runs_kernel<VT>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        const int grid = (int)(m->ls.ntp < sms ? m->ls.ntp : sms);
+        {
+            PSF_TIMED("csr_back_pair_runs_kernel", st);
+            csr_back_pair_runs_kernel<VT><<<grid, PR_T, shm, st>>>(
+                m->ls.ntp, (int)m->ls.nrp, m->row_ptr, m->col, (const VT *)m->val,
+                m->row_scale, qa, qb, m->img2, m->queue + 3, g);
+        }
+        PSF_LAUNCHED();
+        return PSF_OK;
+    });
+}
+
+// img2 = A^T (qa, qb) as an interleaved pair: form -3 the pair-streamed kernel,
+// -4 the one for wide images, -2 the bulk-staged kernel, else the pair kernel at
 // the back projection's launch.
 static int rows_back_pair(const psf_matrix *m, const float *qa, const float *qb, int form,
                           cudaStream_t st) {
     PSF_TRY(cudaMemsetAsync(m->img2, 0, sizeof(float2) * m->n_cols, st));
     if (m->otf) return PSF_EINVAL;  // psf_back_sens traces twice instead
     if (form == -3) return rows_pair_stream<PS_PAIR>(m, qa, qb, nullptr, m->img2, st);
+    if (form == -4) return rows_back_runs(m, qa, qb, st);
     if (form == -2) {
         if (!m->bk_first) return PSF_EINVAL;
         int grid = 0;
