@@ -516,17 +516,19 @@ int psf_matrix_set_stencil_form(psf_matrix *m, int32_t form);
  * voxel on the 3D ring), instead of one global access per entry.  The pair's
  * cells are read from its direct-plane row of the middle ring; an entry whose
  * voxel is not among them, or past the shared-memory capacity, takes the global
- * access, so any rows give the same result up to FP32 summation order.  Used
- * by default once declared where a pair's cells mostly fit beside a table of a
- * byte per (x, y); psf_back_sens on wider images finds the cells by their y rows
- * instead (psf_matrix_autotune times them against the other forms;
- * psf_matrix_set_launch
- * switches psf_forward and psf_back to the launch it sets).  A tuned choice is
- * kept over later psf_matrix_set_spread(_topn) and psf_matrix_set_image calls and
- * applies while the plan allows the form; otherwise the row launches run.  Host
- * only; checks
- * the division constants it derives over the grid's range (PSF_EDEBUG if one
- * fails). */
+ * access, so any rows give the same result up to FP32 summation order.  Used by
+ * default once declared where a pair's cells mostly fit beside a table of a byte
+ * per (x, y); psf_back_sens on wider images finds the cells by their y rows
+ * instead.  psf_matrix_autotune times these forms against the others;
+ * psf_matrix_set_launch switches psf_forward and psf_back to the launch it sets.
+ * A tuned choice is kept over later psf_matrix_set_spread(_topn) and
+ * psf_matrix_set_image calls and applies while the plan allows the form; otherwise
+ * the row launches run.  Where psf_back works by pairs, a plan of 2^20 rows or more
+ * goes row by row, past the rows with value 0, when at most about 5/8 of the
+ * LOR-space values are nonzero (a sample on the device decides, so the calls stay
+ * capturable); otherwise a pair with any nonzero value is read whole.
+ * Host only; checks the division constants it derives over the grid's range
+ * (PSF_EDEBUG if one fails). */
 int psf_matrix_set_image(psf_matrix *m, const psf_image *image);
 
 /*
