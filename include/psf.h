@@ -523,9 +523,9 @@ int psf_matrix_set_stencil_form(psf_matrix *m, int32_t form);
  * psf_matrix_set_launch switches psf_forward and psf_back to the launch it sets.
  * A tuned choice is kept over later psf_matrix_set_spread(_topn) and
  * psf_matrix_set_image calls and applies while the plan allows the form; otherwise
- * the row launches run.  Where psf_back works by pairs, a plan of 2^20 rows or more
- * goes row by row, past the rows with value 0, when at most about 5/8 of the
- * LOR-space values are nonzero (a sample on the device decides, so the calls stay
+ * the row launches run.  Where psf_back works by pairs, a plan of 2^21 rows or more
+ * goes row by row, past the rows with value 0, when about half of its entries or
+ * less are in the others (a sample on the device decides, so the calls stay
  * capturable); otherwise a pair with any nonzero value is read whole.
  * Host only; checks the division constants it derives over the grid's range
  * (PSF_EDEBUG if one fails). */

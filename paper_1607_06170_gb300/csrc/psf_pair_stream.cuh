@@ -131,8 +131,8 @@ __global__ void __launch_bounds__(PsShape<MODE>::T, 1) pair_stream_kernel(
     const VT *__restrict__ val, const float *__restrict__ scale, const float *__restrict__ in,
     const float *__restrict__ in2, float *__restrict__ out, float2 *__restrict__ out2,
     unsigned long long *ctr, int *status, long long limit, PairGrid g,
-    const unsigned long long *nz, int64_t few) {
-    if (MODE == PS_BACK && nz && (int64_t)*nz <= few) return;  // the work queue has it
+    const unsigned long long *sparse) {
+    if (MODE == PS_BACK && sparse && *sparse) return;  // the work queue has it
     extern __shared__ __align__(128) unsigned char rg_raw[];
     constexpr int NV = MODE == PS_PAIR ? 2 : 1;
     constexpr int PS_W = PsShape<MODE>::W, PS_U = PsShape<MODE>::U, PS_B = PsShape<MODE>::B,

@@ -265,11 +265,11 @@ __global__ void csr_back_wq_kernel(int64_t n, const int64_t *__restrict__ ptr,
                                    const int32_t *__restrict__ col, const VT *__restrict__ val,
                                    const float *__restrict__ scale, const float *__restrict__ y,
                                    float *__restrict__ x, unsigned long long *queue, int chunk,
-                                   const unsigned long long *nz = nullptr, int64_t nz_lo = 0,
-                                   int64_t nz_hi = 0) {
+                                   const unsigned long long *listed = nullptr,
+                                   const unsigned long long *sparse = nullptr) {
     const int lane = threadIdx.x & 31;
-    // another form has it when the count of nonzero rows is not in [nz_lo, nz_hi]
-    if (nz && ((int64_t)*nz < nz_lo || (int64_t)*nz > nz_hi)) return;
+    if (listed && *listed <= (unsigned long long)(n >> 2)) return;  // the list form has it
+    if (sparse && !*sparse) return;                                  // the stream has it
     for (int64_t r0 = wq_take(queue, chunk, lane); r0 < n; r0 = wq_take(queue, chunk, lane)) {
         const int64_t r1 = r0 + chunk < n ? r0 + chunk : n;
         // 32 rows at a time: values and extents loaded one per lane, rows with
@@ -349,22 +349,37 @@ __global__ void mask_rows4_kernel(const float *__restrict__ mask, int64_t n,
     }
 }
 
-// How many of NZ_N values spread over q [n] are not 0 (a choice of kernel hangs on
-// it, never a result): one CTA, about 3 us.
-constexpr int NZ_T = 1024, NZ_N = 8 * NZ_T;
+// Do at most half of the stored entries lie in rows with q != 0?  From NZ_T rows
+// spread over the plan (a choice of kernel hangs on it, never a result), into
+// state[0]; the counters state[1] and state[3] of the kernels that follow become 0.
+// One CTA and a row per thread: bound by the latency of the loads (4,096 rows cost
+// 4 us more).
+constexpr int NZ_T = 1024;
 
-__global__ void __launch_bounds__(NZ_T) sample_nonzero_kernel(const float *__restrict__ q,
-                                                              int64_t n, unsigned long long *nz) {
-    float v[NZ_N / NZ_T];
-#pragma unroll
-    for (int u = 0; u < NZ_N / NZ_T; ++u) {  // multiples of the golden ratio, mod 1, times n
-        const uint64_t k = (uint64_t)(u * NZ_T + (int)threadIdx.x) * 0x9e3779b97f4a7c15ull;
-        v[u] = q[__umul64hi(k, (uint64_t)n)];
+__global__ void __launch_bounds__(NZ_T) sample_sparse_kernel(const float *__restrict__ q,
+                                                             const int64_t *__restrict__ ptr,
+                                                             int64_t n, unsigned long long *state) {
+    __shared__ unsigned long long all, on;
+    if (threadIdx.x == 0) all = on = 0;
+    __syncthreads();
+    // multiples of the golden ratio, mod 1, times n
+    const uint64_t k = (uint64_t)threadIdx.x * 0x9e3779b97f4a7c15ull;
+    const int64_t r = (int64_t)__umul64hi(k, (uint64_t)n);
+    const float v = q[r];
+    int64_t a = ptr[r + 1] - ptr[r], b = v != 0.0f ? a : 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    int c = 0;
-#pragma unroll
-    for (int u = 0; u < NZ_N / NZ_T; ++u) c += __syncthreads_count(v[u] != 0.0f);
-    if (threadIdx.x == 0) *nz = (unsigned long long)c;
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&all, (unsigned long long)a);
+        atomicAdd(&on, (unsigned long long)b);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        state[0] = 2 * on <= all;
+        state[1] = state[3] = 0;
+    }
 }
 
 // List the rows with mask != 0 into list, their number into *count (which
@@ -2829,16 +2844,18 @@ static bool pair_form_ok(const psf_matrix *m, int form) {
 }
 
 // One pair-streamed projection (the outputs of the back-projections are added
-// to: the caller clears them).  nz: nothing when *nz <= few.
+// to: the caller clears them).  sparse: after sample_sparse_kernel, nothing when it
+// said so.
 template <int MODE>
 static int rows_pair_stream(const psf_matrix *m, const float *in, const float *in2, float *out,
                             float2 *out2, cudaStream_t st,
-                            const unsigned long long *nz = nullptr, int64_t few = 0) {
+                            const unsigned long long *sparse = nullptr) {
     PairGrid g{};
     int sms = 0;
     bool fits = false;
     if (!pair_grid(m, MODE == PS_PAIR ? 2 : 1, &g, &sms, &fits)) return PSF_EINVAL;
-    PSF_TRY(cudaMemsetAsync(m->queue + 3, 0, sizeof(unsigned long long), st));  // pair counter
+    if (!sparse)  // the pair counter
+        PSF_TRY(cudaMemsetAsync(m->queue + 3, 0, sizeof(unsigned long long), st));
     return dispatch_dtype(m->dtype, [&](auto tag) -> int {
         using VT = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
         PSF_TRY(cudaFuncSetAttribute(pair_stream_kernel<VT, MODE>,
@@ -2851,7 +2868,7 @@ static int rows_pair_stream(const psf_matrix *m, const float *in, const float *i
                       st);
             pair_stream_kernel<VT, MODE><<<grid, PsShape<MODE>::T, g.bytes, st>>>(
                 m->ls.ntp, m->row_ptr, m->col, (const VT *)m->val, m->row_scale, in, in2, out,
-                out2, m->queue + 3, m->status, (long long)wait_limit(), g, nz, few);
+                out2, m->queue + 3, m->status, (long long)wait_limit(), g, sparse);
         }
         PSF_LAUNCHED();
         return PSF_OK;
@@ -2979,22 +2996,21 @@ static int rows_fwd(const psf_matrix *m, const float *x, float *y, cudaStream_t 
 }
 
 // x += G^T y, pair-streamed; on large plans by the work queue, which skips rows
-// with y = 0, when at most 5/8 of the values are not 0 (a subset's events): the
-// stream reads all of a pair for one of them.  RING3D, FP32 (BF16), work queue
-// (tuned) against stream in ms: no value 0.47 against 0.90 (0.48, 0.96), 4.5 % of
-// the rows 1.19 against 6.71 (1.18, 6.65), 34 % 3.9 against 7.05 (3.7, 7.00), 58 %
-// about 6 and 67 % about 7 against 7.1 (6.6, 7.07), all 13.45 against 7.15 (12.45,
-// 7.09).  The sample and the launch that returns at once cost 14 us a call, so
-// plans whose pass takes less than about 0.2 ms are streamed without.
-constexpr int64_t NZ_ROWS = 1 << 20;
-constexpr int NZ_FEW = NZ_N * 5 / 8;
+// with y = 0, when about half of the entries or less are in the others (a subset's
+// events): the stream reads all of a pair for one of them.  RING3D, FP32 (BF16),
+// work queue (tuned) against stream in ms: no value 0.47 against 0.90 (0.48, 0.96),
+// 1e5 events 1.19 against 6.71 (1.18, 6.65), 1e6 3.9 against 7.05 (3.7, 7.00), 3e6,
+// half of the entries, 7.07 against 7.12 (6.6, 7.07), all 13.45 against 7.15
+// (12.45, 7.09).  The sample and the launch that returns at once cost 9 us a
+// call, so smaller plans are streamed without.
+constexpr int64_t NZ_ROWS = 1 << 21;
 
 static int rows_back_stream(const psf_matrix *m, const float *y, float *x, cudaStream_t st) {
     if (m->n_rows < NZ_ROWS)
         return rows_pair_stream<PS_BACK>(m, y, nullptr, x, nullptr, st);
     {
-        PSF_TIMED("sample_nonzero_kernel", st);
-        sample_nonzero_kernel<<<1, NZ_T, 0, st>>>(y, m->n_rows, m->queue);
+        PSF_TIMED("sample_sparse_kernel", st);
+        sample_sparse_kernel<<<1, NZ_T, 0, st>>>(y, m->row_ptr, m->n_rows, m->queue);
     }
     PSF_LAUNCHED();
     const int chunk = m->wq_chunk > 0 ? m->wq_chunk : 64;
@@ -3004,18 +3020,16 @@ static int rows_back_stream(const psf_matrix *m, const float *y, float *x, cudaS
         int grid = 0;
         const int rc = wq_grid(csr_back_wq_kernel<VT>, threads, &grid);
         if (rc) return rc;
-        PSF_TRY(cudaMemsetAsync(m->queue + 1, 0, sizeof(unsigned long long), st));
         {
             PSF_TIMED("csr_back_wq_kernel", st);
             csr_back_wq_kernel<VT><<<grid, threads, 0, st>>>(
                 m->n_rows, m->row_ptr, m->col, (const VT *)m->val, m->row_scale, y, x,
-                m->queue + 1, chunk, m->queue, 0, NZ_FEW);
+                m->queue + 1, chunk, nullptr, m->queue);
         }
         PSF_LAUNCHED();
         return PSF_OK;
     });
-    return rc ? rc
-              : rows_pair_stream<PS_BACK>(m, y, nullptr, x, nullptr, st, m->queue, NZ_FEW);
+    return rc ? rc : rows_pair_stream<PS_BACK>(m, y, nullptr, x, nullptr, st, m->queue);
 }
 
 static int rows_back(const psf_matrix *m, const float *y, float *x, cudaStream_t st) {
@@ -3671,7 +3685,7 @@ static int rows_back_listed(const psf_matrix *m, const float *y, float *x, cudaS
             PSF_TIMED("csr_back_wq_kernel", st);
             csr_back_wq_kernel<VT><<<grid, threads, 0, st>>>(
                 m->n_rows, m->row_ptr, m->col, (const VT *)m->val, m->row_scale, y, x,
-                m->queue + 1, chunk, m->tr_nz, (m->n_rows >> 2) + 1, INT64_MAX);
+                m->queue + 1, chunk, m->tr_nz);
         }
         PSF_LAUNCHED();
         return PSF_OK;

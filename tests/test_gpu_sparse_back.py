@@ -32,17 +32,22 @@ def _plans(P, fan, dtype):
 def _back(P, M, y):
     P.timing_enable(True)
     x = M.back(y)
-    ms = P.timing_read()
+    ms = {k: v[1] for k, v in P.timing_read().items()}
     P.timing_enable(False)
-    return x, set(ms)
+    return x, ms
+
+
+def _streamed(ms):
+    """Which of the two did the work: the other returns at once."""
+    return ms["csr_back_single_kernel"] > ms["csr_back_wq_kernel"]
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
 @pytest.mark.parametrize("tuned", [False, True])
-@pytest.mark.parametrize("fan", [20, 42])  # 1,080,924 and 2,240,940 rows
+@pytest.mark.parametrize("fan", [40, 60])  # 2,135,484 and 3,190,044 rows
 def test_back_by_density(P, fan, dtype, tuned):
-    M, R, _ = _plans(P, fan, dtype)
-    assert M.n_rows >= 1 << 20
+    M, R, rows = _plans(P, fan, dtype)
+    assert M.n_rows >= 1 << 21
     if tuned:
         M.autotune()
     n = M.n_rows
@@ -52,10 +57,17 @@ def test_back_by_density(P, fan, dtype, tuned):
     for share in (0.0, 1e-6, 1e-3, 0.1, 0.4, 0.5, 0.6, 0.9, 1.0):
         y = torch.where(keep < share, dense, 0.0)
         got, ran = _back(P, M, y)
-        assert "sample_nonzero_kernel" in ran or tuned
+        assert "sample_sparse_kernel" in ran or tuned
+        if "sample_sparse_kernel" in ran and share in (0.0, 1e-6, 1.0):
+            assert _streamed(ran) == (share == 1.0)
         want = R.back(y)
         # sums of the same positive products in another order: up to ~2e4 per voxel
         assert_close(got.cpu(), want.cpu(), 2e-5, 1e-6 * float(want.abs().max()) + 1e-30, str(share))
+    # values only where a row has entries: the empty rows say nothing about the work
+    y = (rows[0][1:] > rows[0][:-1]).float()
+    got, ran = _back(P, M, y)
+    assert "sample_sparse_kernel" not in ran or _streamed(ran)
+    assert_close(got.cpu(), R.back(y).cpu(), 2e-5, 1e-6 * float(got.max()), "rows with entries")
     one = torch.zeros(n, device="cuda")
     one[n // 2 + 77] = 2.0  # its neighbours' row starts are a whole pair's away
     assert_close(_back(P, M, one)[0].cpu(), R.back(one).cpu(), 2e-5, 1e-30, "one event")
@@ -63,19 +75,19 @@ def test_back_by_density(P, fan, dtype, tuned):
 
 
 def test_small_plans_stream(P):
-    M, R, _ = _plans(P, 5, "f32")
-    assert M.n_rows < 1 << 20
+    M, R, _ = _plans(P, 39, "f32")  # 2,082,756 rows
+    assert M.n_rows < 1 << 21
     y = torch.zeros(M.n_rows, device="cuda")
     y[::1001] = 1.0
     got, ran = _back(P, M, y)
-    assert "csr_back_single_kernel" in ran and "sample_nonzero_kernel" not in ran
+    assert "csr_back_single_kernel" in ran and "sample_sparse_kernel" not in ran
     assert_close(got.cpu(), R.back(y).cpu(), 2e-5, 1e-30, "small plan")
 
 
 def test_sparse_back_is_captured(P):
     """The choice is taken on the device: a captured back-projection follows the
     values of each replay."""
-    M, R, _ = _plans(P, 20, "f32")
+    M, R, _ = _plans(P, 40, "f32")
     y, out = torch.ones(M.n_rows, device="cuda"), torch.empty(M.n_cols, device="cuda")
     M.back(y, out=out)
     graph = torch.cuda.CUDAGraph()
