@@ -452,7 +452,8 @@ int psf_matrix_destroy(psf_matrix *m);
  * 4096 entries brought into shared memory by cp.async.bulk copies completing
  * on an mbarrier, one chunk ahead; each chunk owns the rows that start in it),
  * and, where psf_matrix_set_image allows it, the pair-streamed form,
- * on all-ones vectors, and keeps the fastest for psf_forward / psf_back of
+ * on an image of ones (the back-projections on its projection), and keeps the
+ * fastest for psf_forward / psf_back of
  * this plan (chunk_out / threads_out name the fastest of the others); the pair
  * back-projection of psf_back_sens takes the fastest of the back launch, the
  * bulk-staged kernel (not a choice of psf_back: it cannot skip rows with y = 0)
@@ -621,6 +622,9 @@ int psf_osem(const psf_matrix *m, const int64_t *rows, int64_t n_events, int32_t
  *   (synchronising with the GPU work they bracket) and returns kernel i of the
  *   accumulators: its name (valid until the next psf_timing_enable), number of
  *   launches and total milliseconds.  PSF_EINVAL past the last kernel.
+ * A kernel's instances have a name each, mostly kernel<instance>;
+ *   pair_stream_kernel's are csr_fwd_patch_kernel (psf_forward),
+ *   csr_back_single_kernel (psf_back) and csr_back_patch_kernel (psf_back_sens).
  * Timing adds two event records per launch; results are unaffected.
  */
 int psf_timing_enable(int32_t on);

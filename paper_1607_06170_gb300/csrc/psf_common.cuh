@@ -123,8 +123,8 @@ int otf_rows_back(const Scan &sc, const Img &im, const LorSet &ls, const int32_t
 // Grid for a grid-stride loop over n items: at most 8 CTAs per SM.
 int grid_for(int64_t n, int block);
 
-// In-place inclusive scan of an int64 array on `st` (three launches);
-// tile_sums needs scan_tile_count(n) slots.
+// In-place inclusive scan of an int64 array on `st` (one launch up to SCAN1_N
+// values, else three); tile_sums needs scan_tile_count(n) slots.
 int64_t scan_tile_count(int64_t n);
 int inclusive_scan(int64_t *x, int64_t n, int64_t *tile_sums, cudaStream_t st);
 

@@ -14,9 +14,10 @@
 // from one multiply-high, its cell from a byte table over the x/y index, its row
 // is the warp's running row.  One more warp prepares the next pair (row starts,
 // row values, cell list) meanwhile, and passes over pairs whose row values are
-// all 0.  An entry whose voxel is not in the table (cells past the ones held, or
-// rows of any other structure) goes to the image directly, so any rows give the
-// same result.  Bound by the warps' chains and the stream together: 3D ring,
+// all 0 (a large plan with few values goes row by row: sample_sparse_kernel).
+// An entry whose voxel is not in the table (cells past the ones held, or rows of
+// any other structure) goes to the image directly, so any rows give the same
+// result.  Bound by the warps' chains and the stream together: 3D ring,
 // 3.97e9 entries (32 GB of columns and values, 4.7 ms at the copy rate): forward
 // 9.14 -> 7.49 ms, back 13.4 -> 7.14 ms, pair 12.05 -> 10.6 ms (the pair had its
 // voxels in shared memory already, found through a run table and two divisions,

@@ -3723,7 +3723,8 @@ extern "C" int psf_matrix_autotune(psf_matrix *m, int32_t *chunk_out, int32_t *t
         // candidates per direction: the grid-stride kernels (chunk 0), the work
         // queue at every (rows per take, threads per CTA) pair and, forward with
         // FP32 rows, the streaming tiles (chunk -1); each timed with CUDA events
-        // on all-ones vectors (one warm-up, best of two), the fastest kept
+        // on an image of ones and its projection (one warm-up, best of two), the
+        // fastest kept
         static const int chunks[] = {-2, -1, 0, 1, 2, 4, 8, 16, 32, 64, 128};
         const bool bulk = bk_table(m, st) == PSF_OK;
         static const int threads[] = {128, 256, 512};

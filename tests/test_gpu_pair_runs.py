@@ -22,7 +22,8 @@ def ring():
     return P, s, ls, w["window"], W
 
 
-SIZES = [(256, 256, 5), (257, 31, 9), (19, 300, 8), (480, 480, 3), (1000, 7, 2)]  # (nx + ny < 1024: the set generator)
+# (nx + ny < 1024: the set generator)
+SIZES = [(256, 256, 5), (257, 31, 9), (19, 300, 8), (480, 480, 3), (1000, 7, 2)]
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
