@@ -939,8 +939,18 @@ __global__ void __launch_bounds__(PJ_T) mlem_ratio_kernel(
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (h.c[u] >= 0) acc = fmaf(h.v[u], x ? x[h.c[u]] : 1.0f, acc);
-        for (int64_t j = h.j0 + 128 + lane; j < h.j1; j += 32)
-            acc = fmaf(ld_val(val, j), x ? x[col[j]] : 1.0f, acc);
+        for (int64_t j = h.j0 + 128 + lane; j < h.j1; j += 128) {
+            int c[4];
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                c[u] = j + 32 * u < h.j1 ? col[j + 32 * u] : -1;
+                v[u] = j + 32 * u < h.j1 ? ld_val(val, j + 32 * u) : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c[u] >= 0) acc = fmaf(v[u], x ? x[c[u]] : 1.0f, acc);
+        }
         acc = warp_sum_f(acc);
         if (lane == 0) {
             const float d = scale ? acc * sc : acc;
@@ -4148,9 +4158,18 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
     unsigned *key = reinterpret_cast<unsigned *>(yhat);
     if (n == 0) PSF_TRY(cudaMallocAsync(&key, sizeof(unsigned), st));
     const int vgrid = grid_for(nv, PJ_T), rgrid = grid_for(n * 32, PJ_T);
-    // three launches an iteration for stored rows at the grid-stride launches
-    // (a tuned plan keeps its own kernels)
-    const bool fused = !m->factored && !m->otf && n > 0 && m->fwd_chunk == 0 && m->wq_chunk == 0;
+    // three launches an iteration for stored rows at the grid-stride launches (a
+    // tuned plan keeps its own kernels) while a warp has at most four rows: with
+    // more, the loads ahead of each row cost more than the launches they hide (rows
+    // with ratio 0 are loaded too, the entries stay in L1 in the image's place).
+    // us an iteration, against the separate kernels: 2,000 rows of 130 entries 6.8
+    // (18.7), 40,000 42 (54), 160,000 173 (166), with 90 % of the data 0 90 (75);
+    // 80,000 rows of 1,600 883 (846); 17 M rows of 90 11.0 ms (9.8).  A first
+    // iteration from ones needs no image and both products of every row: it takes
+    // them at any size (17 M rows: 8.9 ms against 10.3).
+    const bool rows_only =
+        !m->factored && !m->otf && n > 0 && m->fwd_chunk == 0 && m->wq_chunk == 0;
+    const bool fused = rows_only && n <= 4 * (int64_t)rgrid * (PJ_T / 32);
     // (a chain's first kernel is launched plainly: see launch_after)
     auto launch = [&](const char *name, bool first, auto kernel, int grid, auto... args) -> int {
         PSF_TIMED(name, st);
@@ -4162,7 +4181,7 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
         return PSF_OK;
     };
     auto to_ratio = [&](bool ones) -> int {
-        if (!fused) {
+        if (!(ones || fused)) {
             const int rc = psf_forward(m, x, ratio, stream);
             return rc ? rc : psf_em_ratio(y, ratio, ratio, n, stream);
         }
@@ -4198,7 +4217,7 @@ extern "C" int psf_mlem(const psf_matrix *m, const float *y, float *x, float *se
             // first iteration from an image of ones: its forward projection equals
             // that of ones on the voxels the scanner sees (the others' columns are
             // zero), so A^T 1 comes with the first back-projection
-            if (fused) {
+            if (rows_only) {
                 rc = to_ratio(true);
                 if (!rc) rc = back(true);
                 if (!rc) rc = sens_key(true);
