@@ -519,12 +519,13 @@ int psf_matrix_set_stencil_form(psf_matrix *m, int32_t form);
  * voxel is not among them, or past the shared-memory capacity, takes the global
  * access, so any rows give the same result up to FP32 summation order.  Used by
  * default once declared where a pair's cells mostly fit beside a table of a byte
- * per (x, y); psf_back_sens on wider images finds the cells by their y rows
- * instead.  psf_matrix_autotune times these forms against the others;
- * psf_matrix_set_launch switches psf_forward and psf_back to the launch it sets.
- * A tuned choice is kept over later psf_matrix_set_spread(_topn) and
- * psf_matrix_set_image calls and applies while the plan allows the form; otherwise
- * the row launches run.  Where psf_back works by pairs, a plan of 2^21 rows or more
+ * per (x, y) and, for psf_forward and psf_back, a pair's ring pairs times nx + ny
+ * come to 2^17 and 2^15 (or the set has only a few pairs an SM); psf_back_sens on
+ * wider images finds the cells by their y rows instead.  psf_matrix_autotune times
+ * these forms against the others; psf_matrix_set_launch switches psf_forward and
+ * psf_back to the launch it sets.  A tuned choice is kept over later
+ * psf_matrix_set_spread(_topn) and psf_matrix_set_image calls and applies while the
+ * plan allows the form; otherwise the row launches run.  Where psf_back works by pairs, a plan of 2^21 rows or more
  * goes row by row, past the rows with value 0, when about half of its entries or
  * less are in the others (a sample on the device decides, so the calls stay
  * capturable); otherwise a pair with any nonzero value is read whole.

@@ -2887,13 +2887,24 @@ static int rows_pair_stream(const psf_matrix *m, const float *in, const float *i
 
 // Is a direction (0 forward, 1 back) pair-streamed: where the plan as it is now
 // allows it (the spreads or the image may be others than those it was timed
-// with), as timed, else where it fits.
+// with), as timed; nothing timed, where it fits and a pair is worth a CTA.  A pair
+// costs about 2 us of its own (its table, its voxels' exchange) and saves some 10 ns
+// a row forward and 0.25 ns an entry back, a row having up to 0.7 (nx + ny) entries.
+// 32,604 pairs with many empty rows (6,396 full ones) over 160 x 160, time over the
+// row launch's by the rows a pair: forward 1 row 40 (17), 44 2.6 (1.7), 214 1.18
+// (0.98), 448 0.92 (0.84), 1,372 0.68; back 1 row 23 (9), 44 1.6 (0.95), 97 1.06
+// (0.63), 169 0.81 (0.46), 448 0.61 (0.47), 1,372 0.43.  A plan of up to four pairs an SM is
+// streamed whatever its rows: small scanners so go the way of the large ones, which
+// costs them some 10 to 20 us a call until they are tuned.
 static bool use_pair_stream(const psf_matrix *m, int dir) {
     if (m->stream_form[dir] == 1) return false;
     PairGrid g{};
     int sms = 0;
     bool fits = false;
-    return pair_grid(m, 1, &g, &sms, &fits) && (m->stream_form[dir] == 2 || fits);
+    if (!pair_grid(m, 1, &g, &sms, &fits)) return false;
+    const int64_t size = (int64_t)g.nrp * (g.nx + g.ny);
+    const bool pays = size >= (dir == 0 ? 1 << 17 : 1 << 15) || m->ls.ntp <= 4 * (int64_t)sms;
+    return m->stream_form[dir] == 2 || (fits && pays);
 }
 
 static int rows_fwd_with(const psf_matrix *m, const float *x, float *y, int chunk, int threads,

@@ -19,13 +19,13 @@ def P():
 
 def _plans(P, fan, dtype):
     w = I.workload("RING3D")
-    s = dict(w["scanner"], n_block_rings=1)
-    ls, win = dict(fan_half=fan, max_ring_diff=12), (1, 0)
-    im = I.image(60, 72, 13, 2.0, 2.0, 2.2)
+    s = dict(w["scanner"], n_block_rings=2)
+    ls, win = dict(fan_half=fan, max_ring_diff=15), (1, 0)
+    im = I.image(60, 72, 26, 2.0, 2.0, 2.2)
     T, eta = P.response_build(s, w["table"])
     W = P.bin_spread_classes(s, w["table"], T, eta, ls, P.lor_set_classes(s, ls), *win)
     rows = P.sysmat_rows_set_typed(s, im, ls, dtype)
-    make = lambda: P.Matrix(*rows[:3], 60 * 72 * 13, row_scale=rows[3]).set_spread(s, ls, *win, W)
+    make = lambda: P.Matrix(*rows[:3], 60 * 72 * 26, row_scale=rows[3]).set_spread(s, ls, *win, W)
     return make().set_image(im), make().set_launch(0), rows
 
 
@@ -44,7 +44,7 @@ def _streamed(ms):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
 @pytest.mark.parametrize("tuned", [False, True])
-@pytest.mark.parametrize("fan", [40, 60])  # 2,135,484 and 3,190,044 rows
+@pytest.mark.parametrize("fan", [12, 17])  # 2,207,400 and 3,090,360 rows
 def test_back_by_density(P, fan, dtype, tuned):
     M, R, rows = _plans(P, fan, dtype)
     assert M.n_rows >= 1 << 21
@@ -75,7 +75,7 @@ def test_back_by_density(P, fan, dtype, tuned):
 
 
 def test_small_plans_stream(P):
-    M, R, _ = _plans(P, 39, "f32")  # 2,082,756 rows
+    M, R, _ = _plans(P, 11, "f32")  # 2,030,808 rows
     assert M.n_rows < 1 << 21
     y = torch.zeros(M.n_rows, device="cuda")
     y[::1001] = 1.0
@@ -87,7 +87,7 @@ def test_small_plans_stream(P):
 def test_sparse_back_is_captured(P):
     """The choice is taken on the device: a captured back-projection follows the
     values of each replay."""
-    M, R, _ = _plans(P, 40, "f32")
+    M, R, _ = _plans(P, 12, "f32")
     y, out = torch.ones(M.n_rows, device="cuda"), torch.empty(M.n_cols, device="cuda")
     M.back(y, out=out)
     graph = torch.cuda.CUDAGraph()
